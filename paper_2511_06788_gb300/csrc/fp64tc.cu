@@ -19,8 +19,9 @@
 //   below that of FP64 FMA relative to the typical term.
 //
 //   Products.  sum_k X_ak X_bk = sum_{s,t} (sum_k d_s d'_t) 2^(8 (2 ND - 2 - s - t)); the
-//   pairs with s + t <= ND - 1 (28 or 36 MMAs per K step) are kept, summed per level
-//   l = s + t in one TMEM accumulator each (ND accumulators of 128 x 64).  The dropped
+//   pairs with s + t <= ND - 1 (28 or 36 per K step) are kept, summed per level l = s + t in
+//   one TMEM accumulator each (ND adjacent accumulators of 128 x 64).  The pairs of one A
+//   digit with up to four B digits are one MMA (11 or 12 MMAs per K step).  The dropped
 //   levels weigh at most about 2^-(B-1.6) of |X_a| |X_b| per term.
 //
 //   Exactness.  |d_s d'_t| <= 2^14, so over 256 K values a level-l sum is at most
@@ -38,10 +39,9 @@
 // grid points; the update contracts over the 2p columns of [U W] (already contiguous) with
 // one exponent per grid point.  The MMA kernel is warp specialised: one thread issues
 // TMA loads of 32-wide K slabs of all 2 ND digit planes (64-byte swizzle) into a
-// two-stage ring, two threads issue the digit-pair MMAs of each 16-wide K step (each for
-// its own levels: the tensor core takes an MMA about every 45 clocks, and a single issuing
-// thread loses hundreds of clocks at every barrier of the ring), and eight warps drain the
-// accumulators.  CTAs run in clusters of two on two SMs; the pair computes
+// two-stage ring, two threads issue the MMAs of each 16-wide K step (each for its own
+// levels: a single issuing thread loses hundreds of clocks at every barrier of the ring), and
+// eight warps drain the accumulators.  CTAs run in clusters of two on two SMs; the pair computes
 // two output tiles with the same 128 A rows and adjacent 64-row blocks of B, and each CTA
 // loads one 64-row half of the A planes into both CTAs' shared memory (TMA multicast), so
 // a stage moves 2/3 of its bytes from L2.  A slot of the ring is free when the MMAs of
@@ -83,7 +83,7 @@ template <int ND> constexpr int ring_stages() {
 static_assert(kKS == 16 || kKS == 32, "K slab of one or two MMA K steps");
 static_assert(ring_stages<8>() >= 2, "ring of at least two stages");
 template <int ND> constexpr int smem_bytes() { return ring_stages<ND>() * stage_bytes<ND>() + 1024; }
-constexpr int kIssuers = 2;                // warps 1 .. kIssuers issue the MMAs
+constexpr int kIssuers = 2;                // warps 1 and 2 issue the MMAs
 #ifndef FP64TC_DRAIN_WARPS
 #define FP64TC_DRAIN_WARPS 8
 #endif
@@ -92,7 +92,6 @@ constexpr int kDrainCols = 4 * kBN / kDrainWarps;  // output columns per drain t
 static_assert(kDrainCols % 4 == 0 && kDrainCols >= 4, "drain column groups of four");
 constexpr int kThreads = 32 * (1 + kIssuers + kDrainWarps);  // warp 0 TMA, then MMA, drain
 constexpr uint32_t kTmemCols = 512;        // ND x 64 used
-constexpr uint32_t kIdesc = tc::idesc_bf16(kBM, kBN);
 constexpr uint64_t kWaitNs = 2000000000ull;
 
 enum { MODE_GRAM = 0, MODE_UPDATE_DELTA = 1, MODE_UPDATE = 2 };
@@ -193,79 +192,29 @@ __device__ __forceinline__ void mma_commit_mc(uint64_t *bar) {
       : "memory");
 }
 
-// D[tmem] (+)= A B^T (BF16, K = 16) with the A operand kept in the tensor core's collector
-// buffer across a run of MMAs that share it: C = 1 loads A and keeps it (fill), 2 reuses it
-// (use), 3 reuses it for the last time (lastuse), 0 a lone MMA (A read and discarded).
-template <int C>
-__device__ __forceinline__ void mma_bf16_ca(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                            uint32_t idesc, uint32_t accumulate) {
-  if constexpr (C == 1) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}\n"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-  } else if constexpr (C == 2) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n\t}\n"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-  } else if constexpr (C == 3) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n\t}\n"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-  } else {
-    tc::mma_bf16(d_tmem, a_desc, b_desc, idesc, accumulate);
-  }
-}
+// Two threads issue the digit MMAs, each for its own levels (accumulators): the pairs of one
+// level all come from one thread, in order, and while one thread waits at a barrier the other
+// keeps the tensor core busy.  Thread 0 takes levels 0 .. kHiLevels - 1 (the exact ones, summed
+// in `hi`), thread 1 the rest (`lo`).
+constexpr int kHiLevels = 4;
 
-// kIssuers threads issue the digit-pair MMAs, each for the levels in its mask: the pairs
-// of one level (one accumulator) all come from one thread, in order, and while one thread
-// waits at a barrier the others keep the tensor core busy.  The masks balance the pair
-// counts l + 1 of the levels between the threads.
-template <int ND> constexpr unsigned issuer_mask(int which) {
-  constexpr unsigned all = (1u << ND) - 1u;
-  if (kIssuers == 1) return all;
-  if (kIssuers == 2) {
-    constexpr unsigned a = ND == 7 ? 0x47u : 0x8Fu;  // {0,1,2,6} | {0,1,2,3,7}
-    return which == 0 ? a : all & ~a;
-  }
-  // three: {0,1,6} {2,5} {3,4} (10 / 9 / 9 pairs) | {3,7} {4,6} {0,1,2,5} (12 each)
-  constexpr unsigned m7[3] = {0x43u, 0x24u, 0x18u}, m8[3] = {0x88u, 0x50u, 0x27u};
-  return ND == 7 ? m7[which] : m8[which];
-}
-// First and last t of A digit s's MMAs (t < ND - s) whose level s + t is in `mask`.
-constexpr int run_first(int nd, unsigned mask, int s) {
-  for (int t = 0; t < nd - s; ++t)
-    if ((mask >> (s + t)) & 1u) return t;
-  return -1;
-}
-constexpr int run_last(int nd, unsigned mask, int s) {
-  for (int t = nd - s - 1; t >= 0; --t)
-    if ((mask >> (s + t)) & 1u) return t;
-  return -1;
-}
-
-// The MMAs of A digit S against B digits T.. (S + T in MASK); every level starts afresh at
-// its first MMA, (0, l), when `first` is set.  With one issuer (REUSE) A is held in the
-// collector buffer from the first MMA of the run to the last; two issuers interleave their
-// MMAs on the one tensor core, so each MMA then reads its own A.
-template <int ND, unsigned MASK, int S, int T>
-__device__ __forceinline__ void mma_digit_run(uint32_t tmem, uint64_t ad, uint64_t bd0,
-                                              uint32_t first) {
-  if constexpr (T < ND - S) {
-    if constexpr ((MASK >> (S + T)) & 1u) {
-      constexpr int f = run_first(ND, MASK, S), l = run_last(ND, MASK, S);
-      constexpr int C = kIssuers > 1 || f == l ? 0 : (T == f ? 1 : (T == l ? 3 : 2));
-      mma_bf16_ca<C>(tmem + (uint32_t)((S + T) * kBN), ad,
-                     bd0 + (uint64_t)((T * kBPlane) >> 4), kIdesc, S == 0 && first ? 0u : 1u);
-    }
-    mma_digit_run<ND, MASK, S, T + 1>(tmem, ad, bd0, first);
-  }
-}
-template <int ND, unsigned MASK, int S>
+// The MMAs of levels [L0, L1) for one 16-wide K step.  B digits t, t + 1, .. are adjacent
+// 64-row planes of the stage and levels l, l + 1, .. adjacent 64-column accumulators, so the
+// products of A digit s with B digits t0 .. t1 - 1 (levels s + t0 ..) are one MMA of
+// N = 64 (t1 - t0): the A tile is read from shared memory once per MMA instead of once per
+// digit pair (an N = 64 MMA reads 4 KB of A for 2 KB of B and runs at the shared-memory rate).
+// Every level starts afresh at its first MMA, (0, l), when `first` is set; the order of the
+// products inside a level is by s.
+template <int ND, int L0, int L1, int S>
 __device__ __forceinline__ void mma_kstep(uint32_t tmem, uint64_t a0, uint64_t bd0,
                                           uint32_t first) {
-  if constexpr (S < ND) {
-    mma_digit_run<ND, MASK, S, 0>(tmem, a0 + (uint64_t)((S * kAPlane) >> 4), bd0, first);
-    mma_kstep<ND, MASK, S + 1>(tmem, a0, bd0, first);
+  if constexpr (S < L1) {
+    constexpr int t0 = L0 > S ? L0 - S : 0, nt = L1 - S - t0;
+    static_assert(nt >= 1 && nt * kBN <= 256, "one MMA takes at most four B digits");
+    tc::mma_bf16(tmem + (uint32_t)((S + t0) * kBN), a0 + (uint64_t)((S * kAPlane) >> 4),
+                 bd0 + (uint64_t)((t0 * kBPlane) >> 4), tc::idesc_bf16(kBM, nt * kBN),
+                 S == 0 && first ? 0u : 1u);
+    mma_kstep<ND, L0, L1, S + 1>(tmem, a0, bd0, first);
   }
 }
 
@@ -306,7 +255,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int kStageBytes = stage_bytes<ND>();
   constexpr int kStages = ring_stages<ND>();
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t full[kStages], empty[kStages], accfull, accempty, fin;
+  // accumulators of issuer i: complete (accfull[i]), read out (accempty[i])
+  __shared__ uint64_t full[kStages], empty[kStages], accfull[kIssuers], accempty[kIssuers], fin;
   __shared__ uint32_t tmem_sh;
   __shared__ int abort_sh;
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -321,8 +271,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(&full[s], 1);
       tc::mbar_init(&empty[s], 2 * kIssuers);  // both issuers of both CTAs of the pair
     }
-    tc::mbar_init(&accfull, kIssuers);
-    tc::mbar_init(&accempty, kDrainWarps);
+    for (int i = 0; i < kIssuers; ++i) {
+      tc::mbar_init(&accfull[i], 1);
+      tc::mbar_init(&accempty[i], kDrainWarps);
+    }
     tc::mbar_init(&fin, kIssuers);
     tc::fence_mbar_init();
     abort_sh = 0;
@@ -334,9 +286,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = tmem_sh;
   volatile int *abort = &abort_sh;
 
-  // ---- MMA issuers: the digit pairs of the levels in MASK ---------------------------------
-  auto issue = [&](auto maskc) {
-    constexpr unsigned MASK = decltype(maskc)::value;
+  // ---- MMA issuers: issuer 0 levels [0, kHiLevels), issuer 1 the rest -----------------------
+  auto issue = [&](auto which) {
+    constexpr int I = decltype(which)::value;
+    constexpr int L0 = I == 0 ? 0 : kHiLevels, L1 = I == 0 ? kHiLevels : ND;
     long long it = 0, chunk = 0;
     bool ok = true, issued = false;
     for (long long pr = cid; pr < J.npairs && ok; pr += ncl) {
@@ -349,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool cstart = (st % kChunkStages) == 0;
         if (cstart && chunk > 0) {
           // the accumulators start afresh once the drain warps have read them
-          if (!tc::wait_or_abort(&accempty, (uint32_t)((chunk - 1) & 1), abort, kWaitNs)) {
+          if (!tc::wait_or_abort(&accempty[I], (uint32_t)((chunk - 1) & 1), abort, kWaitNs)) {
             ok = false;
             break;
           }
@@ -366,13 +319,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t d0 = desc_sw(tc::smem_u32(smem + slot * kStageBytes));
 #pragma unroll
         for (int ks = 0; ks < kKS / 16; ++ks)
-          mma_kstep<ND, MASK, 0>(tmem, d0 + (uint64_t)((ks * 32) >> 4),
-                                 d0 + (uint64_t)((kDigits * kAPlane + ks * 32) >> 4),
-                                 (cstart && ks == 0) ? 1u : 0u);
+          mma_kstep<ND, L0, L1, 0>(tmem, d0 + (uint64_t)((ks * 32) >> 4),
+                                   d0 + (uint64_t)((kDigits * kAPlane + ks * 32) >> 4),
+                                   (cstart && ks == 0) ? 1u : 0u);
         issued = true;
         mma_commit_mc(&empty[slot]);  // the slot is free in both CTAs once all have read it
         if ((st % kChunkStages) == kChunkStages - 1 || st == nst - 1) {
-          tc::mma_commit(&accfull);
+          tc::mma_commit(&accfull[I]);
           ++chunk;
         }
       }
@@ -425,11 +378,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp <= kIssuers) {
     if (lane == 0) {
       if (warp == 1)
-        issue(std::integral_constant<unsigned, issuer_mask<ND>(0)>{});
-      else if (warp == 2)
-        issue(std::integral_constant<unsigned, issuer_mask<ND>(1)>{});
-      else if constexpr (kIssuers > 2)
-        issue(std::integral_constant<unsigned, issuer_mask<ND>(2)>{});
+        issue(std::integral_constant<int, 0>{});
+      else
+        issue(std::integral_constant<int, 1>{});
     }
   } else {
     // ---- drain warps ---------------------------------------------------------------------
@@ -437,45 +388,62 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int half = (warp - kIssuers - 1) >> 2;    // output columns kDrainCols half + ...
     const int row = q * 32 + lane;                  // tile row
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * kDrainCols);
-    long long chunk = 0;
+    uint32_t par = 0;  // parity of the accumulators' current chunk
     bool ok = true;
     for (long long pr = cid; pr < J.npairs && ok; pr += ncl) {
       int ra, rb;
       long long k0, klen, item;
       bool valid;
       decode_pair(J, pr, rank, &ra, &rb, &k0, &klen, &valid, &item);
-      const long long nst = (klen + kKS - 1) / kKS;
-      const long long nch = (nst + kChunkStages - 1) / kChunkStages;
+      const int nch = (int)((klen + 255) / 256);
       long long hi[kDrainCols], lo[kDrainCols];
 #pragma unroll
       for (int j = 0; j < kDrainCols; ++j) hi[j] = lo[j] = 0;
-      for (long long c = 0; c < nch; ++c, ++chunk) {
-        if (!warp_wait(&accfull, (uint32_t)(chunk & 1), abort)) {
+      for (int c = 0; c < nch; ++c, par ^= 1) {
+        // issuer 0's levels first: its MMAs of the next chunk start while the others are read
+        if (!warp_wait(&accfull[0], par, abort)) {
           ok = false;
           break;
         }
         tc::tc_fence_after();
 #pragma unroll
         for (int g = 0; g < kDrainCols / 4; ++g) {
-          uint32_t v[kLevels][4];
+          uint32_t v[kHiLevels][4];
 #pragma unroll
-          for (int l = 0; l < kLevels; ++l) tmem_ld4(tbase + (uint32_t)(l * kBN + g * 4), v[l]);
+          for (int l = 0; l < kHiLevels; ++l) tmem_ld4(tbase + (uint32_t)(l * kBN + g * 4), v[l]);
           tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            long long L[kLevels];
+          for (int e = 0; e < 4; ++e)
 #pragma unroll
-            for (int l = 0; l < kLevels; ++l) L[l] = (long long)__float2int_rz(__uint_as_float(v[l][e]));
-            hi[g * 4 + e] += (L[0] << 24) + (L[1] << 16) + (L[2] << 8) + L[3];
-            long long lv = 0;
-#pragma unroll
-            for (int l = 4; l < kLevels; ++l) lv += L[l] << (8 * (kLevels - 1 - l));
-            lo[g * 4 + e] += lv;
-          }
+            for (int l = 0; l < kHiLevels; ++l)
+              hi[g * 4 + e] += (long long)__float2int_rz(__uint_as_float(v[l][e])) *
+                               (long long)(1 << (8 * (kHiLevels - 1 - l)));
         }
         tc::tc_fence_before();
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&accempty);
+        if (lane == 0) tc::mbar_arrive(&accempty[0]);
+        if (!warp_wait(&accfull[1], par, abort)) {
+          ok = false;
+          break;
+        }
+        tc::tc_fence_after();
+#pragma unroll
+        for (int g = 0; g < kDrainCols / 4; ++g) {
+          uint32_t v[kLevels - kHiLevels][4];
+#pragma unroll
+          for (int l = kHiLevels; l < kLevels; ++l)
+            tmem_ld4(tbase + (uint32_t)(l * kBN + g * 4), v[l - kHiLevels]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int l = kHiLevels; l < kLevels; ++l)
+              lo[g * 4 + e] += (long long)__float2int_rz(__uint_as_float(v[l - kHiLevels][e])) *
+                               (long long)(1 << (8 * (kLevels - 1 - l)));
+        }
+        tc::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&accempty[1]);
       }
       if (!ok) break;
       if (!valid) continue;  // a stand-in member: zeros in, nothing out
@@ -505,8 +473,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (col < J.ld) {
               double2 o;
               o.x = ldexp(fma((double)hi[j], kHiW, (double)lo[j]), ea + J.eb[col] + kShift);
-              o.y = ldexp(fma((double)hi[j + 1], kHiW, (double)lo[j + 1]),
-                          ea + J.eb[col + 1] + kShift);
+              o.y = ldexp(fma((double)hi[j + 1], kHiW, (double)lo[j + 1]), ea + J.eb[col + 1] + kShift);
               if (J.mode == MODE_UPDATE_DELTA) {
                 const double2 b = *reinterpret_cast<const double2 *>(J.base + r * J.ld + col);
                 o.x += b.x;
