@@ -240,6 +240,41 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// (hi 2^W + lo) 2^e in FP64, rounded once to nearest even: the 128-bit sum is normalised and
+// packed with integer instructions.  The FP64 pipe runs two instructions per clock and SM, so
+// two int64 conversions, an fma and an ldexp per output cost more than the 36 MMAs of a
+// short-K output; they remain for results outside the normal range.
+template <int W>
+__device__ __forceinline__ double pack_int128(long long hi, long long lo, int e) {
+  const unsigned long long l0 = (unsigned long long)hi << W;
+  unsigned long long tl = l0 + (unsigned long long)lo;
+  long long th = (hi >> (64 - W)) + (lo >> 63) + (tl < l0 ? 1 : 0);
+  const bool neg = th < 0;
+  if (neg) {  // |hi 2^W + lo| < 2^127
+    tl = 0ull - tl;
+    th = ~th + (tl == 0 ? 1 : 0);
+  }
+  // normalise: m holds the leading 64 bits of the magnitude, rest (non-zero or not) the others
+  const int lz = th ? __clzll(th) : 64 + __clzll((long long)tl);
+  unsigned long long m, rest;
+  if (th) {
+    m = ((unsigned long long)th << lz) | ((tl >> 1) >> (63 - lz));
+    rest = tl << lz;
+  } else {
+    m = tl << (lz & 63);
+    rest = 0;
+  }
+  if (lz >= 128) return 0.0;
+  const int be = 1023 + 127 - lz + e;  // biased exponent before rounding
+  if (be < 1 || be > 2045) return ldexp(fma((double)hi, (double)(1ll << W), (double)lo), e);
+  unsigned long long q = m >> 11;
+  const unsigned rem = (unsigned)m & 0x7FFu;
+  if (rem > 0x400u || (rem == 0x400u && (rest != 0 || (q & 1)))) ++q;
+  // q carries the leading one at bit 52 (a carry out of it raises the exponent)
+  q += (unsigned long long)(be - 1) << 52;
+  return __longlong_as_double((long long)(q | ((unsigned long long)neg << 63)));
+}
+
 // Lane 0 waits (bounded, or until another role aborted); the result goes to the warp.
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
   int ok = 0;
@@ -448,7 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       if (!valid) continue;  // a stand-in member: zeros in, nothing out
       // epilogue: (2^(8 (ND - 4)) hi + lo) 2^(e_a + e_b - 2 (8 ND - 1) + 8 (ND - 1))
-      constexpr double kHiW = (double)(1ll << (8 * (ND - 4)));
+      constexpr int kW = 8 * (ND - 4);
       constexpr int kShift = -2 * (8 * ND - 1) + 8 * (ND - 1);
       if (J.mode == MODE_GRAM) {
         // rows and columns beyond nc hold zero digits (the loads past the planes read 0)
@@ -459,8 +494,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int cb = rb + half * kDrainCols + j;
           const int eb0 = cb < J.nc ? J.eb[cb] : 0, eb1 = cb + 1 < J.nc ? J.eb[cb + 1] : 0;
           double2 o;
-          o.x = ldexp(fma((double)hi[j], kHiW, (double)lo[j]), ea + eb0 + kShift);
-          o.y = ldexp(fma((double)hi[j + 1], kHiW, (double)lo[j + 1]), ea + eb1 + kShift);
+          o.x = pack_int128<kW>(hi[j], lo[j], ea + eb0 + kShift);
+          o.y = pack_int128<kW>(hi[j + 1], lo[j + 1], ea + eb1 + kShift);
           *reinterpret_cast<double2 *>(dst + j) = o;
         }
       } else {
@@ -472,8 +507,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int col = rb + half * kDrainCols + j;
             if (col < J.ld) {
               double2 o;
-              o.x = ldexp(fma((double)hi[j], kHiW, (double)lo[j]), ea + J.eb[col] + kShift);
-              o.y = ldexp(fma((double)hi[j + 1], kHiW, (double)lo[j + 1]), ea + J.eb[col + 1] + kShift);
+              o.x = pack_int128<kW>(hi[j], lo[j], ea + J.eb[col] + kShift);
+              o.y = pack_int128<kW>(hi[j + 1], lo[j + 1], ea + J.eb[col + 1] + kShift);
               if (J.mode == MODE_UPDATE_DELTA) {
                 const double2 b = *reinterpret_cast<const double2 *>(J.base + r * J.ld + col);
                 o.x += b.x;
@@ -505,11 +540,9 @@ __device__ __forceinline__ int exponent_of(double mx) {
   return e;
 }
 
-// The ND balanced base-256 digits of X = round(a 2^(8 ND - 1 - e)) (|a| < 2^e), as BF16 bit
-// patterns; integer arithmetic on the bits of a.  Subnormal a (below 2^-1022) count as 0.
-template <int ND>
-__device__ __forceinline__ void digits_of(double a, int e, uint16_t (&d)[ND]) {
-  constexpr int kDigits = ND;
+// X = round(a 2^(8 ND - 1 - e)) for |a| < 2^e, by integer arithmetic on the bits of a.
+// Subnormal a (below 2^-1022) count as 0.
+template <int ND> __device__ __forceinline__ long long scaled_int(double a, int e) {
   const long long bits = __double_as_longlong(a);
   const int be = (int)((bits >> 52) & 0x7FF);
   long long X = 0;
@@ -525,14 +558,38 @@ __device__ __forceinline__ void digits_of(double a, int e, uint16_t (&d)[ND]) {
     }
     if (bits < 0) X = -X;
   }
+  return X;
+}
+
+// The ND balanced base-256 digits of two values (a first, in the low half) as packed pairs of
+// BF16.  Adding 128 to every lower digit at once turns the balanced digits into plain bytes
+// (byte - 128 is the digit, in [-128, 127]; the carries ripple in one 64-bit addition), and a
+// signed byte s becomes BF16 exactly as (128 + (s & 127)) - (128 + (s & 128)): about 2 + 2
+// instructions a digit and no integer-to-float conversions.  The top digit is in [-128, 128].
+template <int ND>
+__device__ __forceinline__ void digit_pairs(double a, double b, int e, uint32_t (&d)[ND]) {
+  constexpr int kTop = 8 * (ND - 1);
+  constexpr unsigned long long kMask = (1ull << kTop) - 1;
+  constexpr unsigned long long kBias = 0x8080808080808080ull & kMask;
+  const long long Xa = scaled_int<ND>(a, e), Xb = scaled_int<ND>(b, e);
+  const unsigned long long ya = ((unsigned long long)Xa & kMask) + kBias;
+  const unsigned long long yb = ((unsigned long long)Xb & kMask) + kBias;
+  const int ta = (int)(Xa >> kTop) + (int)(ya >> kTop);
+  const int tb = (int)(Xb >> kTop) + (int)(yb >> kTop);
+  d[0] = __byte_perm(__float_as_uint((float)ta), __float_as_uint((float)tb), 0x7632);
+  const uint32_t al = (uint32_t)ya ^ 0x80808080u, ah = (uint32_t)(ya >> 32) ^ 0x80808080u;
+  const uint32_t bl = (uint32_t)yb ^ 0x80808080u, bh = (uint32_t)(yb >> 32) ^ 0x80808080u;
 #pragma unroll
-  for (int s = kDigits - 1; s >= 1; --s) {
-    const int lo8 = (int)(X & 0xFF);
-    const int dd = lo8 - ((lo8 & 0x80) << 1);
-    d[s] = (uint16_t)(__float_as_uint((float)dd) >> 16);
-    X = (X - dd) >> 8;
+  for (int s = 1; s < ND; ++s) {
+    const int k = ND - 1 - s;  // byte index of digit s
+    // both values' bytes in the low bytes of the two halves (the high bytes are masked off)
+    const uint32_t w = __byte_perm(k < 4 ? al : ah, k < 4 ? bl : bh,
+                                   (uint32_t)((k & 3) | ((4 + (k & 3)) << 8)));
+    const uint32_t lo7 = (w & 0x007F007Fu) | 0x43004300u, hi1 = (w & 0x00800080u) | 0x43004300u;
+    const __nv_bfloat162 v = __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&lo7),
+                                     *reinterpret_cast<const __nv_bfloat162 *>(&hi1));
+    d[s] = *reinterpret_cast<const uint32_t *>(&v);
   }
-  d[0] = (uint16_t)(__float_as_uint((float)(int)X) >> 16);
 }
 
 // Column exponents of Y = [U W] (nc = ld or 2 ld columns) over grid points [x0, x0 + m),
@@ -567,41 +624,52 @@ __global__ void k_decode_exp(const int *__restrict__ enc, int *__restrict__ e, i
 
 // Digit planes P[s][c][x] (x contiguous, pitch xp) of the columns of Y over grid points
 // [x0, x0 + m): 64 x 64 tiles transposed through shared memory; x in [m, xp) gets zeros.
+// Bound by HBM (8 bytes read, 2 ND written per value) once the digits cost few instructions.
+// A thread writes 16 bytes (8 points) of a column, 8 threads a 128-byte line of it; the tile's
+// columns are rotated by two per 8 points, so the 16 threads of a half warp (8 point groups x
+// 2 columns) read 16 different 8-byte banks.
 template <int ND>
 __global__ void __launch_bounds__(256)
     k_split_cols(const double *__restrict__ U, const double *__restrict__ W, int ld, int nc,
                  long long x0, long long m, long long xp, const int *__restrict__ ecol,
                  uint16_t *__restrict__ P) {
-  __shared__ double tile[64][65];
+  __shared__ __align__(16) double tile[64 * 64];
   const long long xb = (long long)blockIdx.x * 64;
   const int cb = blockIdx.y * 64;
-  for (int i = threadIdx.x; i < 64 * 64; i += 256) {
-    const int r = i >> 6, cc = i & 63, c = cb + cc;
-    const long long x = xb + r;
-    double v = 0.0;
-    if (x < m && c < nc) v = c < ld ? U[(x0 + x) * ld + c] : W[(x0 + x) * ld + (c - ld)];
-    tile[r][cc] = v;
+  auto at = [](int r, int c) { return r * 64 + ((c + 2 * (r >> 3)) & 63); };
+  {
+    const int cc = (threadIdx.x & 31) * 2, c = cb + cc, r0 = threadIdx.x >> 5;
+    const double *src = c < ld ? U + c : W + (c - ld);
+    double2 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const long long x = xb + r0 + 8 * i;
+      v[i] = make_double2(0.0, 0.0);
+      if (x < m && c < nc) v[i] = __ldg(reinterpret_cast<const double2 *>(src + (x0 + x) * ld));
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      *reinterpret_cast<double2 *>(tile + at(r0 + 8 * i, cc)) = v[i];
   }
   __syncthreads();
-  const int cc = threadIdx.x >> 2, rq = (threadIdx.x & 3) * 16, c = cb + cc;
-  if (c >= nc) return;
-  constexpr int kDigits = ND;
-  const int e = ecol[c];
-  uint32_t w[kDigits][8];
 #pragma unroll
-  for (int r = 0; r < 16; r += 2) {
-    uint16_t d0[kDigits], d1[kDigits];
-    digits_of<ND>(tile[rq + r][cc], e, d0);
-    digits_of<ND>(tile[rq + r + 1][cc], e, d1);
+  for (int h = 0; h < 2; ++h) {
+    const int cc = (threadIdx.x >> 3) + 32 * h, rq = (threadIdx.x & 7) * 8, c = cb + cc;
+    if (c >= nc) return;
+    const int e = ecol[c];
+    uint32_t w[ND][4];
 #pragma unroll
-    for (int s = 0; s < kDigits; ++s) w[s][r >> 1] = (uint32_t)d0[s] | ((uint32_t)d1[s] << 16);
-  }
-  const long long off = (long long)c * xp + xb + rq;
+    for (int r = 0; r < 8; r += 2) {
+      uint32_t d[ND];
+      digit_pairs<ND>(tile[at(rq + r, cc)], tile[at(rq + r + 1, cc)], e, d);
 #pragma unroll
-  for (int s = 0; s < kDigits; ++s) {
-    uint4 *dst = reinterpret_cast<uint4 *>(P + (long long)s * nc * xp + off);
-    dst[0] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-    dst[1] = make_uint4(w[s][4], w[s][5], w[s][6], w[s][7]);
+      for (int s = 0; s < ND; ++s) w[s][r >> 1] = d[s];
+    }
+    const long long off = (long long)c * xp + xb + rq;
+#pragma unroll
+    for (int s = 0; s < ND; ++s)
+      *reinterpret_cast<uint4 *>(P + (long long)s * nc * xp + off) =
+          make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
   }
 }
 
@@ -632,11 +700,10 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const double2 v = *reinterpret_cast<const double2 *>(src + 2 * i);
-      uint16_t d0[kDigits], d1[kDigits];
-      digits_of<ND>(v.x, e, d0);
-      digits_of<ND>(v.y, e, d1);
+      uint32_t d[kDigits];
+      digit_pairs<ND>(v.x, v.y, e, d);
 #pragma unroll
-      for (int s = 0; s < kDigits; ++s) w[s][i] = (uint32_t)d0[s] | ((uint32_t)d1[s] << 16);
+      for (int s = 0; s < kDigits; ++s) w[s][i] = d[s];
     }
 #pragma unroll
     for (int s = 0; s < kDigits; ++s)
@@ -670,11 +737,10 @@ __global__ void __launch_bounds__(256)
     uint32_t w[kDigits][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      uint16_t d0[kDigits], d1[kDigits];
-      digits_of<ND>(val(k + 2 * i), e, d0);
-      digits_of<ND>(val(k + 2 * i + 1), e, d1);
+      uint32_t d[kDigits];
+      digit_pairs<ND>(val(k + 2 * i), val(k + 2 * i + 1), e, d);
 #pragma unroll
-      for (int s = 0; s < kDigits; ++s) w[s][i] = (uint32_t)d0[s] | ((uint32_t)d1[s] << 16);
+      for (int s = 0; s < kDigits; ++s) w[s][i] = d[s];
     }
 #pragma unroll
     for (int s = 0; s < kDigits; ++s)
