@@ -1,0 +1,608 @@
+// Step 1 of §4.1 for blocks that stay in L2: the whole block CG in one cooperative launch.
+//
+// What bounds a small solve is not memory but the sequence itself: four or five launches of
+// 3 to 10 us an iteration and a host synchronisation every other one, for passes that take a
+// microsecond or two.  Here one grid of at most one CTA per SM runs the start and every
+// iteration: each CTA owns a contiguous range of grid points (its stencil neighbours are
+// mostly its own, so they come from L1), the dot products meet in a grid-wide barrier, and
+// every CTA sums the partials of all CTAs itself, in the same order, so alpha, beta and the
+// active columns need no second pass and no host.  The arithmetic per element is that of the
+// row kernels (stencil_cg.cu): FP32 recomputes P = R + beta P at the stencil points and takes
+// two barriers an iteration; FP64 stores Q and P and takes three (recomputing would cost six
+// more FP64 operations per element, and GB300 runs two a clock and SM).
+//
+// What is left of an iteration: tiny solves 5.4 us of shuffles, barriers and latency (32 x 32 x 8,
+// one cluster; 28 us by kernels), FP64 the FP64 pipe (199 x 199 x 16: 25 us, of which 11 for its
+// 10 operations an element; 55 us by kernels), FP32 the L2 latency of its stencil loads.
+//
+// Every wait of the barrier is bounded; a CTA that gives up sets the error word and returns.
+#include <string.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "common.cuh"
+#include "kernels.cuh"
+#include "tc.cuh"
+
+namespace opevo {
+
+namespace {
+
+constexpr int kCoopThreads = 512;
+// Largest block of a cooperative solve.  FP32: the four blocks of an iteration have to stay in
+// the 126 MB L2, and on 3-D grids the TMA direction kernel takes over: 56^3 x 40 (28 MB) 1.80 ms
+// here and 2.90 ms by kernels, 56^3 x 64 (45 MB) 3.43 and 3.54, 64^3 x 84 (92 MB) 8.9 and 7.7.
+// FP64: bound by the FP64 pipe either way: 64^3 x 64 (134 MB, the largest tried) 32.9 and 38.1.
+template <typename T> constexpr long long kCoopBytes = (sizeof(T) == 4 ? 48ll : 140ll) << 20;
+// polls of the barrier (several hundred clocks each) before a CTA gives up: some seconds
+constexpr int kBarrierPolls = 1 << 23;
+// ctl words (256 bytes): 2 iterations, 3 error, 32 the barrier's arrivals
+constexpr int kCtlBar = 32;
+
+// Grid-wide barrier: `target` is the number of arrivals that completes it.  False when the
+// wait gave up (the error word is set and every CTA gives up in turn).
+__device__ __forceinline__ bool grid_barrier(int *ctl, unsigned target, int *ok_sh) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned *cnt = reinterpret_cast<unsigned *>(ctl + kCtlBar);
+    int ok = 1;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+    // (no clock is read here: %globaltimer alone costs more than a poll)
+    int left = kBarrierPolls;
+    for (;;) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+      if (v >= target) break;
+      if (--left == 0) {
+        atomicExch(ctl + 3, 1);
+        ok = 0;
+        break;
+      }
+    }
+    *ok_sh = ok;
+  }
+  __syncthreads();
+  return *ok_sh != 0;
+}
+
+// Barrier of the CTAs of one cluster (in hardware: every CTA of a cluster is resident).
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Running sum across threads and CTAs.  FP64 blocks: a double.  FP32 blocks: an unevaluated pair
+// of floats (error-free two-sum, 48 bits): the terms are FP32 sums, and a warp's FP64 addition
+// takes 64 clocks of its scheduler on GB300, which made the reductions half of an iteration.
+template <typename T> struct Sum;
+// Threads that share the sums of the columns: all of them for FP32 pairs, one warp a scheduler
+// for FP64 (its additions queue on the one FP64 pipe, and idle lanes cost as much as busy ones).
+template <typename T> constexpr int kSumThreads = sizeof(T) == 4 ? kCoopThreads : 128;
+template <> struct Sum<double> {
+  double h = 0.0;
+  __device__ __forceinline__ void add(double x) { h += x; }
+  __device__ __forceinline__ void add(const Sum &o) { h += o.h; }
+  __device__ __forceinline__ double value() const { return h; }
+  __device__ __forceinline__ Sum down(int o) const {
+    Sum s;
+    s.h = __shfl_down_sync(0xffffffffu, h, o);
+    return s;
+  }
+  __device__ __forceinline__ Sum from(int lane, int width) const {
+    Sum s;
+    s.h = __shfl_sync(0xffffffffu, h, lane, width);
+    return s;
+  }
+  __device__ __forceinline__ static Sum load(const Sum *p) {
+    Sum s;
+    s.h = __ldcg(&p->h);
+    return s;
+  }
+  __device__ __forceinline__ static double ratio(const Sum &a, const Sum &b) { return a.h / b.h; }
+  __device__ __forceinline__ bool positive() const { return h > 0.0; }
+};
+template <> struct __align__(8) Sum<float> {
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    h = s;
+  }
+  __device__ __forceinline__ void add(const Sum &o) {
+    add(o.h);
+    l = __fadd_rn(l, o.l);
+  }
+  // (an overflowed sum has no low part)
+  __device__ __forceinline__ double value() const { return l == l ? (double)h + (double)l : (double)h; }
+  __device__ __forceinline__ Sum down(int o) const {
+    Sum s;
+    s.h = __shfl_down_sync(0xffffffffu, h, o);
+    s.l = __shfl_down_sync(0xffffffffu, l, o);
+    return s;
+  }
+  __device__ __forceinline__ Sum from(int lane, int width) const {
+    Sum s;
+    s.h = __shfl_sync(0xffffffffu, h, lane, width);
+    s.l = __shfl_sync(0xffffffffu, l, lane, width);
+    return s;
+  }
+  __device__ __forceinline__ static Sum load(const Sum *p) {
+    const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+    Sum s;
+    s.h = v.x;
+    s.l = v.y;
+    return s;
+  }
+  // a / b to about 46 bits, rounded to FP32 (what the FP64 quotient rounds to)
+  __device__ __forceinline__ static float ratio(const Sum &a, const Sum &b) {
+    const float bh = b.h + b.l, bl = __fsub_rn(b.l, __fsub_rn(bh, b.h));
+    const float q = a.h / bh;
+    const float r = fmaf(-q, bh, a.h) + fmaf(-q, bl, a.l);
+    const float c = r / bh;
+    return c == c ? q + c : q;
+  }
+  __device__ __forceinline__ bool positive() const { return h + l > 0.f; }
+};
+
+// v into CTA `rank`'s copy of the shared-memory slot p.
+template <typename S> __device__ __forceinline__ void store_cluster(S *p, int rank, const S &v) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(tc::smem_u32(p)), "r"(rank));
+  unsigned long long bits;
+  static_assert(sizeof(S) == 8, "one 8-byte store");
+  memcpy(&bits, &v, 8);
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(bits) : "memory");
+}
+
+struct CoopArgs {
+  Geom g;
+  const void *Vt, *U;
+  void *W, *R, *P, *Q;
+  int p, ld, max_iter, rows_per_cta, inv_rows, cluster;
+  double rtol2, shift;
+  double *part;
+  int *ctl;
+};
+
+template <typename T>
+__device__ __forceinline__ Pack<T> ldp(const T *x) {  // plain load: other CTAs write the blocks
+  return Pack<T>::load_rw(x);
+}
+
+// Row i of (H + sigma) applied to the values at(offset): the point's and its neighbours'.  A
+// neighbour outside the grid is read at the point itself and counted as zero, so the loads of
+// all points are issued together, without branches between them.
+template <typename T, typename F>
+__device__ __forceinline__ Pack<T> stencil_sum(const Geom &g, int i, int ld, T diag,
+                                               const Pack<T> &xc, F &&at) {
+  constexpr int N = Pack<T>::N;
+  const unsigned r = (unsigned)i / (unsigned)g.nx;
+  const int ix = i - (int)r * g.nx;
+  const unsigned iz = r / (unsigned)g.ny;
+  const int iy = (int)r - (int)iz * g.ny;
+  const int sy = g.nx * ld, sz = g.nx * g.ny * ld;
+  const bool bx0 = ix > 0, bx1 = ix < g.nx - 1, by0 = iy > 0, by1 = iy < g.ny - 1;
+  const T cx = (T)g.c[0], cy = (T)g.c[1], cz = (T)g.c[2];
+  const Pack<T> x0 = at(bx0 ? -ld : 0), x1 = at(bx1 ? ld : 0);
+  const Pack<T> y0 = at(by0 ? -sy : 0), y1 = at(by1 ? sy : 0);
+  Pack<T> y;
+  if (g.dim == 3) {
+    const bool bz0 = iz > 0, bz1 = (int)iz < g.nz - 1;
+    const Pack<T> z0 = at(bz0 ? -sz : 0), z1 = at(bz1 ? sz : 0);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const T s0 = (bx0 ? x0.v[k] : T(0)) + (bx1 ? x1.v[k] : T(0));
+      const T s1 = (by0 ? y0.v[k] : T(0)) + (by1 ? y1.v[k] : T(0));
+      const T s2 = (bz0 ? z0.v[k] : T(0)) + (bz1 ? z1.v[k] : T(0));
+      y.v[k] = diag * xc.v[k] - cx * s0 - cy * s1 - cz * s2;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const T s0 = (bx0 ? x0.v[k] : T(0)) + (bx1 ? x1.v[k] : T(0));
+      const T s1 = (by0 ? y0.v[k] : T(0)) + (by1 ? y1.v[k] : T(0));
+      y.v[k] = diag * xc.v[k] - cx * s0 - cy * s1;
+    }
+  }
+  return y;
+}
+
+// L: neighbouring lanes that reduce one column
+template <typename T, bool JAC, int L>
+__global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
+  constexpr int N = Pack<T>::N;
+  constexpr bool kFused = std::is_same<T, float>::value;
+  extern __shared__ __align__(16) double sm[];
+  __shared__ int ok_sh, nact_sh;
+  const Geom &g = A.g;
+  const int ld = A.ld, nv = ld / N, nr = kCoopThreads / nv;
+  const int tx = threadIdx.x % nv, ty = threadIdx.x / nv;
+  const bool on = ty < nr;
+  const int nra = min(nr, A.rows_per_cta);  // rows of threads that hold points
+  const int col = tx * N, G = gridDim.x;
+  const int r0 = blockIdx.x * A.rows_per_cta;
+  const int r1 = min(r0 + A.rows_per_cta, (int)g.n);
+  const T *Vt = (const T *)A.Vt, *U = (const T *)A.U;
+  T *W = (T *)A.W, *R = (T *)A.R;
+  const T shift = (T)A.shift;
+  // shared memory: per-column state, 1 / diag of the CTA's points, the cluster's partials
+  // [2][CTA][3 ld], the threads' sums
+  using S = Sum<T>;
+  double *target = sm;
+  S *rho = reinterpret_cast<S *>(target + ld);
+  T *al = reinterpret_cast<T *>(rho + ld), *be = al + ld;
+  int *act = reinterpret_cast<int *>(be + ld);
+  T *inv_sh = reinterpret_cast<T *>(act + ld);
+  S *xch = reinterpret_cast<S *>(inv_sh + A.inv_rows);
+  T *rows = reinterpret_cast<T *>(xch + (A.cluster ? 6 * G * ld : 0));
+  S *tot = reinterpret_cast<S *>(rows);  // (the threads' sums are read before)
+  constexpr int jstep = kCoopThreads / L;
+  const int lane = threadIdx.x & (L - 1);
+  const int jw = (int)(threadIdx.x & ~31u) / L, jl = (int)(threadIdx.x & 31) / L;
+  unsigned epoch = 0;
+  int odd = 0;
+
+  if (JAC && A.inv_rows) {
+    for (int i = r0 + (int)threadIdx.x; i < r1; i += kCoopThreads)
+      inv_sh[i - r0] = T(1) / (__ldg(Vt + i) + shift);
+    __syncthreads();
+  }
+  auto inv_of = [&](int i, T dg) -> T { return A.inv_rows ? inv_sh[i - r0] : T(1) / dg; };
+
+  // All CTAs arrive, and see what the others wrote before.
+  auto meet = [&]() -> bool {
+    if (G == 1) {
+      __syncthreads();
+      return true;
+    }
+    if (A.cluster) {
+      cluster_barrier();
+      return true;
+    }
+    epoch += G;
+    return grid_barrier(A.ctl, epoch, &ok_sh);
+  };
+
+  // Totals over the grid of the per-thread sums acc[c][k] (column col + k): over the CTA's rows,
+  // then over the CTAs, in the same order in every CTA; one lane a column gets fin(j, sums).
+  // A cluster's partials go straight into every member's shared memory.
+  auto total = [&](auto &acc, auto &&fin) -> bool {
+    constexpr int NC = sizeof(acc) / sizeof(acc[0]);
+    const int w = NC * ld, pitch = w | 1;
+    __syncthreads();
+    if (ty < nra) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int k = 0; k < N; ++k) rows[ty * pitch + c * ld + col + k] = acc[c][k];
+    }
+    __syncthreads();
+    // alternate buffers: a CTA may still read the last totals' partials
+    S *part = reinterpret_cast<S *>(A.part) + odd * 3 * G * ld;
+    S *mine = xch + odd * 3 * G * ld;
+    odd ^= 1;
+    for (int jb = jw; jb < ld; jb += jstep) {  // (whole warps)
+      const int j = jb + jl;
+      S s[NC];
+      if (j < ld)
+#pragma unroll 4
+        for (int y = lane; y < nra; y += L)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) s[c].add(rows[y * pitch + c * ld + j]);
+#pragma unroll
+      for (int o = L >> 1; o > 0; o >>= 1)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c].add(s[c].down(o));
+      if (G == 1) {
+        if (lane == 0 && j < ld) fin(j, s);
+      } else if (A.cluster) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const S v = s[c].from(0, L);
+          if (j < ld)
+            for (int r = lane; r < G; r += L) store_cluster(mine + blockIdx.x * w + c * ld + j, r, v);
+        }
+      } else if (lane == 0 && j < ld) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) part[blockIdx.x * w + c * ld + j] = s[c];
+      }
+    }
+    if (G > 1) {
+      if (!meet()) return false;
+      // the CTAs' partials: a cluster's are here; a grid's come from L2 as whole lines, summed
+      // in `gg` interleaved groups first
+      const S *from = mine;
+      int terms = G, pitch2 = w;
+      if (!A.cluster) {
+        const int gg = max(1, min(G, max(kSumThreads<T>, min(kCoopThreads, 4 * w)) / w));
+        pitch2 = w | 1;
+        for (int t = threadIdx.x; t < gg * w; t += kCoopThreads) {
+          const int q = t / w, e = t - q * w;
+          S s;
+#pragma unroll 8
+          for (int b = q; b < G; b += gg) s.add(S::load(part + b * w + e));
+          tot[q * pitch2 + e] = s;
+        }
+        __syncthreads();
+        from = tot;
+        terms = gg;
+      }
+      for (int jb = jw; jb < ld; jb += jstep) {  // (whole warps)
+        const int j = jb + jl;
+        S s[NC];
+        if (j < ld)
+#pragma unroll 4
+          for (int b = lane; b < terms; b += L)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s[c].add(from[b * pitch2 + c * ld + j]);
+#pragma unroll
+        for (int o = L >> 1; o > 0; o >>= 1)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) s[c].add(s[c].down(o));
+        if (lane == 0 && j < ld) fin(j, s);
+      }
+    }
+    __syncthreads();
+    return true;
+  };
+  if (A.cluster) cluster_barrier();  // every member runs before its shared memory is written
+
+  // start: R = U - (H + sigma) W (Z = R / d with the Jacobi preconditioner); FP64: P = R
+  bool ok;
+  {
+    T acc[3][N] = {};
+    if (on)
+      for (int i = r0 + ty; i < r1; i += nr) {
+        const long long o = (long long)i * ld + col;
+        const T dg = __ldg(Vt + i) + shift;
+        const Pack<T> wc = ldp(W + o), u = ldp(U + o);
+        const Pack<T> aw = stencil_sum<T>(g, i, ld, dg, wc, [&](int d) { return ldp(W + o + d); });
+        const T inv = JAC ? inv_of(i, dg) : T(1);
+        Pack<T> r;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const T rk = u.v[k] - aw.v[k];
+          r.v[k] = JAC ? rk * inv : rk;
+          acc[0][k] += rk * r.v[k];
+          acc[1][k] += u.v[k] * u.v[k];
+          acc[2][k] += rk * rk;
+        }
+        r.store(R + o);
+        if (!kFused) r.store((T *)A.P + o);
+      }
+    if (threadIdx.x == 0) nact_sh = 0;
+    ok = total(acc, [&](int j, S (&s)[3]) {
+      const double bb = s[1].value();
+      rho[j] = s[0];
+      target[j] = A.rtol2 * bb;
+      al[j] = be[j] = T(0);
+      const int a = (j < A.p) && (s[2].value() > A.rtol2 * bb) && (bb > 0.0);
+      act[j] = a;
+      if (a) atomicAdd(&nact_sh, 1);
+    });
+  }
+  int it = 0;
+  while (ok && nact_sh > 0 && it < A.max_iter) {
+    // FP32 alternates the two direction buffers; FP64 keeps P and stores Q = (H + sigma) P
+    const T *Po = (const T *)((kFused && (it & 1)) ? A.Q : A.P);
+    T *Pn = (T *)((kFused && !(it & 1)) ? A.Q : A.P);
+    T *Q = (T *)A.Q;
+    {
+      T acc[1][N] = {};
+      if (on) {
+        T b[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) b[k] = be[col + k];
+        const bool first = it == 0;
+        for (int i = r0 + ty; i < r1; i += nr) {
+          const long long o = (long long)i * ld + col;
+          const T dg = __ldg(Vt + i) + shift;
+          Pack<T> pc, q;
+          if (kFused) {
+            auto dir = [&](int d) {
+              Pack<T> r = ldp(R + o + d);
+              if (!first) {
+                const Pack<T> x = ldp(Po + o + d);
+#pragma unroll
+                for (int k = 0; k < N; ++k) r.v[k] += b[k] * x.v[k];
+              }
+              return r;
+            };
+            pc = dir(0);
+            q = stencil_sum<T>(g, i, ld, dg, pc, dir);
+            pc.store(Pn + o);
+          } else {
+            pc = ldp(Po + o);
+            q = stencil_sum<T>(g, i, ld, dg, pc, [&](int d) { return ldp(Po + o + d); });
+            q.store(Q + o);
+          }
+#pragma unroll
+          for (int k = 0; k < N; ++k) acc[0][k] += pc.v[k] * q.v[k];
+        }
+      }
+      ok = total(acc, [&](int j, S (&s)[1]) {
+        al[j] = (act[j] && s[0].positive()) ? (T)S::ratio(rho[j], s[0]) : T(0);
+      });
+      if (!ok) break;
+      if (threadIdx.x == 0) nact_sh = 0;  // (every thread has read it for this iteration)
+    }
+    {
+      constexpr int NC = JAC ? 2 : 1;
+      T acc[NC][N] = {};
+      if (on) {
+        T a[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) a[k] = al[col + k];
+        for (int i = r0 + ty; i < r1; i += nr) {
+          const long long o = (long long)i * ld + col;
+          const T dg = __ldg(Vt + i) + shift;
+          const Pack<T> pc = ldp(Pn + o);
+          Pack<T> q, w = ldp(W + o), r = ldp(R + o);
+          if (kFused)
+            q = stencil_sum<T>(g, i, ld, dg, pc, [&](int d) { return ldp(Pn + o + d); });
+          else
+            q = ldp(Q + o);
+          const T inv = JAC ? inv_of(i, dg) : T(1);
+#pragma unroll
+          for (int k = 0; k < N; ++k) {
+            w.v[k] += a[k] * pc.v[k];
+            if (JAC) {
+              r.v[k] -= a[k] * (q.v[k] * inv);
+              const T rk = dg * r.v[k];
+              acc[0][k] += rk * r.v[k];
+              acc[NC - 1][k] += rk * rk;
+            } else {
+              r.v[k] -= a[k] * q.v[k];
+              acc[0][k] += r.v[k] * r.v[k];
+            }
+          }
+          w.store(W + o);
+          r.store(R + o);
+        }
+      }
+      ok = total(acc, [&](int j, S (&s)[NC]) {
+        int a = act[j];
+        be[j] = (a && rho[j].positive()) ? (T)S::ratio(s[0], rho[j]) : T(0);
+        if (a) {
+          rho[j] = s[0];
+          a = s[NC - 1].value() > target[j];
+          act[j] = a;
+        }
+        if (a) atomicAdd(&nact_sh, 1);
+      });
+      if (!ok) break;
+      ++it;
+    }
+    if (!kFused && nact_sh > 0 && it < A.max_iter) {
+      if (on) {
+        T b[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) b[k] = be[col + k];
+        for (int i = r0 + ty; i < r1; i += nr) {
+          const long long o = (long long)i * ld + col;
+          const Pack<T> r = ldp(R + o);
+          Pack<T> pp = ldp(Pn + o);
+#pragma unroll
+          for (int k = 0; k < N; ++k) pp.v[k] = r.v[k] + b[k] * pp.v[k];
+          pp.store(Pn + o);
+        }
+      }
+      ok = meet();
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl[2] = it;
+}
+
+// CTAs of a solve and their grid points (*rows).  Up to a few vectors a thread in one cluster of
+// 16 CTAs (their barrier is in hardware and the partials stay in shared memory); FP64 only up
+// to one, since 16 SMs run 32 FP64 operations a clock.  Larger ones take at most one CTA per SM:
+// FP32 as many as give every thread the same number of vectors, FP64 all of them.
+constexpr int kCluster = 16;
+template <typename T> int coop_ctas(long long n, int ld, int *rows) {
+  const bool f32 = sizeof(T) == 4;
+  const long long nr = kCoopThreads / (ld / Pack<T>::N), sms = num_sms();
+  if (n > nr && n <= (f32 ? 4 : 1) * nr * kCluster && ld <= 64) {
+    *rows = (int)((n + kCluster - 1) / kCluster);
+    return kCluster;
+  }
+  const long long k = (n + nr * sms - 1) / (nr * sms);
+  *rows = (int)(f32 || k == 1 ? nr * k : (n + sms - 1) / sms);
+  return (int)((n + *rows - 1) / *rows);
+}
+
+template <typename T, bool JAC> const void *coop_kernel(int lanes) {
+  switch (lanes) {
+    case 1: return (const void *)k_cg_coop<T, JAC, 1>;
+    case 2: return (const void *)k_cg_coop<T, JAC, 2>;
+    case 4: return (const void *)k_cg_coop<T, JAC, 4>;
+    case 8: return (const void *)k_cg_coop<T, JAC, 8>;
+    case 16: return (const void *)k_cg_coop<T, JAC, 16>;
+    default: return (const void *)k_cg_coop<T, JAC, 32>;
+  }
+}
+
+}  // namespace
+
+template <typename T> bool cg_coop_eligible(long long n, int ld) {
+  return ld / Pack<T>::N <= 64 && n * ld * (long long)sizeof(T) <= kCoopBytes<T>;
+}
+
+template <typename T>
+op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, int p, int ld,
+                  double rtol, int max_iter, CGWork &w, int *iters, cudaStream_t st) {
+  constexpr int N = Pack<T>::N;
+  int rows = 0;
+  const int G = coop_ctas<T>(g.n, ld, &rows);
+  const bool cluster = G == kCluster;
+  CoopArgs a{};
+  a.g = g;
+  a.Vt = Vt;
+  a.U = U;
+  a.W = W;
+  a.R = w.R;
+  a.P = w.P;
+  a.Q = w.Q;
+  a.p = p;
+  a.ld = ld;
+  a.max_iter = max_iter;
+  a.rows_per_cta = rows;
+  a.inv_rows = w.jacobi && rows <= 8192 ? (rows + 1) / 2 * 2 : 0;  // (8-byte alignment after it)
+  a.rtol2 = rtol * rtol;
+  a.shift = g.cdiag + sigma;
+  a.part = w.part;
+  a.ctl = w.ctl;
+  a.cluster = cluster;
+  // as laid out in the kernel; the threads' sums have an odd pitch
+  const size_t smem = (size_t)ld * (2 * sizeof(double) + 2 * sizeof(T) + sizeof(int)) +
+                      (size_t)a.inv_rows * sizeof(T) + (cluster ? (size_t)6 * G * ld * 8 : 0) +
+                      std::max(((size_t)kCoopThreads * N * 3 + kCoopThreads / (ld / N) + 1) * sizeof(T),
+                               (size_t)(2 * kCoopThreads + 3 * ld + 2) * 8);
+  OP_CUDA(cudaMemsetAsync(w.ctl, 0, 256, st));
+  void *args[] = {&a};
+  int lanes = 1;
+  while (lanes < 32 && 2 * lanes * ld <= kSumThreads<T>) lanes *= 2;
+  const void *fn = w.jacobi ? coop_kernel<T, true>(lanes) : coop_kernel<T, false>(lanes);
+  OP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  prof_begin(w.prof, PK_CG_APPLY, st);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(G);
+  cfg.blockDim = dim3(kCoopThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  if (cluster) {
+    OP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kCluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  OP_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
+  count_launch();
+  prof_end(w.prof, st);
+  OP_CUDA(cudaMemcpyAsync(w.host_ctl, w.ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
+  OP_CUDA(cudaStreamSynchronize(st));
+  prof_harvest(w.prof);
+  if (w.host_ctl[3]) {
+    set_error("the cooperative CG gave up a bounded wait of its grid barrier");
+    return OP_ERR_TIMEOUT;
+  }
+  *iters = w.host_ctl[2];
+  w.expect_iters = *iters;
+  return OP_OK;
+}
+
+#define OPEVO_INST(T)                                                                          \
+  template bool cg_coop_eligible<T>(long long, int);                                           \
+  template op_status cg_coop<T>(const Geom &, const T *, double, const T *, T *, int, int,     \
+                                double, int, CGWork &, int *, cudaStream_t);
+OPEVO_INST(float)
+OPEVO_INST(double)
+#undef OPEVO_INST
+
+}  // namespace opevo
