@@ -244,7 +244,7 @@ __device__ __forceinline__ void gj32_body(int p, int ld, const double *__restric
     }
   bool bad = false;
 #pragma unroll 1
-  for (int k0 = 0; k0 < 128; k0 += kG) {
+  for (int k0 = 0; k0 < p; k0 += kG) {  // (the padding is an identity block: its pivots do nothing)
     const int ak = k0 >> 5, r0 = k0 & 31;
     // publish the pivot rows (owners: a == ak, ty in [r0, r0 + kG)) and columns
     // (owners: b == ak, tx in [r0, r0 + kG))

@@ -592,29 +592,62 @@ __device__ __forceinline__ void digit_pairs(double a, double b, int e, uint32_t 
   }
 }
 
+// High word of |x| (0 for NaN): the exponent of the largest |x| is the exponent field of the
+// largest of these.  Comparing them takes an integer instruction a value; fmax runs on the FP64
+// pipe, two a clock and SM, which alone took longer than reading the values.
+__device__ __forceinline__ uint32_t mag_hi(double x) {
+  const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+  return h > 0x7FF00000u || (h == 0x7FF00000u && __double2loint(x) != 0) ? 0u : h;
+}
+// Exponent of the largest |value| from its high word: |value| < 2^e (0 for zeros and
+// subnormals, whose digits are zero).
+__device__ __forceinline__ int exponent_of_hi(uint32_t h) {
+  return h < 0x00100000u ? 0 : exponent_of(__hiloint2double((int)h, 0));
+}
+
 // Column exponents of Y = [U W] (nc = ld or 2 ld columns) over grid points [x0, x0 + m),
-// encoded as e + 4096 (0: all zero); grid (column blocks of 256, row splits).
-__global__ void k_colexp(const double *__restrict__ U, const double *__restrict__ W, int ld,
-                         int nc, long long x0, long long m, int *__restrict__ enc) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nc) return;
-  const double *X = c < ld ? U : W;
-  const int cc = c < ld ? c : c - ld;
+// encoded as e + 4096 (0: all zero).  Blocks of up to 32 column pairs by 256 / pairs rows;
+// grid (column blocks, row splits).  Bound by HBM: 4.3 GB (n = 262144, p = 1024) in
+// 0.62 ms, 1.06 ms with fmax.
+__global__ void __launch_bounds__(256)
+    k_colexp(const double *__restrict__ U, const double *__restrict__ W, int ld, int nc,
+             long long x0, long long m, int *__restrict__ enc) {
+  __shared__ uint32_t red[512];
+  const int bx = blockDim.x, tx = threadIdx.x, ty = threadIdx.y, by = blockDim.y;
+  const int c = (blockIdx.x * bx + tx) * 2;
   const long long per = (m + gridDim.y - 1) / gridDim.y;
   const long long r0 = (long long)blockIdx.y * per;
   const long long r1 = r0 + per < m ? r0 + per : m;
-  const double *col = X + x0 * ld + cc;
-  double mx = 0.0, m1 = 0.0, m2 = 0.0, m3 = 0.0;
-  long long r = r0;
-  for (; r + 4 <= r1; r += 4) {  // four independent loads in flight per thread
-    mx = fmax(mx, fabs(col[r * ld]));
-    m1 = fmax(m1, fabs(col[(r + 1) * ld]));
-    m2 = fmax(m2, fabs(col[(r + 2) * ld]));
-    m3 = fmax(m3, fabs(col[(r + 3) * ld]));
+  uint32_t ha = 0, hb = 0;
+  if (c < nc) {
+    const double *col = (c < ld ? U + c : W + (c - ld)) + x0 * ld;
+    long long r = r0 + ty;
+    for (; r + 3 * by < r1; r += 4 * by) {  // four independent loads in flight per thread
+      double2 v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        v[q] = __ldg(reinterpret_cast<const double2 *>(col + (r + q * by) * ld));
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        ha = max(ha, mag_hi(v[q].x));
+        hb = max(hb, mag_hi(v[q].y));
+      }
+    }
+    for (; r < r1; r += by) {
+      const double2 v = __ldg(reinterpret_cast<const double2 *>(col + r * ld));
+      ha = max(ha, mag_hi(v.x));
+      hb = max(hb, mag_hi(v.y));
+    }
   }
-  for (; r < r1; ++r) mx = fmax(mx, fabs(col[r * ld]));
-  mx = fmax(fmax(mx, m1), fmax(m2, m3));
-  if (mx > 0.0) atomicMax(enc + c, exponent_of(mx) + 4096);
+  red[2 * (ty * bx + tx)] = ha;
+  red[2 * (ty * bx + tx) + 1] = hb;
+  __syncthreads();
+  const int t = ty * bx + tx;
+  if (t < 2 * bx && blockIdx.x * bx * 2 + t < nc) {
+    uint32_t h = 0;
+    for (int y = 0; y < by; ++y) h = max(h, red[2 * y * bx + t]);
+    if (h >= 0x00100000u) atomicMax(enc + blockIdx.x * bx * 2 + t, exponent_of_hi(h) + 4096);
+  }
 }
 
 __global__ void k_decode_exp(const int *__restrict__ enc, int *__restrict__ e, int n) {
@@ -684,15 +717,15 @@ __global__ void __launch_bounds__(256)
   if (r >= m) return;
   const double *ur = U + (x0 + r) * ld;
   const double *wr = W ? W + (x0 + r) * ld : nullptr;
-  double mx = 0.0;
+  uint32_t mx = 0;
+#pragma unroll 4
   for (int k = 2 * lane; k < kdim; k += 64) {
     const double2 v = *reinterpret_cast<const double2 *>(k < ld ? ur + k : wr + (k - ld));
-    mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+    mx = max(mx, max(mag_hi(v.x), mag_hi(v.y)));
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  mx = __reduce_max_sync(0xffffffffu, mx);
   constexpr int kDigits = ND;
-  const int e = exponent_of(mx);
+  const int e = exponent_of_hi(mx);
   if (lane == 0) erow[r] = e;
   for (int k = 8 * lane; k < kdim; k += 256) {
     const double *src = k < ld ? ur + k : wr + (k - ld);
@@ -867,7 +900,9 @@ int gram_tiles(int nc, int *nI, int *nJ, int *npt = nullptr) {
 // (two SMs each).
 int gram_ranges(int npt, long long m) {
   const int slots = std::max(1, num_sms() / 2);
-  const long long maxr = std::max<long long>(1, (m + 1023) / 1024);
+  // at least the 256 grid points between two read-outs each: a range of a small Gram is then
+  // one read-out long (n = 1024, p = 8: 70 -> 34 us)
+  const long long maxr = std::max<long long>(1, (m + 255) / 256);
   int best = 1;
   double best_eff = 0.0;
   for (int r = 1; r <= 64 && r <= maxr; ++r) {
@@ -962,9 +997,10 @@ op_status gram_fp64tc(long long n, int p, int ld, const double *U, const double 
     const long long m = std::min(rows, n - x0);
     const long long xp = (m + 63) / 64 * 64;
     OP_CUDA(cudaMemsetAsync(cv.enc, 0, (size_t)nc * sizeof(int), st));
-    const int ysplit = (int)std::min<long long>(std::max<long long>(1, m / 512),
-                                                std::max(1, 4 * num_sms() / ((nc + 255) / 256)));
-    k_colexp<<<dim3((nc + 255) / 256, ysplit), 256, 0, st>>>(U, W, ld, nc, x0, m, cv.enc);
+    const int bx = std::min(32, nc / 2), by = 256 / bx, gx = (nc / 2 + bx - 1) / bx;
+    const int ysplit = (int)std::max<long long>(
+        1, std::min<long long>((m + 8 * by - 1) / (8 * by), 8 * num_sms() / gx));
+    k_colexp<<<dim3(gx, ysplit), dim3(bx, by), 0, st>>>(U, W, ld, nc, x0, m, cv.enc);
     count_launch();
     k_decode_exp<<<(nc + 255) / 256, 256, 0, st>>>(cv.enc, cv.e2, nc);
     count_launch();
