@@ -16,8 +16,10 @@
 namespace opevo {
 namespace tc {
 
-// Iteration limit of every mbarrier wait (each poll sleeps ~64 ns): about a second.
+// Iteration limit of every mbarrier wait (a poll sleeps ~64 ns once the first few thousand
+// found nothing: a sleeping thread sees a completion late): about a second.
 constexpr long long kSpinLimit = 1ll << 24;
+constexpr long long kSpinAwake = 4096;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -53,7 +55,7 @@ __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   for (long long i = 0; i < kSpinLimit; ++i) {
     if (mbar_test(bar, parity)) return true;
-    __nanosleep(64);
+    if (i > kSpinAwake) __nanosleep(64);
   }
   return false;
 }
@@ -66,12 +68,12 @@ __device__ __forceinline__ uint64_t global_ns() {
 
 // Wait for the phase of `parity` of `bar` in a warp-specialised kernel: false once
 // limit_ns nanoseconds have passed (the waiter then sets *abort) or once another role
-// has set *abort.
+// has set *abort.  The clock and *abort are read once in 256 polls (see tma::bar_wait).
 __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort,
                                               uint64_t limit_ns) {
   const uint32_t a = smem_u32(bar);
   uint64_t t0 = 0;
-  for (;;) {
+  for (uint32_t polls = 1;; ++polls) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -81,6 +83,7 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, vo
         : "r"(a), "r"(parity)
         : "memory");
     if (ok) return true;
+    if (polls & 255u) continue;
     if (*abort) return false;
     const uint64_t now = global_ns();
     if (t0 == 0) {
