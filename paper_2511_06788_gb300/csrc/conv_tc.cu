@@ -8,13 +8,24 @@
 // (27 taps, zero outside the grid) or the point itself (1 tap).
 //
 // Tiling: one CTA per 128 grid points (the MMA's M), all output channels at once
-// (N = Cout rounded up to 16, at most 128), K in slabs of 64 (one 128-byte row of BF16
-// per operand row, 128-byte swizzled K-major).  The 256 threads gather a slab of A
-// (converting FP32 to BF16, round to nearest) and copy the slab of the weights, which a
-// small kernel has laid out once per call as BF16 [Cout][K] (zero padded); one thread
-// issues the four K = 16 MMAs of the slab.  Two slabs are staged in turn: the gather of
-// slab s + 1 runs while the tensor core works on slab s.  Every wait is bounded; a wait
-// that gives up sets the error word and the CTA writes nothing.
+// (N = Cout rounded up to 16, at most 128), one FP32 accumulator, K in order.  Two kernels with
+// the same products in the same order (bit-identical results):
+//
+// k_conv_tma (Cin a multiple of 8, or few K values).  A first pass rounds X to BF16 once, into a copy with one
+// point of zeros around the grid, so a tap of a run of points is the same run shifted by a
+// constant number of rows: TMA loads A as boxes of 128 rows, 64, 32 or 16 channels wide, and two
+// 8-wide boxes for a K step that straddles two taps.  No value is gathered or converted again;
+// the tiles run over the padded points between the first and the last grid point (about 9 %
+// more at 48^3).  A stage of the ring holds up to 64 K values (as many pieces as fit).  One thread
+// loads, one issues the MMAs, four warps write the outputs.  What is left is the issue of the
+// copies and MMAs, 500 to 700 clocks a piece for one thread each.  The 11 layers at 48^3, widths
+// 24, 48, 96, p = 64: 0.50 ms and 0.10 ms for the copies, by k_conv_tc 1.37 ms.
+//
+// k_conv_tc (other layers).  K in slabs of 64; the 256 threads gather a slab of A from FP32 (27
+// taps, zero padding) and convert it, one thread issues the slab's MMAs; the gather of slab
+// s + 1 runs while the tensor core works on slab s.
+//
+// Every wait is bounded; a wait that gives up sets the error word and the CTA writes nothing.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -22,6 +33,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "tc.cuh"
+#include "tma.cuh"
 
 namespace opevo {
 namespace {
@@ -229,19 +241,330 @@ __global__ void __launch_bounds__(256) k_conv_tc(const ConvTc a) {
   }
 }
 
+// ---- TMA-fed kernel -------------------------------------------------------------------
+constexpr int kTmaThreads = 192;           // producer, MMA and four epilogue warps
+constexpr int kMaxStages = 8;
+constexpr uint64_t kWaitNs = 2000000000ull;
+
+// BF16 weights as k_conv_wt, and the BF16 copy of X: rows of cin values, the grid points with
+// one point of zeros around them (pad = 1, row ((z + 1) Np + y + 1) Np + x + 1, Np = N + 2) or
+// as they are (pad = 0); or (gcin > 0) the gathered rows themselves, cin = K rounded up values of
+// the taps of gcin channels.  One thread per 8 values.
+__global__ void k_conv_prep(const float *__restrict__ W, int K, int cout, int Kp, int coutp,
+                            uint16_t *__restrict__ Wt, const float *__restrict__ X, int N, int cin,
+                            int pad, int gcin, uint16_t *__restrict__ Xb) {
+  const long long wtot = (long long)coutp * Kp, step = (long long)gridDim.x * blockDim.x;
+  const long long e0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  for (long long e = e0; e < wtot; e += step) {
+    const int co = (int)(e / Kp), k = (int)(e % Kp);
+    Wt[e] = (uint16_t)bf16_bits((co < cout && k < K) ? W[(long long)k * cout + co] : 0.f);
+  }
+  const unsigned Np = (unsigned)(N + 2 * pad), nv = (unsigned)cin / 8;
+  const long long total = (long long)Np * Np * Np * nv;
+  for (long long e = e0; e < total; e += step) {
+    const unsigned q = (unsigned)(e / nv), v = (unsigned)(e - (long long)q * nv);
+    const unsigned r = q / Np;
+    const int x = (int)(q - r * Np) - pad, y = (int)(r % Np) - pad, z = (int)(r / Np) - pad;
+    uint4 o = make_uint4(0, 0, 0, 0);
+    if (gcin > 0) {
+      ConvTc a;
+      a.X = X;
+      a.N = N;
+      a.taps = K == gcin ? 1 : 27;
+      a.cin = gcin;
+      a.K = K;
+      o = gather8(a, x, y, z, true, 8 * (int)v);
+    } else if (x >= 0 && x < N && y >= 0 && y < N && z >= 0 && z < N) {
+      const float4 *src = reinterpret_cast<const float4 *>(
+          X + (((long long)z * N + y) * N + x) * cin + 8 * v);
+      const float4 a = __ldg(src), b = __ldg(src + 1);
+      o = make_uint4(bf16_bits(a.x) | (bf16_bits(a.y) << 16), bf16_bits(a.z) | (bf16_bits(a.w) << 16),
+                     bf16_bits(b.x) | (bf16_bits(b.y) << 16), bf16_bits(b.z) | (bf16_bits(b.w) << 16));
+    }
+    *reinterpret_cast<uint4 *>(Xb + e * 8) = o;
+  }
+}
+
+// The K axis as pieces: `width` values (64, 32 or 16) of one tap from channel `off`, or (width 8)
+// the last 8 channels of a tap and the first 8 of the next.  Consecutive pieces share a stage
+// while they are at most 64 K values together.  The host lists them: a single thread walking the
+// channels took longer per piece (some 500 clocks) than the copies.
+struct __align__(16) KPiece {
+  int row, row2;        // the tap's row shift; of the next tap (width 8)
+  uint16_t off;
+  uint8_t width, stage;  // stage: K values of the stage that starts here, 0: the same stage
+};
+constexpr int kMaxPieces = 320;  // (27 taps of at most 512 channels: at most 11 pieces a tap)
+struct KPieces {
+  int count;
+  KPiece p[kMaxPieces];
+};
+
+struct ConvTma {
+  const float *bias;
+  float *Z, *A;
+  int N, pad, cout, coutp, stages;
+  int q0, q1;            // first output row and one past the last
+  int *err;
+};
+
+// Shared-memory descriptors of K-major operands: rows of 64 or 32 bytes swizzled over 8 rows,
+// and core matrices of 8 rows x 16 bytes without swizzle (the next 8 rows 128 bytes on, the
+// next 8 K values 2048 bytes on).
+__device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr, int lead, int stride, int layout) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lead >> 4) << 16) |
+         ((uint64_t)(stride >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)layout << 61);
+}
+
+__global__ void __launch_bounds__(kTmaThreads)
+    k_conv_tma(const __grid_constant__ CUtensorMap a64, const __grid_constant__ CUtensorMap a32,
+               const __grid_constant__ CUtensorMap a16, const __grid_constant__ CUtensorMap a8,
+               const __grid_constant__ CUtensorMap b64, const __grid_constant__ CUtensorMap b32,
+               const __grid_constant__ CUtensorMap b16, const __grid_constant__ KPieces pc,
+               const ConvTma c) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ uint64_t full[kMaxStages], empty[kMaxStages], fin;
+  __shared__ uint32_t tmem_sh;
+  __shared__ int abort_sh;
+  __shared__ KPiece piece[kMaxPieces];
+  for (int i = threadIdx.x; i < pc.count; i += kTmaThreads) piece[i] = pc.p[i];
+  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q0 = c.q0 + blockIdx.x * kCM;
+  const uint32_t ncols = c.coutp <= 32 ? 32u : (c.coutp <= 64 ? 64u : 128u);
+  const int stage_bytes = kAPiece + c.coutp * 128;
+  if (warp == 1) tc::tmem_alloc(&tmem_sh, ncols);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < c.stages; ++s) {
+      tc::mbar_init(&full[s], 1);
+      tc::mbar_init(&empty[s], 1);
+    }
+    tc::mbar_init(&fin, 1);
+    tc::fence_mbar_init();
+    abort_sh = 0;
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = tmem_sh;
+  volatile int *abort = &abort_sh;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0, slot = 0, o = 0, k = 0;
+      uint32_t phase = 1;  // of the slot's last release (the first use of a slot passes)
+      uint8_t *as = smem;
+      for (int i = 0; i < pc.count; ++i) {
+        const KPiece s = piece[i];
+        if (s.stage) {  // a new stage
+          if (it > 0 && ++slot == c.stages) {
+            slot = 0;
+            phase ^= 1;
+          }
+          if (it >= c.stages && !tc::wait_or_abort(&empty[slot], phase, abort, kWaitNs)) break;
+          as = smem + slot * stage_bytes;
+          o = 0;
+          tma::bar_expect(&full[slot], (uint32_t)(s.stage * (2 * kCM + 2 * c.coutp)));
+          ++it;
+        }
+        uint64_t *bar = &full[slot];
+        uint8_t *ap = as + o * 2 * kCM, *bp = as + kAPiece + o * 2 * c.coutp;
+        const int r = q0 + s.row;
+        int len = s.width;
+        if (s.width == 64) {
+          tma::load_2d(ap, &a64, s.off, r, bar);
+          tma::load_2d(bp, &b64, k, 0, bar);
+        } else if (s.width == 32) {
+          tma::load_2d(ap, &a32, s.off, r, bar);
+          tma::load_2d(bp, &b32, k, 0, bar);
+        } else {
+          if (s.width == 16) {
+            tma::load_2d(ap, &a16, s.off, r, bar);
+          } else {
+            tma::load_2d(ap, &a8, s.off, r, bar);
+            tma::load_2d(ap + 16 * kCM, &a8, 0, q0 + s.row2, bar);
+            len = 16;
+          }
+          tma::load_2d(bp, &b16, k, 0, bar);
+        }
+        o += len;
+        k += len;
+      }
+      // the copies issued last land before the CTA may exit
+      for (int u = it - 1; u >= 0 && u >= it - c.stages; --u)
+        tma::bar_wait(&full[u % c.stages], (uint32_t)((u / c.stages) & 1), kWaitNs);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = tc::idesc_bf16(kCM, c.coutp);
+      int it = 0, slot = 0, o = 0;
+      uint32_t acc = 0, phase = 0, as = 0;
+      for (int i = 0; i < pc.count; ++i) {
+        const KPiece s = piece[i];
+        if (s.stage) {
+          if (it > 0) {
+            tc::mma_commit(&empty[slot]);
+            if (++slot == c.stages) {
+              slot = 0;
+              phase ^= 1;
+            }
+          }
+          if (!tc::wait_or_abort(&full[slot], phase, abort, kWaitNs)) break;
+          tc::tc_fence_after();
+          as = tc::smem_u32(smem + slot * stage_bytes);
+          o = 0;
+          ++it;
+        }
+        const uint32_t ap = as + o * 2 * kCM, bp = as + kAPiece + o * 2 * c.coutp;
+        if (s.width == 64) {
+          const uint64_t ad = desc_kmajor(ap, 16, 1024, 2), bd = desc_kmajor(bp, 16, 1024, 2);
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks, acc = 1)
+            tc::mma_bf16(tmem, ad + 2 * ks, bd + 2 * ks, idesc, acc);
+          o += 64;
+        } else if (s.width == 32) {
+          const uint64_t ad = desc_kmajor(ap, 16, 512, 4), bd = desc_kmajor(bp, 16, 512, 4);
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks, acc = 1)
+            tc::mma_bf16(tmem, ad + 2 * ks, bd + 2 * ks, idesc, acc);
+          o += 32;
+        } else {
+          const uint64_t ad =
+              s.width == 16 ? desc_kmajor(ap, 16, 256, 6) : desc_kmajor(ap, 16 * kCM, 128, 0);
+          tc::mma_bf16(tmem, ad, desc_kmajor(bp, 16, 256, 6), idesc, acc);
+          acc = 1;
+          o += 16;
+        }
+      }
+      if (it > 0) tc::mma_commit(&fin);
+      else tc::mbar_arrive(&fin);
+      tma::bar_wait(&fin, 0u, kWaitNs);
+    }
+  } else {
+    int ok = 0;
+    if (lane == 0) ok = tc::wait_or_abort(&fin, 0u, abort, kWaitNs) && !*abort;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    if (ok) {
+      tc::tc_fence_after();
+      const int quarter = warp & 3, q = q0 + quarter * 32 + lane;
+      long long m = q;
+      bool in = q < c.q1;
+      if (c.pad) {
+        const unsigned Np = (unsigned)c.N + 2, r = (unsigned)q / Np;
+        const int x = (int)((unsigned)q - r * Np) - 1, y = (int)(r % Np) - 1, z = (int)(r / Np) - 1;
+        in = in && x >= 0 && x < c.N && y >= 0 && y < c.N && z >= 0 && z < c.N;
+        m = ((long long)z * c.N + y) * c.N + x;
+      }
+      const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16);
+      for (int c0 = 0; c0 < c.coutp; c0 += 8) {
+        float v[8];
+        tmem_ld8(tb + (uint32_t)c0, v);
+        if (!in) continue;
+        if (c.cout % 4 == 0) {
+#pragma unroll
+          for (int h = 0; h < 8; h += 4) {
+            if (c0 + h >= c.cout) continue;
+            float4 z, y;
+            const float *bi = c.bias ? c.bias + c0 + h : nullptr;
+            z.x = v[h] + (bi ? __ldg(bi) : 0.f);
+            z.y = v[h + 1] + (bi ? __ldg(bi + 1) : 0.f);
+            z.z = v[h + 2] + (bi ? __ldg(bi + 2) : 0.f);
+            z.w = v[h + 3] + (bi ? __ldg(bi + 3) : 0.f);
+            if (c.Z) *reinterpret_cast<float4 *>(c.Z + m * c.cout + c0 + h) = z;
+            if (c.A) {
+              y.x = z.x / (1.0f + expf(-z.x));
+              y.y = z.y / (1.0f + expf(-z.y));
+              y.z = z.z / (1.0f + expf(-z.z));
+              y.w = z.w / (1.0f + expf(-z.w));
+              *reinterpret_cast<float4 *>(c.A + m * c.cout + c0 + h) = y;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int co = c0 + j;
+            if (co >= c.cout) continue;
+            const float z = v[j] + (c.bias ? __ldg(c.bias + co) : 0.f);
+            if (c.Z) c.Z[m * c.cout + co] = z;
+            if (c.A) c.A[m * c.cout + co] = z / (1.0f + expf(-z));
+          }
+        }
+      }
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, ncols);
+  }
+  if (threadIdx.x == 0 && abort_sh) atomicExch(c.err, 1);
+}
+
+// Rows and row length of the BF16 copy (0: the layer is left to k_conv_tc).  Channels in 16-byte
+// groups: the padded points.  Other layers with few K values (the 4-channel first one): the
+// gathered rows, written once (at 48^3, 4 -> 24: 64 us in all, by k_conv_tc 73).  At most 8 GiB
+// beside the FP32 activations.
+long long copy_rows(int N, int taps, int cin) {
+  const long long m = taps == 27 && cin % 8 == 0 ? N + 2 : N;
+  return m * m * m;
+}
+int copy_len(int N, int taps, int cin) {
+  const int len = cin % 8 == 0 ? cin : (taps * cin <= 256 ? (taps * cin + 15) / 16 * 16 : 0);
+  return copy_rows(N, taps, cin) * len * 2 <= (8ll << 30) ? len : 0;
+}
+// Pieces of taps x cin K values over a copy of `rows` rows (Np points an axis with the padding).
+void list_pieces(int taps, int cin, int Np, long long rows, KPieces *out) {
+  auto shift = [&](int t) -> int {
+    if (t >= taps) return (int)rows;  // past the last row: zeros
+    return taps == 1 ? 0 : ((t / 9 - 1) * Np + (t / 3) % 3 - 1) * Np + t % 3 - 1;
+  };
+  int n = 0, used = kCK, first = 0, off = 0;
+  for (int t = 0; t < taps;) {
+    KPiece &p = out->p[n];
+    const int rem = cin - off;
+    p.width = (uint8_t)(rem >= 64 ? 64 : (rem >= 32 ? 32 : (rem >= 16 ? 16 : 8)));
+    p.off = (uint16_t)off;
+    p.row = shift(t);
+    p.row2 = shift(t + 1);
+    p.stage = 0;
+    const int len = p.width == 8 ? 16 : p.width;
+    if (used + len > kCK) {
+      first = n;
+      used = 0;
+    }
+    used += len;
+    out->p[first].stage = (uint8_t)used;
+    ++n;
+    off += p.width;
+    if (p.width == 8) {  // the first 8 channels of the next tap came along
+      ++t;
+      off = 8;
+    }
+    if (off >= cin) {
+      off = 0;
+      ++t;
+    }
+  }
+  out->count = n;
+}
+size_t weight_bytes(int taps, int cin, int cout) {
+  const long long Kp = ((long long)taps * cin + kCK - 1) / kCK * kCK;
+  return (size_t)(Kp * ((cout + 15) / 16 * 16) * 2 + 255) / 256 * 256;
+}
+
 }  // namespace
 
-size_t conv_tc_scratch_bytes(int taps, int cin, int cout) {
-  const long long Kp = ((long long)taps * cin + kCK - 1) / kCK * kCK;
-  const long long coutp = (cout + 15) / 16 * 16;
-  return (size_t)(Kp * coutp * 2 + 255) / 256 * 256;
+size_t conv_tc_scratch_bytes(int N, int taps, int cin, int cout) {
+  return weight_bytes(taps, cin, cout) +
+         (size_t)copy_rows(N, taps, cin) * copy_len(N, taps, cin) * 2;
 }
 
 op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const float *W,
                        const float *bias, float *Z, float *A, void *scratch, size_t scratch_bytes,
                        int *err, cudaStream_t st) {
   if (!X || !W || !scratch || !err || N < 1 || (taps != 1 && taps != 27) || cin < 1 ||
-      cout < 1 || cout > 128 || scratch_bytes < conv_tc_scratch_bytes(taps, cin, cout) ||
+      cout < 1 || cout > 128 || scratch_bytes < conv_tc_scratch_bytes(N, taps, cin, cout) ||
       ((uintptr_t)scratch & 15) != 0) {
     set_error("conv_bf16_tc: bad arguments (N=%d taps=%d cin=%d cout=%d)", N, taps, cin, cout);
     return OP_ERR_ARG;
@@ -249,6 +572,51 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
   if (cin % 8 == 0 && ((uintptr_t)X & 15) != 0) {
     set_error("conv_bf16_tc: X must be 16-byte aligned");
     return OP_ERR_ARG;
+  }
+  const int K = taps * cin, coutp = (cout + 15) / 16 * 16, Kp = (K + kCK - 1) / kCK * kCK;
+  const int clen = copy_len(N, taps, cin);
+  if (clen > 0 && (!Z || ((uintptr_t)Z & 15) == 0) &&
+      (!A || ((uintptr_t)A & 15) == 0)) {
+    uint16_t *Wt = (uint16_t *)scratch;
+    uint16_t *Xb = (uint16_t *)((char *)scratch + weight_bytes(taps, cin, cout));
+    const int gcin = cin % 8 == 0 ? 0 : cin, pad = taps == 27 && !gcin ? 1 : 0;
+    const long long rows = copy_rows(N, taps, cin);
+    const long long work = std::max(rows * (clen / 8), (long long)coutp * Kp);
+    k_conv_prep<<<(unsigned)std::min<long long>((work + 255) / 256, 16LL * num_sms()), 256, 0, st>>>(
+        W, K, cout, Kp, coutp, Wt, X, N, clen, pad, gcin, Xb);
+    count_launch();
+    OP_LAUNCH("k_conv_prep");
+    ConvTma c;
+    c.bias = bias;
+    c.Z = Z;
+    c.A = A;
+    c.N = N;
+    c.pad = pad;
+    c.cout = cout;
+    c.coutp = coutp;
+    c.err = err;
+    const int Np = N + 2;
+    c.q0 = pad ? Np * Np + Np + 1 : 0;
+    c.q1 = (int)rows - c.q0;
+    // with no more tiles than SMs a CTA has the SM to itself and is bound by the latency of its
+    // loads: as many stages as fit; else two CTAs per SM
+    const int tiles = (c.q1 - c.q0 + kCM - 1) / kCM, stage = kAPiece + coutp * 128;
+    c.stages = std::min(kMaxStages, ((tiles <= num_sms() ? 220 : 110) * 1024) / stage);
+    CUtensorMap ma[4], mb[3];
+    const int wid[4] = {64, 32, 16, 8};
+    for (int i = 0; i < 4; ++i)
+      OP_TRY(tma_map_2d_bf16(&ma[i], Xb, (uint64_t)clen, (uint64_t)rows, wid[i], kCM));
+    for (int i = 0; i < 3; ++i)
+      OP_TRY(tma_map_2d_bf16(&mb[i], Wt, (uint64_t)Kp, (uint64_t)coutp, wid[i], coutp));
+    KPieces pc;
+    list_pieces(gcin ? 1 : taps, clen, Np, rows, &pc);
+    const int smem = c.stages * (kAPiece + coutp * 128) + 1024;
+    OP_CUDA(cudaFuncSetAttribute(k_conv_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_conv_tma<<<(unsigned)tiles, kTmaThreads, smem, st>>>(
+        ma[0], ma[1], ma[2], ma[3], mb[0], mb[1], mb[2], pc, c);
+    count_launch();
+    OP_LAUNCH("k_conv_tma");
+    return OP_OK;
   }
   ConvTc a;
   a.X = X;
@@ -260,9 +628,9 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
   a.taps = taps;
   a.cin = cin;
   a.cout = cout;
-  a.coutp = (cout + 15) / 16 * 16;
-  a.K = taps * cin;
-  a.Kp = (a.K + kCK - 1) / kCK * kCK;
+  a.coutp = coutp;
+  a.K = K;
+  a.Kp = Kp;
   a.err = err;
   const long long wt = (long long)a.coutp * a.Kp;
   k_conv_wt<<<(unsigned)std::min<long long>((wt + 255) / 256, 4LL * num_sms()), 256, 0, st>>>(

@@ -594,7 +594,7 @@ op_status forward(opnet *net, const double *V) {
 // (k_flip into Wf, taps * cin * cout floats of scratch).  OPNET_CONV_BF16_TC runs it on the
 // tensor cores when cin <= 128 (the kernel's output-channel limit; BF16 operands, FP32
 // accumulation), otherwise it runs on the FP32 CUDA cores.  tc_ws: scratch of
-// conv_tc_scratch_bytes(taps, cout, cin) bytes for the tensor-core form.
+// conv_tc_scratch_bytes(N, taps, cout, cin) bytes for the tensor-core form.
 op_status conv_dgrad(int kind, const float *dZ, int N, int taps, int cin, int cout,
                      const float *W, float *Wf, float *dX, void *tc_ws, size_t tc_bytes, int *err,
                      cudaStream_t st) {
@@ -847,11 +847,11 @@ op_status opnet_create(opnet **out, const opnet_config *cfg) {
     for (int i = 0; i < kLayers; ++i) {
       const Layer &l = net->L[i];
       net->conv_ws_bytes =
-          std::max(net->conv_ws_bytes, conv_tc_scratch_bytes(l.taps, l.cin, l.cout));
+          std::max(net->conv_ws_bytes, conv_tc_scratch_bytes(l.grid, l.taps, l.cin, l.cout));
       // the tensor-core data gradient: the same kernel with cin and cout exchanged
       if (l.cin <= 128)
         net->conv_ws_bytes =
-            std::max(net->conv_ws_bytes, conv_tc_scratch_bytes(l.taps, l.cout, l.cin));
+            std::max(net->conv_ws_bytes, conv_tc_scratch_bytes(l.grid, l.taps, l.cout, l.cin));
     }
     s = net_alloc(net, &net->conv_ws, net->conv_ws_bytes);
   }
@@ -971,7 +971,7 @@ op_status opnet_conv(int kind, const float *X, int N, int taps, int cin, int cou
     OP_CUDA(cudaStreamSynchronize(st));
     return OP_OK;
   }
-  const size_t wb = conv_tc_scratch_bytes(taps, cin, cout);
+  const size_t wb = conv_tc_scratch_bytes(N, taps, cin, cout);
   void *ws = nullptr;
   OP_CUDA(cudaMalloc(&ws, wb + 256));
   int *err = (int *)((char *)ws + wb);
@@ -1001,7 +1001,7 @@ op_status opnet_conv_dgrad(int kind, const float *dZ, int N, int taps, int cin, 
   }
   cudaStream_t st = (cudaStream_t)stream;
   const size_t wf = ((size_t)taps * cin * cout * sizeof(float) + 255) / 256 * 256;
-  const size_t wb = conv_tc_scratch_bytes(taps, cout, cin);
+  const size_t wb = conv_tc_scratch_bytes(N, taps, cout, cin);
   void *ws = nullptr;
   OP_CUDA(cudaMalloc(&ws, wf + wb + 256));
   float *Wf = (float *)ws;

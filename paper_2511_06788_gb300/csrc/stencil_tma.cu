@@ -531,4 +531,34 @@ op_status tma_map_3d_bf16_sw(CUtensorMap *map, const void *base, uint64_t inner,
   return OP_OK;
 }
 
+op_status tma_map_2d_bf16(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows,
+                          uint32_t box_k, uint32_t box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) {
+    set_error("cuTensorMapEncodeTiled is not available from the driver");
+    return OP_ERR_CUDA;
+  }
+  if (((uintptr_t)base & 15) != 0 || inner % 8 != 0 || box_rows < 1 || box_rows > 256 ||
+      (box_k != 64 && box_k != 32 && box_k != 16 && box_k != 8)) {
+    set_error("tensor map: base or row pitch not 16-byte aligned, or bad box");
+    return OP_ERR_ARG;
+  }
+  cuuint64_t gd[2] = {inner, rows};
+  cuuint64_t gs[1] = {inner * 2};
+  cuuint32_t bx[2] = {box_k, box_rows};
+  cuuint32_t es[2] = {1, 1};
+  const CUtensorMapSwizzle sw = box_k == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                : box_k == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                : box_k == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                              : CU_TENSOR_MAP_SWIZZLE_NONE;
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), gd, gs, bx,
+                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    set_error("cuTensorMapEncodeTiled failed (CUresult %d)", (int)r);
+    return OP_ERR_CUDA;
+  }
+  return OP_OK;
+}
+
 }  // namespace opevo

@@ -39,6 +39,13 @@ op_status tma_map_2d_f32_sw128(CUtensorMap *map, const void *base, uint64_t inne
 op_status tma_map_3d_bf16_sw(CUtensorMap *map, const void *base, uint64_t inner,
                              uint64_t rows, uint64_t planes, uint32_t box_rows, uint32_t box_k);
 
+// 2-D BF16 tensor map over a row-major [rows][inner] array (inner a multiple of 8) with a box of
+// box_k x box_rows elements, box_k = 64, 32, 16 (rows of 2 box_k bytes in the 128-, 64- or
+// 32-byte swizzled K-major layout) or 8 (rows of 16 bytes, one after another).  Every inner
+// coordinate: a multiple of 8.
+op_status tma_map_2d_bf16(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows,
+                          uint32_t box_k, uint32_t box_rows);
+
 namespace tma {
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
