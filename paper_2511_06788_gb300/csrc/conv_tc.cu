@@ -601,7 +601,7 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
     // with no more tiles than SMs a CTA has the SM to itself and is bound by the latency of its
     // loads: as many stages as fit; else two CTAs per SM
     const int tiles = (c.q1 - c.q0 + kCM - 1) / kCM, stage = kAPiece + coutp * 128;
-    c.stages = std::min(kMaxStages, ((tiles <= num_sms() ? 220 : 110) * 1024) / stage);
+    c.stages = std::min(kMaxStages, ((tiles <= num_sms() ? 215 : 104) * 1024) / stage);
     CUtensorMap ma[4], mb[3];
     const int wid[4] = {64, 32, 16, 8};
     for (int i = 0; i < 4; ++i)

@@ -7,7 +7,7 @@
 //   forward  out[m][co] = b[co] + sum_k A[m][k] W[k][co],  A[m][t Cin + ci] = X[m + off_t][ci]
 //   dgrad    the same kernel on dZ with the tap-reversed, transposed weights
 //            (dX[m][ci] = sum_t sum_co dZ[m - off_t][co] W[t][ci][co]);
-//   wgrad    (FP32 CUDA cores) dW[k][co] = sum_m A[m][k] dZ[m][co] (split over point chunks, partials
+//   wgrad    (FP32 CUDA cores) dW[k][co] = sum_m A[m][k] dZ[m][co] (split over point runs, partials
 //            summed in a fixed order), with a row of ones appended to A so that
 //            the same pass yields db = sum_m dZ[m] as row K of the (K + 1) x Cout
 //            block that W and b form in the parameter vector.
@@ -269,14 +269,188 @@ __global__ void __launch_bounds__(256) k_wgrad(WgradArgs a) {
   }
 }
 
-// out[e] = sum_s part[s][e] (fixed order, FP32 partials summed in FP64).
-__global__ void k_reduce_parts(const float *__restrict__ part, int splits, long long count,
-                               float *__restrict__ out) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
+// ---- weight gradients over padded points (channel counts that are multiples of 4) --------
+// Xp and dZp are FP32 copies of X and dZ with one point of zeros around the grid (27 taps; the
+// arrays themselves for 1 tap), so A[q][t Cin + ci] = Xp[q + off_t][ci] needs no coordinates and
+// no bounds, and the taps dx = -1, 0, 1 of one (dz, dy) are one window of 3 Cin consecutive values
+// that starts Cin later for the next point:
+//   dW[(dz, dy)][k][co] = sum_q Xp[(q + off_dz,dy - 1) Cin + k] dZp[q][co],  k < 3 Cin.
+// A CTA takes ng of the nine (dz, dy), a range of k, all channels co and a run of points; a thread
+// 8 x 8 outputs of one (dz, dy) in FP32 (k 4 kt .. and 4 (kthr + kt) .., co likewise: a warp's
+// 16-byte shared loads are consecutive).  Points come 32 at a time by cp.async, two stages ahead.
+// Bound by the FP32 pipe (64 multiply-adds per four 16-byte shared loads).  At 48^3, widths 24,
+// 48, 96, p = 64, the 11 layers take 1.72 ms (57 GFLOP with the borders: 33 TFLOP/s), by k_wgrad 7.0.
+struct WgradPadArgs {
+  const float *X, *dZ;
+  float *part;       // [splits][K + 1][cout]
+  int cin, cout, K;
+  int win, kthr, kblocks, cothr, ng, Np, pad;
+  int q0, q1, rows;  // output points, rows of X
+  int chunk;         // points per split (multiple of 32)
+  int apitch, bpitch;  // floats of a stage's A window run (per (dz, dy)) and of its B rows
+};
+constexpr int kWP = 32, kWStages = 3;  // points per stage, stages
+
+__device__ __forceinline__ void cp_async16(float *dst, const float *src, bool in) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(in ? 16 : 0)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(512) k_wgrad_pad(const WgradPadArgs a) {
+  extern __shared__ __align__(16) float wsm[];
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int kb = blockIdx.x % a.kblocks, g0 = (blockIdx.x / a.kblocks) * a.ng;
+  const int per = a.kthr * a.cothr, gi = tid / per, r = tid - gi * per;
+  const int ct = r / a.kthr, kt = r - ct * a.kthr;
+  const bool on = gi < a.ng;
+  const int ka = 8 * a.kthr * kb + 4 * kt, kc = ka + 4 * a.kthr;  // this thread's k: ka .., kc ..
+  const int ca = 4 * ct, cc = ca + 4 * a.cothr;
+  const int qs = a.q0 + blockIdx.y * a.chunk;
+  const int qe = min(qs + a.chunk, a.q1);
+  const int stage = a.ng * a.apitch + a.bpitch;
+  const int arows = kWP + 2 * a.pad;
+  const long long xend = (long long)a.rows * a.cin;
+
+  auto load = [&](int s, int q) {
+    float *dst = wsm + s * stage;
+    for (int g = 0; g < a.ng; ++g) {
+      const int gg = g0 + g;
+      const int row = a.pad ? q + ((gg / 3 - 1) * a.Np + gg % 3 - 1) * a.Np - 1 : q;
+      const long long base = (long long)row * a.cin;
+      for (int e = 4 * tid; e < arows * a.cin; e += 4 * nt) {
+        const bool in = q < qe && base + e < xend;
+        cp_async16(dst + g * a.apitch + e, in ? a.X + base + e : a.X, in);
+      }
+    }
+    const long long base = (long long)q * a.cout, end = (long long)qe * a.cout;
+    for (int e = 4 * tid; e < kWP * a.cout; e += 4 * nt) {
+      const bool in = base + e < end;
+      cp_async16(dst + a.ng * a.apitch + e, in ? a.dZ + base + e : a.dZ, in);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  // the slack behind a stage's runs is read by threads past the last k or co: finite values
+  for (int e = tid; e < kWStages * stage; e += nt) wsm[e] = 0.f;
+  __syncthreads();
+  float acc[8][8], bias[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+  load(0, qs);
+  load(1, qs + kWP);
+  int s = 0;
+  for (int q = qs; q < qe; q += kWP) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    load(s == 0 ? 2 : s - 1, q + 2 * kWP);  // the stage read two steps ago
+    const float *B = wsm + s * stage + a.ng * a.apitch;
+    if (on) {
+      const float *A = wsm + s * stage + gi * a.apitch;
+#pragma unroll 4
+      for (int p = 0; p < kWP; ++p) {
+        const float4 x0 = *reinterpret_cast<const float4 *>(A + p * a.cin + ka);
+        const float4 x1 = *reinterpret_cast<const float4 *>(A + p * a.cin + kc);
+        const float4 z0 = *reinterpret_cast<const float4 *>(B + p * a.cout + ca);
+        const float4 z1 = *reinterpret_cast<const float4 *>(B + p * a.cout + cc);
+        const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+        const float z[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(x[i], z[j], acc[i][j]);
+      }
+    }
+    if (blockIdx.x == 0) {
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int c = tid + v * nt;
+        if (c < a.cout)
+          for (int p = 0; p < kWP; ++p) bias[v] += B[p * a.cout + c];
+      }
+    }
+    s = s == kWStages - 1 ? 0 : s + 1;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  float *dst = a.part + (long long)blockIdx.y * (a.K + 1) * a.cout;
+  if (on) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = (i < 4 ? ka : kc) + (i & 3);
+      if (k >= a.win) continue;
+      float *row = dst + (long long)((g0 + gi) * a.win + k) * a.cout;
+#pragma unroll
+      for (int j = 0; j < 8; j += 4) {
+        const int co = j < 4 ? ca : cc;  // (cout is a multiple of 4)
+        if (co < a.cout)
+          *reinterpret_cast<float4 *>(row + co) =
+              make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+      }
+    }
+  }
+  if (blockIdx.x == 0) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int c = tid + v * nt;
+      if (c < a.cout) dst[(long long)a.K * a.cout + c] = bias[v];
+    }
+  }
+}
+
+// Xp, dZp: the padded copies of k_wgrad_pad (C and D channels, multiples of 4).
+__global__ void k_wgrad_copy(int N, int C, const float *__restrict__ X, float *__restrict__ Xp, int D,
+                             const float *__restrict__ dZ, float *__restrict__ dZp) {
+  const unsigned Np = (unsigned)N + 2, nv = (unsigned)(C + D) / 4;
+  const long long total = (long long)Np * Np * Np * nv;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < splits; ++k) s += part[(long long)k * count + e];
-    out[e] = (float)s;
+    const unsigned q = (unsigned)(e / nv), v = (unsigned)(e - (long long)q * nv) * 4;
+    const unsigned r = q / Np;
+    const int x = (int)(q - r * Np) - 1, y = (int)(r % Np) - 1, z = (int)(r / Np) - 1;
+    const bool in = x >= 0 && x < N && y >= 0 && y < N && z >= 0 && z < N;
+    const long long m = ((long long)z * N + y) * N + x;
+    const bool first = v < (unsigned)C;
+    const float *src = first ? X + m * C + v : dZ + m * D + (v - C);
+    float *dst = first ? Xp + (long long)q * C + v : dZp + (long long)q * D + (v - C);
+    *reinterpret_cast<float4 *>(dst) =
+        in ? __ldg(reinterpret_cast<const float4 *>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// out[e] = sum_s part[s][e] (fixed order): blocks of 32 elements by 16 interleaved sums over the
+// splits, each an error-free pair of floats (two-sum, 48 bits; a warp's FP64 conversion and
+// addition take 64 clocks each), joined in FP64.  The 11 layers at 48^3: 467 us with one FP64 sum
+// an element, 293 us so (cold).
+__global__ void __launch_bounds__(512) k_reduce_parts(const float *__restrict__ part, int splits,
+                                                      long long count, float *__restrict__ out) {
+  __shared__ float2 red[16][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  for (long long e0 = blockIdx.x * 32ll; e0 < count; e0 += gridDim.x * 32ll) {
+    const long long e = e0 + x;
+    float h = 0.f, l = 0.f;
+    if (e < count)
+#pragma unroll 8
+      for (int k = y; k < splits; k += 16) {
+        const float v = part[(long long)k * count + e];
+        const float s = __fadd_rn(h, v), b = __fsub_rn(s, h);
+        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b)));
+        h = s;
+      }
+    red[y][x] = make_float2(h, l);
+    __syncthreads();
+    if (y == 0 && e < count) {
+      // (an overflowed sum has no low part)
+      double s = 0.0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float2 v = red[j][x];
+        s += v.y == v.y ? (double)v.x + (double)v.y : (double)v.x;
+      }
+      out[e] = (float)s;
+    }
+    __syncthreads();
   }
 }
 
@@ -628,26 +802,77 @@ op_status back_layer(opnet *net, int i, const float *X, const float *dZ, float *
   cudaStream_t st = net->st;
   const long long n = (long long)l.grid * l.grid * l.grid;
   const int K = l.taps * l.cin;
-  long long chunk = 2048;
-  int splits = (int)((n + chunk - 1) / chunk);
-  while ((long long)splits * (K + 1) * l.cout > net->part_floats) {  // cannot happen for the
-    chunk *= 2;                                                        // sizes allocated
+  int splits = 0;
+  if (l.cin % 4 == 0 && l.cout % 4 == 0) {
+    WgradPadArgs w{};
+    w.pad = l.taps == 27 ? 1 : 0;
+    w.X = X;
+    w.dZ = dZ;
+    w.Np = l.grid + 2 * w.pad;
+    w.rows = (int)((long long)w.Np * w.Np * w.Np);
+    if (w.pad) {
+      // dA and dX are free here: the layer's own gradient is in dZ, its data gradient comes after
+      k_wgrad_copy<<<ew_blocks(w.rows * (long long)(l.cin + l.cout) / 4), 256, 0, st>>>(
+          l.grid, l.cin, X, net->dX, l.cout, dZ, net->dA);
+      count_launch();
+      w.X = net->dX;
+      w.dZ = net->dA;
+      w.q0 = w.Np * w.Np + w.Np + 1;
+    }
+    w.q1 = w.rows - w.q0;
+    w.part = net->part;
+    w.cin = l.cin;
+    w.cout = l.cout;
+    w.K = K;
+    w.win = w.pad ? 3 * l.cin : l.cin;
+    // threads: (win / 8) x (cout / 8) per (dz, dy), up to 512; several (dz, dy) while they fit 384
+    w.cothr = (l.cout + 7) / 8;
+    const int kall = (w.win + 7) / 8;
+    w.kblocks = (kall * w.cothr + 511) / 512;
+    w.kthr = (kall + w.kblocks - 1) / w.kblocks;
+    w.kblocks = (kall + w.kthr - 1) / w.kthr;
+    const int per = w.kthr * w.cothr, groups = w.pad ? 9 : 1;
+    w.ng = groups == 9 && per * 9 <= 384 ? 9 : (groups == 9 && per * 3 <= 384 ? 3 : 1);
+    w.apitch = ((kWP + 2 * w.pad) * l.cin + 8 * w.kthr * w.kblocks - w.win + 11) / 4 * 4;
+    w.bpitch = (kWP * l.cout + 19) / 4 * 4;
+    auto bytes = [&](int ng) {
+      return kWStages * (ng * w.apitch + w.bpitch) * (int)sizeof(float);
+    };
+    while (w.ng > 1 && bytes(w.ng) > 200 * 1024) w.ng /= 3;
+    const int threads = (per * w.ng + 31) / 32 * 32, gx = groups / w.ng * w.kblocks;
+    // runs of at most 2048 points, more of them while CTAs are missing and the partials fit
+    const long long points = w.q1 - w.q0, cap = net->part_floats / ((K + 1) * (long long)l.cout);
+    long long want = std::min<long long>((4LL * num_sms() + gx - 1) / gx, points / 96);
+    want = std::max(std::min(want, cap), std::min((points + 2047) / 2048, cap));
+    want = std::max(want, 1LL);
+    w.chunk = (int)(((points + want - 1) / want + kWP - 1) / kWP * kWP);
+    splits = (int)((points + w.chunk - 1) / w.chunk);
+    const int smem = bytes(w.ng);
+    OP_CUDA(cudaFuncSetAttribute(k_wgrad_pad, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_wgrad_pad<<<dim3((unsigned)gx, (unsigned)splits), threads, smem, st>>>(w);
+  } else {
+    long long chunk = 2048;
     splits = (int)((n + chunk - 1) / chunk);
+    while ((long long)splits * (K + 1) * l.cout > net->part_floats) {  // cannot happen for the
+      chunk *= 2;                                                        // sizes allocated
+      splits = (int)((n + chunk - 1) / chunk);
+    }
+    WgradArgs w;
+    w.X = X;
+    w.dZ = dZ;
+    w.part = net->part;
+    w.N = l.grid;
+    w.taps = l.taps;
+    w.cin = l.cin;
+    w.cout = l.cout;
+    w.chunk = chunk;
+    const dim3 grid((unsigned)((K + 1 + 63) / 64), (unsigned)((l.cout + 63) / 64), (unsigned)splits);
+    k_wgrad<<<grid, 256, 0, st>>>(w);
   }
-  WgradArgs w;
-  w.X = X;
-  w.dZ = dZ;
-  w.part = net->part;
-  w.N = l.grid;
-  w.taps = l.taps;
-  w.cin = l.cin;
-  w.cout = l.cout;
-  w.chunk = chunk;
-  const dim3 grid((unsigned)((K + 1 + 63) / 64), (unsigned)((l.cout + 63) / 64), (unsigned)splits);
-  k_wgrad<<<grid, 256, 0, st>>>(w);
   count_launch();
   const long long cnt = (long long)(K + 1) * l.cout;
-  k_reduce_parts<<<ew_blocks(cnt), 256, 0, st>>>(net->part, splits, cnt, net->grad + l.woff);
+  k_reduce_parts<<<(unsigned)std::min<long long>((cnt + 31) / 32, 16LL * num_sms()), 512, 0, st>>>(
+      net->part, splits, cnt, net->grad + l.woff);
   count_launch();
   OP_LAUNCH("k_wgrad");
   if (dX)
@@ -780,7 +1005,7 @@ op_status opnet_create(opnet **out, const opnet_config *cfg) {
       {27, kCin, c0, N},         {27, c0, c0, N},     {27, c0, c1, N / 2}, {27, c1, c1, N / 2},
       {27, c1, c2, N / 4},       {27, c2, c2, N / 4}, {27, c2 + c1, c1, N / 2},
       {27, c1, c1, N / 2},       {27, c1 + c0, c1, N}, {27, c1, c1, N}, {1, c1, p, N}};
-  long long off = 0, max_wf = 0, max_part = 0;
+  long long off = 0, max_wf = 0, max_part = 0, max_xp = 0, max_zp = 0;
   for (int i = 0; i < kLayers; ++i) {
     Layer &l = net->L[i];
     l.taps = shapes[i][0];
@@ -791,9 +1016,11 @@ op_status opnet_create(opnet **out, const opnet_config *cfg) {
     const long long K = (long long)l.taps * l.cin;
     off += K * l.cout + l.cout;
     if (K * l.cout > max_wf) max_wf = K * l.cout;
-    const long long n = (long long)l.grid * l.grid * l.grid;
-    const long long splits = (n + 2047) / 2048;
+    const long long np = (long long)(l.grid + 2) * (l.grid + 2) * (l.grid + 2);
+    const long long splits = (np + 2047) / 2048;  // (of padded points)
     if (splits * (K + 1) * l.cout > max_part) max_part = splits * (K + 1) * l.cout;
+    max_xp = std::max(max_xp, np * l.cin);
+    max_zp = std::max(max_zp, np * l.cout);
   }
   net->nparam = off;
   net->part_floats = max_part;
@@ -820,9 +1047,10 @@ op_status opnet_create(opnet **out, const opnet_config *cfg) {
     if (i != L_OUT) NET_ALLOC(net->A[i], n * l.cout);
     else net->A[i] = nullptr;
   }
-  NET_ALLOC(net->dA, n0 * wide);
+  // (dA and dX also hold the padded copies of the weight gradients)
+  NET_ALLOC(net->dA, std::max(n0 * wide, max_zp));
   NET_ALLOC(net->dZ, n0 * wide);
-  NET_ALLOC(net->dX, n0 * wide);
+  NET_ALLOC(net->dX, std::max(n0 * wide, max_xp));
   NET_ALLOC(net->ge0, n0 * c0);
   NET_ALLOC(net->ge1, n1 * c1);
   NET_ALLOC(net->gsm, n1 * (c1 > c2 ? c1 : c2));
