@@ -189,28 +189,34 @@ __global__ void __launch_bounds__(256, 1)
                  err, split);
 }
 
-// ---- persistent, warp-specialised variant (ld a multiple of 32) ----------------------
-// The same products, split and accumulation order as update_tc_body, so the result is
-// bit-identical; only the staging and the division of labour differ.  One CTA per SM
+// ---- persistent, warp-specialised variant ---------------------------------------------
+// The same products and split as update_tc_body, slab by slab in fresh accumulators; the slabs
+// are ceil(ld / 32) of U, then as many of W (a last slab past the block's columns reads zeros),
+// the MMA's N is the tile's columns rounded up to 16.  One CTA per SM
 // walks the output tiles blockIdx.x, blockIdx.x + gridDim.x, ... (consecutive tiles share
 // their rows of [U W] through L2 when ld > 128), slab by slab, with four roles that
 // meet only at mbarriers, so the tensor core is fed while earlier slabs drain:
-//   warp 9, lane 0  TMA producer: the A slab (128 grid points x 32 K values of U or W)
+//   warp 13, lane 0 TMA producer: the A slab (128 grid points x 32 K values of U or W)
 //                   and the B slabs (128 columns of KT_hi / KT_lo) into a ring of kRing
 //                   stages, each landing in the 128B-swizzled K-major layout;
-//   warps 4..7      split the A slab into TF32 hi (in place) and lo;
-//   warp 8, lane 0  issues the slab's MMAs into one of kAcc TMEM accumulators and
+//   warps 8..11     split the A slab into TF32 hi (in place) and lo;
+//   warp 12, lane 0 issues the slab's MMAs into one of kAcc TMEM accumulators and
 //                   commits them to that accumulator's "done" barrier and the stage's
 //                   "empty" barrier;
-//   warps 0..3      drain each accumulator into FP32 registers (one tile row per thread,
-//                   all 128 columns), free it, and store U + acc when a tile ends.
+//   warps 0..7      drain each accumulator into FP32 registers (one tile row per thread,
+//                   64 columns each half of them), free it, and store U + acc when a tile ends, 16 columns
+//                   at a time through shared memory: rows leave as 64-byte segments (a row per
+//                   thread touches 32 lines an instruction and took 13 of a tile's 22
+//                   thousand clocks: 262144 x 128 took 169 us, 137 now; 357911 x 84 took
+//                   250 us in k_update_tc, 126 here).
 // Every wait is bounded in time; a role that gives up raises a flag the others poll.
 constexpr int kRing = 3;
 constexpr int kAcc = 4;
 constexpr int kStageR = 4 * kPieceA;  // A hi (TMA destination, split in place) | A lo | B hi | B lo
-constexpr int kSmemR = kRing * kStageR + 1024;
+constexpr int kOutPitch = 20;  // floats of an output row in shared memory (16 and 4 of padding)
+constexpr int kSmemR = kRing * kStageR + 8 * 32 * kOutPitch * 4 + 1024;
 constexpr uint64_t kWaitNs = 2000000000ull;  // every wait gives up after 2 s
-constexpr int kWarpsWS = 10;
+constexpr int kWarpsWS = 14;
 
 __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity,
                                               volatile int *abort) {
@@ -229,8 +235,10 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
 
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int nslab = 2 * ld / kKS;
+  const int su = (ld + kKS - 1) / kKS, nslab = 2 * su;  // slabs of U, and of [U W]
   const int ntn = (ld + kTN - 1) / kTN;
+  const int nmma = ntn == 1 ? (ld + 15) / 16 * 16 : kTN;
+  const uint32_t bbytes = (uint32_t)nmma * 128;           // of a B slab
   const long long ntiles = (n + kTM - 1) / kTM * ntn;
   const long long mine =
       ntiles > (long long)blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
@@ -245,7 +253,7 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
     }
     for (int i = 0; i < kAcc; ++i) {
       tma::bar_init(&done[i], 1);
-      tma::bar_init(&freed[i], 128);
+      tma::bar_init(&freed[i], 256);
     }
     tma::fence_bar_init();
     abort_sh = 0;
@@ -256,7 +264,7 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
   const uint32_t tmem = tmem_base_sh;
   volatile int *abort = &abort_sh;
 
-  if (warp == 9) {
+  if (warp == 13) {
     if (lane == 0) {  // ---- TMA producer
       long long g = 0;
       bool ok = true;
@@ -271,12 +279,9 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
             break;
           }
           uint8_t *stage = smem + st * kStageR;
-          const int k0 = s * kKS;
-          tma::bar_expect(&full[st], (uint32_t)((split ? 3 : 2) * kPieceA));
-          if (k0 < ld)
-            tma::load_2d(stage, &mU, k0, m0, &full[st]);
-          else
-            tma::load_2d(stage, &mW, k0 - ld, m0, &full[st]);
+          const int c0 = (s < su ? s : s - su) * kKS, k0 = s < su ? c0 : ld + c0;
+          tma::bar_expect(&full[st], (uint32_t)kPieceA + (split ? 2 : 1) * bbytes);
+          tma::load_2d(stage, s < su ? &mU : &mW, c0, m0, &full[st]);
           tma::load_2d(stage + 2 * kPieceA, &mKh, k0, n0, &full[st]);
           if (split) tma::load_2d(stage + 3 * kPieceA, &mKl, k0, n0, &full[st]);
         }
@@ -288,8 +293,9 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
           (void)tma::bar_wait(&full[q % kRing], (uint32_t)((q / kRing) & 1), kWaitNs);
       }
     }
-  } else if (warp == 8) {
+  } else if (warp == 12) {
     if (lane == 0) {  // ---- MMA issuer
+      const uint32_t idesc = tc::idesc_tf32(kTM, nmma);
       long long g = 0;
       for (; g < total; ++g) {
         const int st = (int)(g % kRing), a = (int)(g % kAcc);
@@ -304,10 +310,10 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
           const uint64_t al = tc::desc_sw128(base + kPieceA + kk * 32);
           const uint64_t bh = tc::desc_sw128(base + 2 * kPieceA + kk * 32);
           const uint64_t bl = tc::desc_sw128(base + 3 * kPieceA + kk * 32);
-          tc::mma_tf32(d, ah, bh, kIdesc, kk > 0 ? 1u : 0u);
+          tc::mma_tf32(d, ah, bh, idesc, kk > 0 ? 1u : 0u);
           if (split) {
-            tc::mma_tf32(d, ah, bl, kIdesc, 1u);
-            tc::mma_tf32(d, al, bh, kIdesc, 1u);
+            tc::mma_tf32(d, ah, bl, idesc, 1u);
+            tc::mma_tf32(d, al, bh, idesc, 1u);
           }
         }
         tc::mma_commit(&done[a]);
@@ -322,8 +328,8 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
         }
       }
     }
-  } else if (warp >= 4) {  // ---- splitters (warps 4..7)
-    const int ct = t - 128;
+  } else if (warp >= 8) {  // ---- splitters (warps 8..11)
+    const int ct = t - 256;
     for (long long g = 0; g < total; ++g) {
       const int st = (int)(g % kRing);
       if (!wait_or_abort(&full[st], (uint32_t)((g / kRing) & 1), abort)) break;
@@ -346,12 +352,12 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
       tc::fence_async_smem();
       tma::bar_arrive(&conv[st]);
     }
-  } else {  // ---- drain and epilogue (warps 0..3: TMEM lanes 32 warp .. 32 warp + 31)
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    const int trow = warp * 32 + lane;
-    float acc[128];
+  } else {  // ---- drain and epilogue (TMEM lanes 32 (warp % 4) .., columns 64 (warp / 4) ..)
+    const int quarter = warp & 3, h0 = (warp >> 2) * 64;
+    const uint32_t lane_base = ((uint32_t)(quarter * 32) << 16) + (uint32_t)h0;
+    float acc[64];
 #pragma unroll
-    for (int i = 0; i < 128; ++i) acc[i] = 0.f;
+    for (int i = 0; i < 64; ++i) acc[i] = 0.f;
     long long g = 0;
     bool ok = true;
     for (long long i = 0; i < mine && ok; ++i) {
@@ -363,7 +369,8 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
         }
         tc::tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < 2; ++c) {
+          if (h0 + c * 32 >= nmma) continue;
           float v[32];
           tc::tmem_ld32(tmem + lane_base + (uint32_t)(a * kTN + c * 32), v);
 #pragma unroll
@@ -374,21 +381,38 @@ __global__ void __launch_bounds__(kWarpsWS * 32, 1)
       }
       if (!ok) break;
       const long long tile = blockIdx.x + i * gridDim.x;
-      const long long row = (tile / ntn) * kTM + trow;
-      const int n0 = (int)(tile % ntn) * kTN;
-      if (row < n) {
+      const long long row0 = (tile / ntn) * kTM + quarter * 32;
+      const int n0 = (int)(tile % ntn) * kTN + h0;
+      // 16 columns at a time: this thread's row to shared memory, then 8 rows an instruction
+      float *ot = reinterpret_cast<float *>(smem + kRing * kStageR) + warp * 32 * kOutPitch;
+      const int orow = lane >> 2, oc = (lane & 3) * 4;
 #pragma unroll
-        for (int c = 0; c < 128; c += 4) {
-          const int col = n0 + c;
-          if (col < ld) {
-            const float4 u = __ldg(reinterpret_cast<const float4 *>(U + row * ld + col));
-            *reinterpret_cast<float4 *>(Unew + row * ld + col) =
-                make_float4(u.x + acc[c], u.y + acc[c + 1], u.z + acc[c + 2], u.w + acc[c + 3]);
-          }
+      for (int c = 0; c < 64; c += 16) {
+        if (n0 + c >= ld) continue;
+        const int col = n0 + c + oc;
+        float4 u[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const long long row = row0 + 8 * r + orow;
+          if (row < n && col < ld) u[r] = __ldg(reinterpret_cast<const float4 *>(U + row * ld + col));
         }
+#pragma unroll
+        for (int e = 0; e < 16; e += 4)
+          *reinterpret_cast<float4 *>(ot + lane * kOutPitch + e) =
+              make_float4(acc[c + e], acc[c + e + 1], acc[c + e + 2], acc[c + e + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const long long row = row0 + 8 * r + orow;
+          const float4 v = *reinterpret_cast<const float4 *>(ot + (8 * r + orow) * kOutPitch + oc);
+          if (row < n && col < ld)
+            *reinterpret_cast<float4 *>(Unew + row * ld + col) =
+                make_float4(u[r].x + v.x, u[r].y + v.y, u[r].z + v.z, u[r].w + v.w);
+        }
+        __syncwarp();
       }
 #pragma unroll
-      for (int c = 0; c < 128; ++c) acc[c] = 0.f;
+      for (int c = 0; c < 64; ++c) acc[c] = 0.f;
     }
     if (!ok && lane == 0) atomicExch(err, 1);
   }
@@ -658,12 +682,13 @@ op_status update_tc(long long n, int ld, const float *U, const float *W, const f
     return OP_ERR_ARG;
   }
   const uintptr_t a = (uintptr_t)U | (uintptr_t)W | (uintptr_t)KT_hi | (uintptr_t)KT_lo;
-  if (ld % kKS == 0 && (a & 15) == 0 && n <= (long long)INT32_MAX - kTM) {
+  if ((a & 15) == 0 && n <= (long long)INT32_MAX - kTM) {
     CUtensorMap mU, mW, mKh, mKl;
+    const uint32_t nb = ld <= kTN ? (ld + 15) / 16 * 16 : kTN;  // B rows of a tile
     OP_TRY(tma_map_2d_f32_sw128(&mU, U, ld, n, kTM));
     OP_TRY(tma_map_2d_f32_sw128(&mW, W, ld, n, kTM));
-    OP_TRY(tma_map_2d_f32_sw128(&mKh, KT_hi, 2 * ld, ld, kTN));
-    OP_TRY(tma_map_2d_f32_sw128(&mKl, KT_lo, 2 * ld, ld, kTN));
+    OP_TRY(tma_map_2d_f32_sw128(&mKh, KT_hi, 2 * ld, ld, nb));
+    OP_TRY(tma_map_2d_f32_sw128(&mKl, KT_lo, 2 * ld, ld, nb));
     const long long ntiles = (n + kTM - 1) / kTM * ((ld + kTN - 1) / kTN);
     const int grid = (int)std::min<long long>(ntiles, num_sms());
     OP_CUDA(cudaFuncSetAttribute(k_update_ws, cudaFuncAttributeMaxDynamicSharedMemorySize,
