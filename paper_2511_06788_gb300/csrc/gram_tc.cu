@@ -8,20 +8,24 @@
 // one-signed error of ~2^-22 in the squared norms of <U,U> and <W,W>).  With
 // split = 0 (the TF32 mixed mode) one MMA per product on tf32(x) is used.
 //
-// Work split: one CTA per (output tile of 128 x 128, chunk of grid points).
-// The contraction index is the grid point (the row of the n x ld blocks), so
-// the operand tiles are transposed while they are staged: each thread loads a
-// 4 x 4 patch (4 grid points x 4 columns) with 16-byte loads, splits it, and
-// writes 16-byte K-chunks into the 128B-swizzled K-major layout the MMA reads.
+// Work split: items of (output tile of 128 x 128, chunk of grid points), one persistent CTA per
+// SM.  The contraction index is the grid point (the row of the n x ld blocks), so the operand
+// tiles are transposed while they are staged: each thread loads a 4 x 4 patch (4 grid points x
+// 4 columns) with 16-byte loads, splits it, and writes 16-byte K-chunks into the 128B-swizzled
+// K-major layout the MMA reads.
 //
-// Accumulation: the tensor core adds into its FP32 accumulator with
-// truncation, so a long run of additions drifts by about (run length) x 2^-24
-// of the accumulated value (for <U,U> = I that is a systematic error of the
-// orthogonality).  Each 32-point slab therefore starts a fresh accumulator (two
-// TMEM accumulators alternate) and, while the tensor core works on slab s, the
-// 8 warps drain slab s-1 into FP32 registers (round-to-nearest additions).
-// The loads run two slabs ahead of the shared-memory stores (one CTA per SM).
-// Chunk partials are written in FP64 and summed over chunks in a fixed order.
+// Accumulation: the tensor core adds into its FP32 accumulator with truncation, so a long run of
+// additions drifts by about (run length) x 2^-24 of the accumulated value (for <U,U> = I that is
+// a systematic error of the orthogonality).  Each 32-point slab therefore starts a fresh
+// accumulator (four TMEM accumulators in turn), which is drained into FP32 registers
+// (round-to-nearest additions); a chunk's FP32 sums are its partial tile, and the partials are
+// added over the chunks in a fixed order as error-free pairs of floats.
+//
+// Roles (k_gram_ws), meeting only at mbarriers: eight warps stage slabs into a ring of three,
+// one thread issues the MMAs (16 a slab, 74 clocks each: the bound), eight warps drain.  With
+// every warp staging, waiting and draining in lockstep (one CTA per item) a slab took 3050
+// clocks, 1190 of them the MMAs.  262144 x 128, C, S and D: 216 us, 301 before (an MMA takes 111
+// clocks beside the staging: both load shared memory).
 #include "common.cuh"
 #include "kernels.cuh"
 #include "tc.cuh"
@@ -36,8 +40,12 @@ constexpr int kReduceSlices = kTM * kTM / 256;
 constexpr int kKS = 32;                       // grid points per slab (one 128-byte K row)
 constexpr int kPiece = kTM * 128;             // bytes of one operand piece (128 rows x 128 B)
 constexpr int kStage = 4 * kPiece;            // A_hi, A_lo, B_hi, B_lo
-constexpr int kStages = 2;
-constexpr int kSmem = kStages * kStage + 1024;  // + alignment slack
+constexpr int kRing = 3;                        // staged slabs
+constexpr int kAcc = 4;                         // TMEM accumulators
+constexpr int kSmem = kRing * kStage + 1024;    // + alignment slack
+constexpr int kStageWarps = 8, kDrainWarps = 8;
+constexpr int kThreadsWs = 32 * (kStageWarps + kDrainWarps + 1);
+constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr uint32_t kIdesc = tc::idesc_tf32(kTM, kTM);
 
 enum { PROD_C = 0, PROD_S = 1, PROD_D = 2 };
@@ -79,6 +87,20 @@ __device__ __forceinline__ void load_patch(const float *__restrict__ X, long lon
   }
 }
 
+// The patch at p (row pitch ld) of a slab that lies inside the chunk; `in`: its columns exist.
+__device__ __forceinline__ void load_patch_in(const float *__restrict__ p, int ld, bool in,
+                                              float (&v)[4][4]) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (in) x = __ldg(reinterpret_cast<const float4 *>(p + r * ld));
+    v[r][0] = x.x;
+    v[r][1] = x.y;
+    v[r][2] = x.z;
+    v[r][3] = x.w;
+  }
+}
+
 // Split the patch and store it transposed: operand row m = 4q + e gets the
 // K-chunk kq = (v[0][e], .., v[3][e]).  Without `split` only tf32(x) is stored.
 __device__ __forceinline__ void store_patch(uint8_t *hi, uint8_t *lo, int q, int kq,
@@ -96,139 +118,256 @@ __device__ __forceinline__ void store_patch(uint8_t *hi, uint8_t *lo, int q, int
   }
 }
 
-// One CTA: output tile (ti, tj) of product `prod` over grid points [r0, r1) of the
-// n x ld blocks U, W, written as a 128 x 128 FP64 partial tile at dst.
-__device__ __forceinline__ void gram_tc_body(long long n, int ld, const float *__restrict__ U,
-                                             const float *__restrict__ W, int prod, int ti,
-                                             int tj, long long r0, long long r1,
-                                             double *__restrict__ dst_tile, int *err, int split,
-                                             bool atomic_out = false) {
+// One item: output tile of A^T B over grid points [r0, r1), rows ca .., columns cb ..; its partial
+// tile is written column by column (element (i, j) at j 128 + i: the drain threads own rows, so a
+// warp writes 128 consecutive bytes) as FP32, or added to an FP64 tile with atomics.
+struct GramTask {
+  const float *A, *B;
+  int ld, ca, cb, nslab;
+  bool same;  // A and B are the same columns: staged once
+  long long r0, r1;
+  float *part;
+  double *sum;  // not null: atomics instead of `part`
+  int *err;
+};
+
+__device__ __forceinline__ void set_task(GramTask *t, long long n, int ld, const float *U,
+                                         const float *W, int prod, int ti, int tj, long long r0,
+                                         long long r1) {
+  t->A = (prod == PROD_D) ? U : W;
+  t->B = (prod == PROD_S) ? W : U;
+  t->ld = ld;
+  t->ca = ti * kTM;
+  t->cb = tj * kTM;
+  t->same = (t->A == t->B) && ti == tj;
+  t->r0 = r0;
+  t->r1 = r1 < n ? r1 : n;
+  t->nslab = t->r1 > r0 ? (int)((t->r1 - r0 + kKS - 1) / kKS) : 0;
+}
+
+// Items of one problem: split s of job j is item s njobs + j.
+struct GramSrc {
+  long long n, rps, items;
+  int ld, mask, nt, njobs;
+  const float *U, *W;
+  float *part;
+  double *sum;
+  int *err;
+  __device__ __forceinline__ bool get(long long i, GramTask *t) const {
+    const int job = (int)(i % njobs);
+    const long long r0 = i / njobs * rps;
+    int prod, ti, tj;
+    decode_job(job, mask, nt, &prod, &ti, &tj);
+    set_task(t, n, ld, U, W, prod, ti, tj, r0, r0 + rps);
+    t->part = part + i * (kTM * kTM);
+    t->sum = sum ? sum + (long long)job * (kTM * kTM) : nullptr;
+    t->err = err;
+    return true;
+  }
+};
+// Items of a batch (problem, job, chunk), all three products; a frozen problem's are skipped.
+struct GramBatchSrc {
+  long long items;
+  const BatchProb *B;
+  const GramItem *list;
+  int parity;
+  __device__ __forceinline__ bool get(long long i, GramTask *t) const {
+    const GramItem it = list[i];
+    const BatchProb &pb = B[it.prob];
+    if (*pb.frozen) return false;
+    int prod, ti, tj;
+    decode_job(it.job, 7, (pb.ld + kTM - 1) / kTM, &prod, &ti, &tj);
+    set_task(t, pb.g.n, pb.ld, pb.U[parity], pb.W, prod, ti, tj, it.r0, it.r1);
+    t->part = (float *)pb.gram_part + ((long long)it.split * pb.gram_jobs + it.job) * (kTM * kTM);
+    t->sum = nullptr;
+    t->err = pb.err;
+    return true;
+  }
+};
+
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
+  int ok = 0;
+  if ((threadIdx.x & 31) == 0) ok = tc::wait_or_abort(bar, parity, abort, kWaitNs) ? 1 : 0;
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+template <typename Src>
+__global__ void __launch_bounds__(kThreadsWs, 1) k_gram_ws(const Src src, int split) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t mbar[2];  // one per TMEM accumulator
-  __shared__ uint32_t tmem_base_sh;
+  __shared__ uint64_t full[kRing], empty[kRing], done[kAcc], freed[kAcc];
+  __shared__ uint32_t tmem_sh;
   __shared__ int abort_sh;
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-
-  const float *A = (prod == PROD_D) ? U : W;
-  const float *B = (prod == PROD_S) ? W : U;
-  const int ca = ti * kTM, cb = tj * kTM;
-  // diagonal tiles of S = W^T W and D = U^T U: A and B are the same data, staged once
-  // (the B descriptors point at A's pieces; the MMAs and their order are unchanged)
-  const bool same = (A == B) && (ca == cb);
-  if (r1 > n) r1 = n;
-  const int nslab = r1 > r0 ? (int)((r1 - r0 + kKS - 1) / kKS) : 0;
-
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int kq = t & 7, q = t >> 3;        // staging patch: points 4kq.., columns 4q..
-  const int row = (warp & 3) * 32 + lane;  // drain: accumulator row (TMEM lane)
-  const int half = warp >> 2;              // drain: columns 64 half .. 64 half + 63
-
-  if (warp == 0) tc::tmem_alloc(&tmem_base_sh, 2 * kTM);
+  constexpr int kMma = kStageWarps + kDrainWarps;
+  if (warp == kMma) tc::tmem_alloc(&tmem_sh, kAcc * kTM);
   if (t == 0) {
-    tc::mbar_init(&mbar[0], 1);
-    tc::mbar_init(&mbar[1], 1);
+    for (int i = 0; i < kRing; ++i) {
+      tc::mbar_init(&full[i], kStageWarps);
+      tc::mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < kAcc; ++i) {
+      tc::mbar_init(&done[i], 1);
+      tc::mbar_init(&freed[i], kDrainWarps);
+    }
     tc::fence_mbar_init();
     abort_sh = 0;
   }
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
-  const uint32_t tmem = tmem_base_sh;
-  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+  const uint32_t tmem = tmem_sh;
+  volatile int *abort = &abort_sh;
+  int *err = nullptr;  // of the last item this thread saw
 
-  float acc[64];
-#pragma unroll
-  for (int i = 0; i < 64; ++i) acc[i] = 0.f;
-
-  // drain the accumulator of slab s (called after the MMAs of slab s+1 were issued)
-  auto drain = [&](int s) -> bool {
-    const int a = s & 1;
-    if (t == 0 && !tc::mbar_wait(&mbar[a], (uint32_t)((s >> 1) & 1))) abort_sh = 1;
-    __syncthreads();
-    if (abort_sh) return false;
-    tc::tc_fence_after();
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float v[32];
-      tc::tmem_ld32(tmem + lane_base + (uint32_t)(a * kTM + half * 64 + c * 32), v);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) acc[c * 32 + i] += v[i];
-    }
-    tc::tc_fence_before();
-    return true;
-  };
-
-  // stage slab s from the register buffer (va, vb), refill the buffer with slab s + 2,
-  // issue the MMAs of slab s and drain slab s - 1
-  auto step = [&](int s, float (&va)[4][4], float (&vb)[4][4]) -> bool {
-    const int st = s & 1;
-    uint8_t *stage = smem + st * kStage;
-    // stage st was read by the MMAs of slab s-2, which the drain of slab s-2 waited for
-    store_patch(stage, stage + kPiece, q, kq, va, split != 0);
-    if (!same) store_patch(stage + 2 * kPiece, stage + 3 * kPiece, q, kq, vb, split != 0);
-    if (s + 2 < nslab) {
-      const long long r = r0 + (long long)(s + 2) * kKS + 4 * kq;
-      load_patch(A, r, r1, ca + 4 * q, ld, va);
-      if (!same) load_patch(B, r, r1, cb + 4 * q, ld, vb);
-    }
-    tc::fence_async_smem();
-    tc::tc_fence_before();
-    __syncthreads();
-    if (t == 0) {
-      tc::tc_fence_after();
-      const uint32_t base = tc::smem_u32(stage);
-      const uint32_t bbase = same ? base : base + 2 * kPiece;
-      const uint32_t d = tmem + (uint32_t)(st * kTM);
-#pragma unroll
-      for (int kk = 0; kk < kKS / 8; ++kk) {
-        const uint64_t ah = tc::desc_sw128(base + kk * 32);
-        const uint64_t al = tc::desc_sw128(base + kPiece + kk * 32);
-        const uint64_t bh = tc::desc_sw128(bbase + kk * 32);
-        const uint64_t bl = tc::desc_sw128(bbase + kPiece + kk * 32);
-        tc::mma_tf32(d, ah, bh, kIdesc, kk > 0 ? 1u : 0u);
-        if (split) {
-          tc::mma_tf32(d, ah, bl, kIdesc, 1u);
-          tc::mma_tf32(d, al, bh, kIdesc, 1u);
-          tc::mma_tf32(d, al, bl, kIdesc, 1u);
+  if (warp < kStageWarps) {
+    // ---- staging: points 4 kq .. of a slab, columns 4 q .. of the tile
+    const int kq = t & 7, q = t >> 3;
+    uint32_t slot = 0, phase = 1, g = 0;  // phase of the slot's last release
+    bool ok = true;
+    for (long long i = blockIdx.x; i < src.items && ok; i += gridDim.x) {
+      GramTask k;
+      if (!src.get(i, &k)) continue;
+      err = k.err;
+      float va[4][4], vb[4][4];
+      if (k.nslab > 0) {
+        load_patch(k.A, k.r0 + 4 * kq, k.r1, k.ca + 4 * q, k.ld, va);
+        if (!k.same) load_patch(k.B, k.r0 + 4 * kq, k.r1, k.cb + 4 * q, k.ld, vb);
+      }
+      // lines of slab kAhead on (row t / 4, 32 columns t % 4): A by the first 128 threads, B by the
+      // others; the loads of a slab then come from L2
+      constexpr int kAhead = 3;
+      const int pcol = (t < 128 ? k.ca : k.cb) + 32 * (t & 3), prow = (t & 127) >> 2;
+      const bool pin = pcol < k.ld && (t < 128 || !k.same);
+      const float *pf = (t < 128 ? k.A : k.B) + (k.r0 + kAhead * kKS + prow) * k.ld + pcol;
+      const int pslabs = pin ? (int)((k.r1 - k.r0 - prow + kKS - 1) / kKS) - kAhead : 0;
+      // this thread's patches of the next slab
+      const bool ina = k.ca + 4 * q < k.ld, inb = k.cb + 4 * q < k.ld;
+      const float *pa = k.A + (k.r0 + kKS + 4 * kq) * k.ld + k.ca + 4 * q;
+      const float *pb = k.B + (k.r0 + kKS + 4 * kq) * k.ld + k.cb + 4 * q;
+      const int inside = (int)((k.r1 - k.r0) / kKS), step = kKS * k.ld;
+      for (int s = 0; s < k.nslab; ++s, ++g) {
+        if (g >= kRing && !warp_wait(&empty[slot], phase, abort)) {
+          ok = false;
+          break;
+        }
+        uint8_t *stage = smem + slot * kStage;
+        store_patch(stage, stage + kPiece, q, kq, va, split != 0);
+        if (!k.same) store_patch(stage + 2 * kPiece, stage + 3 * kPiece, q, kq, vb, split != 0);
+        // (the loads of the next slab come after the fence, which waits for every access before it)
+        tc::fence_async_smem();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&full[slot]);
+        if (s + 1 < inside) {
+          load_patch_in(pa, k.ld, ina, va);
+          if (!k.same) load_patch_in(pb, k.ld, inb, vb);
+        } else if (s + 1 < k.nslab) {  // the chunk's ragged last slab
+          const long long r = k.r0 + (long long)(s + 1) * kKS + 4 * kq;
+          load_patch(k.A, r, k.r1, k.ca + 4 * q, k.ld, va);
+          if (!k.same) load_patch(k.B, r, k.r1, k.cb + 4 * q, k.ld, vb);
+        }
+        if (s < pslabs) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf) : "memory");
+        pa += step;
+        pb += step;
+        pf += step;
+        if (++slot == kRing) {
+          slot = 0;
+          phase ^= 1;
         }
       }
-      tc::mma_commit(&mbar[st]);
     }
-    return s >= 1 ? drain(s - 1) : true;
-  };
-
-  float va0[4][4], vb0[4][4], va1[4][4], vb1[4][4];
-  if (nslab > 0) {
-    load_patch(A, r0 + 4 * kq, r1, ca + 4 * q, ld, va0);
-    if (!same) load_patch(B, r0 + 4 * kq, r1, cb + 4 * q, ld, vb0);
-  }
-  if (nslab > 1) {
-    load_patch(A, r0 + kKS + 4 * kq, r1, ca + 4 * q, ld, va1);
-    if (!same) load_patch(B, r0 + kKS + 4 * kq, r1, cb + 4 * q, ld, vb1);
-  }
-  bool ok = true;
-  for (int s = 0; s < nslab && ok; s += 2) {
-    ok = step(s, va0, vb0);
-    if (ok && s + 1 < nslab) ok = step(s + 1, va1, vb1);
-  }
-  if (ok && nslab > 0) ok = drain(nslab - 1);
-  __syncthreads();
-  if (!ok || abort_sh) {
-    if (t == 0) atomicExch(err, 1);
+  } else if (warp == kMma) {
+    if (lane == 0) {
+      uint32_t slot = 0, phase = 0, g = 0;
+      bool ok = true;
+      for (long long i = blockIdx.x; i < src.items && ok; i += gridDim.x) {
+        GramTask k;
+        if (!src.get(i, &k)) continue;
+        err = k.err;
+        for (int s = 0; s < k.nslab; ++s, ++g) {
+          const uint32_t a = g % kAcc;
+          if ((g >= kAcc && !tc::wait_or_abort(&freed[a], (g / kAcc - 1) & 1, abort, kWaitNs)) ||
+              !tc::wait_or_abort(&full[slot], phase, abort, kWaitNs)) {
+            ok = false;
+            break;
+          }
+          tc::tc_fence_after();
+          const uint32_t base = tc::smem_u32(smem + slot * kStage);
+          const uint32_t bbase = k.same ? base : base + 2 * kPiece;
+          const uint32_t d = tmem + a * kTM;
+#pragma unroll
+          for (int kk = 0; kk < kKS / 8; ++kk) {
+            const uint64_t ah = tc::desc_sw128(base + kk * 32);
+            const uint64_t al = tc::desc_sw128(base + kPiece + kk * 32);
+            const uint64_t bh = tc::desc_sw128(bbase + kk * 32);
+            const uint64_t bl = tc::desc_sw128(bbase + kPiece + kk * 32);
+            tc::mma_tf32(d, ah, bh, kIdesc, kk > 0 ? 1u : 0u);
+            if (split) {
+              tc::mma_tf32(d, ah, bl, kIdesc, 1u);
+              tc::mma_tf32(d, al, bh, kIdesc, 1u);
+              tc::mma_tf32(d, al, bl, kIdesc, 1u);
+            }
+          }
+          tc::mma_commit(&empty[slot]);
+          tc::mma_commit(&done[a]);
+          if (++slot == kRing) {
+            slot = 0;
+            phase ^= 1;
+          }
+        }
+      }
+      // MMAs issued but not drained finish before the TMEM is freed
+      if (!ok && g > 0) (void)tc::mbar_wait(&done[(g - 1) % kAcc], ((g - 1) / kAcc) & 1);
+    }
   } else {
-    double *dst = dst_tile + row * kTM + half * 64;
-    if (atomic_out) {
-      // the chunk partials of a tile meet in one FP64 tile (fixed-scratch entry point)
+    // ---- drain: accumulator row (TMEM lane) 32 (warp % 4) + lane, columns 64 half ..
+    const int quarter = warp & 3, half = (warp - kStageWarps) >> 2, row = quarter * 32 + lane;
+    const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 64);
+    uint32_t g = 0;
+    bool ok = true;
+    for (long long i = blockIdx.x; i < src.items && ok; i += gridDim.x) {
+      GramTask k;
+      if (!src.get(i, &k)) continue;
+      err = k.err;
+      float acc[64];
 #pragma unroll
-      for (int i = 0; i < 64; ++i) atomicAdd(dst + i, (double)acc[i]);
-    } else {
+      for (int e = 0; e < 64; ++e) acc[e] = 0.f;
+      for (int s = 0; s < k.nslab; ++s, ++g) {
+        const uint32_t a = g % kAcc;
+        if (!warp_wait(&done[a], (g / kAcc) & 1, abort)) {
+          ok = false;
+          break;
+        }
+        tc::tc_fence_after();
 #pragma unroll
-      for (int i = 0; i < 64; ++i) dst[i] = (double)acc[i];
+        for (int c = 0; c < 4; ++c) {
+          float v[16];
+          tc::tmem_ld16(tb + a * kTM + (uint32_t)(c * 16), v);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) acc[c * 16 + e] += v[e];
+        }
+        tc::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&freed[a]);
+      }
+      if (!ok) break;
+      const int at = half * 64 * kTM + row;
+      if (k.sum) {
+#pragma unroll
+        for (int e = 0; e < 64; ++e) atomicAdd(k.sum + at + e * kTM, (double)acc[e]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 64; ++e) k.part[at + e * kTM] = acc[e];
+      }
     }
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 2 * kTM);
+  if (warp == kMma) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, kAcc * kTM);
+  }
+  if (lane == 0 && abort_sh && err) atomicExch(err, 1);
 }
 
 // ---- BF16 variants -------------------------------------------------------------------
@@ -278,7 +417,7 @@ __device__ __forceinline__ void store_patch8(uint8_t *piece0, int q, int kq, con
 __device__ __forceinline__ void gram_bf16_body(long long n, int ld, const float *__restrict__ U,
                                                const float *__restrict__ W, int prod, int ti,
                                                int tj, long long r0, long long r1,
-                                               double *__restrict__ dst_tile, int *err,
+                                               float *__restrict__ dst_tile, int *err,
                                                bool three) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t mbar[2];
@@ -383,9 +522,9 @@ __device__ __forceinline__ void gram_bf16_body(long long n, int ld, const float 
   if (!ok || abort_sh) {
     if (t == 0) atomicExch(err, 1);
   } else {
-    double *dst = dst_tile + row * kTM + half * 64;
+    float *dst = dst_tile + half * 64 * kTM + row;  // column by column
 #pragma unroll
-    for (int i = 0; i < 64; ++i) dst[i] = (double)acc[i];
+    for (int i = 0; i < 64; ++i) dst[i * kTM] = acc[i];
   }
   tc::tc_fence_before();
   __syncthreads();
@@ -394,7 +533,7 @@ __device__ __forceinline__ void gram_bf16_body(long long n, int ld, const float 
 
 __global__ void __launch_bounds__(256, 1)
     k_gram_bf16(long long n, int ld, const float *__restrict__ U, const float *__restrict__ W,
-                int mask, int nt, int njobs, long long rows_per_split, double *__restrict__ part,
+                int mask, int nt, int njobs, long long rows_per_split, float *__restrict__ part,
                 int *err, int three) {
   int prod, ti, tj;
   decode_job(blockIdx.x, mask, nt, &prod, &ti, &tj);
@@ -404,72 +543,70 @@ __global__ void __launch_bounds__(256, 1)
                  three != 0);
 }
 
-__global__ void __launch_bounds__(256, 1)
-    k_gram_tc(long long n, int ld, const float *__restrict__ U, const float *__restrict__ W,
-              int mask, int nt, int njobs, long long rows_per_split, double *__restrict__ part,
-              int *err, int split, int atomic_out) {
-  int prod, ti, tj;
-  decode_job(blockIdx.x, mask, nt, &prod, &ti, &tj);
-  const long long r0 = (long long)blockIdx.y * rows_per_split;
-  const long long slot = atomic_out ? 0 : (long long)blockIdx.y;
-  gram_tc_body(n, ld, U, W, prod, ti, tj, r0, r0 + rows_per_split,
-               part + (slot * njobs + blockIdx.x) * (kTM * kTM), err, split, atomic_out != 0);
+// Sum over the splits of element e of a partial tile, in order: FP32 partials as an error-free
+// pair of floats (two-sum; the FP64 pipe would take longer than reading them), or FP64.
+__device__ __forceinline__ double sum_splits(const float *p, long long stride, int nsplit) {
+  float h = 0.f, l = 0.f;
+#pragma unroll 8
+  for (int sp = 0; sp < nsplit; ++sp) {
+    const float v = p[sp * stride], s = __fadd_rn(h, v), b = __fsub_rn(s, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b)));
+    h = s;
+  }
+  return l == l ? (double)h + (double)l : (double)h;  // (an overflowed sum has no low part)
+}
+__device__ __forceinline__ double sum_splits(const double *p, long long stride, int nsplit) {
+  double s = 0.0;
+  for (int sp = 0; sp < nsplit; ++sp) s += p[sp * stride];
+  return s;
 }
 
-// Batched: one CTA per GramItem (problem, job, grid-point chunk); all three products.
-__global__ void __launch_bounds__(256, 1)
-    k_b_gram_tc(const BatchProb *__restrict__ Bp, const GramItem *__restrict__ items, int parity) {
-  const GramItem it = items[blockIdx.x];
-  const BatchProb &pb = Bp[it.prob];
-  if (*pb.frozen) return;
-  const int nt = (pb.ld + kTM - 1) / kTM;
-  int prod, ti, tj;
-  decode_job(it.job, 7, nt, &prod, &ti, &tj);
-  gram_tc_body(pb.g.n, pb.ld, pb.U[parity], pb.W, prod, ti, tj, it.r0, it.r1,
-               pb.gram_part + ((long long)it.split * pb.gram_jobs + it.job) * (kTM * kTM), pb.err,
-               1);
+// out(i, j) = the summed tile element, zero outside p x p, both triangles of S and D.
+template <typename P>
+__device__ __forceinline__ void reduce_tile(int prod, int ti, int tj, int slice, int slices,
+                                            const P *part, long long stride, int nsplit, int p,
+                                            int ld, double *out) {
+  for (int e = slice * blockDim.x + threadIdx.x; e < kTM * kTM; e += slices * blockDim.x) {
+    const int i = ti * kTM + e % kTM, j = tj * kTM + e / kTM;
+    if (i >= ld || j >= ld) continue;
+    const double s = sum_splits(part + e, stride, nsplit);
+    const double v = (i < p && j < p) ? s : 0.0;
+    out[(long long)i * ld + j] = v;
+    if (prod != PROD_C && ti != tj) out[(long long)j * ld + i] = v;
+  }
 }
 
 // Batched reduce: grid (jobs, problems, element slices).
 __global__ void k_b_gram_tc_reduce(const BatchProb *__restrict__ Bp) {
   const BatchProb &pb = Bp[blockIdx.y];
   if (*pb.frozen || (int)blockIdx.x >= pb.gram_jobs) return;
-  const int ld = pb.ld, p = pb.p;
-  const int nt = (ld + kTM - 1) / kTM;
   int prod, ti, tj;
-  decode_job(blockIdx.x, 7, nt, &prod, &ti, &tj);
-  double *out = prod == PROD_C ? pb.C : (prod == PROD_S ? pb.S : pb.D);
-  for (int e = blockIdx.z * blockDim.x + threadIdx.x; e < kTM * kTM;
-       e += gridDim.z * blockDim.x) {
-    const int i = ti * kTM + e / kTM, j = tj * kTM + e % kTM;
-    if (i >= ld || j >= ld) continue;
-    double s = 0.0;
-#pragma unroll 8
-    for (int sp = 0; sp < pb.n_gram_splits; ++sp)
-      s += pb.gram_part[((long long)sp * pb.gram_jobs + blockIdx.x) * (kTM * kTM) + e];
-    const double v = (i < p && j < p) ? s : 0.0;
-    out[(long long)i * ld + j] = v;
-    if (prod != PROD_C && ti != tj) out[(long long)j * ld + i] = v;
-  }
+  decode_job(blockIdx.x, 7, (pb.ld + kTM - 1) / kTM, &prod, &ti, &tj);
+  reduce_tile(prod, ti, tj, blockIdx.z, gridDim.z,
+              (const float *)pb.gram_part + (long long)blockIdx.x * (kTM * kTM),
+              (long long)pb.gram_jobs * (kTM * kTM), pb.n_gram_splits, pb.p, pb.ld,
+              prod == PROD_C ? pb.C : (prod == PROD_S ? pb.S : pb.D));
 }
 
+template <typename P>
 __global__ void k_gram_tc_reduce(int mask, int nt, int njobs, int nsplit,
-                                 const double *__restrict__ part, int p, int ld, double *C,
-                                 double *S, double *D) {
+                                 const P *__restrict__ part, int p, int ld, double *C, double *S,
+                                 double *D) {
   int prod, ti, tj;
   decode_job(blockIdx.x, mask, nt, &prod, &ti, &tj);
-  double *out = prod == PROD_C ? C : (prod == PROD_S ? S : D);
-  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < kTM * kTM; e += gridDim.y * blockDim.x) {
-    const int i = ti * kTM + e / kTM, j = tj * kTM + e % kTM;
-    if (i >= ld || j >= ld) continue;
-    double s = 0.0;
-#pragma unroll 8
-    for (int sp = 0; sp < nsplit; ++sp)
-      s += part[((long long)sp * njobs + blockIdx.x) * (kTM * kTM) + e];
-    const double v = (i < p && j < p) ? s : 0.0;
-    out[(long long)i * ld + j] = v;
-    if (prod != PROD_C && ti != tj) out[(long long)j * ld + i] = v;
-  }
+  reduce_tile(prod, ti, tj, blockIdx.y, gridDim.y, part + (long long)blockIdx.x * (kTM * kTM),
+              (long long)njobs * (kTM * kTM), nsplit, p, ld,
+              prod == PROD_C ? C : (prod == PROD_S ? S : D));
+}
+
+template <typename Src> op_status launch_gram_ws(const Src &src, int split, cudaStream_t st) {
+  OP_CUDA(cudaFuncSetAttribute(k_gram_ws<Src>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+  const long long grid = src.items < num_sms() ? src.items : num_sms();
+  if (grid < 1) return OP_OK;
+  k_gram_ws<Src><<<(unsigned)grid, kThreadsWs, kSmem, st>>>(src, split);
+  count_launch();
+  OP_LAUNCH("k_gram_ws");
+  return OP_OK;
 }
 
 int tc_jobs(int nt, int mask) {
@@ -516,7 +653,7 @@ op_status gram_tc(long long n, int p, int ld, const float *U, const float *W, do
     set_error("gram_tc: workspace too small (%zu < %zu)", ws_bytes, need);
     return OP_ERR_ARG;
   }
-  double *part = (double *)ws;
+  float *part = (float *)ws;
   if (split >= 2) {  // BF16: 2 three pieces, 3 one piece
     OP_CUDA(cudaFuncSetAttribute(k_gram_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kSmemB16));
@@ -525,13 +662,10 @@ op_status gram_tc(long long n, int p, int ld, const float *U, const float *W, do
     count_launch();
     OP_LAUNCH("k_gram_bf16");
   } else {
-    OP_CUDA(cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-    k_gram_tc<<<dim3(nj, nsplit), 256, kSmem, st>>>(n, ld, U, W, mask, nt, nj, rps, part, err,
-                                                     split, 0);
-    count_launch();
-    OP_LAUNCH("k_gram_tc");
+    OP_TRY(launch_gram_ws(GramSrc{n, rps, (long long)nj * nsplit, ld, mask, nt, nj, U, W, part,
+                                  nullptr, err}, split, st));
   }
-  k_gram_tc_reduce<<<dim3(nj, kReduceSlices), 256, 0, st>>>(mask, nt, nj, nsplit, part, p, ld,
+  k_gram_tc_reduce<float><<<dim3(nj, kReduceSlices), 256, 0, st>>>(mask, nt, nj, nsplit, part, p, ld,
                                                              C, S, D);
   count_launch();
   OP_LAUNCH("k_gram_tc_reduce");
@@ -563,12 +697,9 @@ op_status gram_tc_fixed_scratch(long long n, int p, int ld, const float *U, cons
   long long rps;
   plan_tc(n, nj, &nsplit, &rps);
   OP_CUDA(cudaMemsetAsync(part, 0, (size_t)nj * tile_bytes, st));
-  OP_CUDA(cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-  k_gram_tc<<<dim3(nj, nsplit), 256, kSmem, st>>>(n, ld, U, W, mask, nt, nj, rps, (double *)part,
-                                                   err, 1, 1);
-  count_launch();
-  OP_LAUNCH("k_gram_tc");
-  k_gram_tc_reduce<<<dim3(nj, kReduceSlices), 256, 0, st>>>(mask, nt, nj, 1, (const double *)part,
+  OP_TRY(launch_gram_ws(GramSrc{n, rps, (long long)nj * nsplit, ld, mask, nt, nj, U, W, nullptr,
+                                (double *)part, err}, 1, st));
+  k_gram_tc_reduce<double><<<dim3(nj, kReduceSlices), 256, 0, st>>>(mask, nt, nj, 1, (const double *)part,
                                                              p, ld, C, S, D);
   count_launch();
   OP_LAUNCH("k_gram_tc_reduce");
@@ -577,10 +708,7 @@ op_status gram_tc_fixed_scratch(long long n, int p, int ld, const float *U, cons
 
 op_status launch_b_gram(const BatchProb *B, const GramItem *items, int nitems, int nprob,
                         int parity, cudaStream_t st) {
-  OP_CUDA(cudaFuncSetAttribute(k_b_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-  k_b_gram_tc<<<nitems, 256, kSmem, st>>>(B, items, parity);
-  count_launch();
-  OP_LAUNCH("k_b_gram_tc");
+  OP_TRY(launch_gram_ws(GramBatchSrc{nitems, B, items, parity}, 1, st));
   // at most 3 * 8 * 8 + ... jobs for ld <= 1024: grid x covers the largest job count
   k_b_gram_tc_reduce<<<dim3(tc_jobs(8, 7), nprob, 4), 256, 0, st>>>(B);
   count_launch();
