@@ -483,14 +483,15 @@ __device__ __forceinline__ void gram_bf16_body(long long n, int ld, const float 
     // stage st was read by the MMAs of slab s-2, which the drain of slab s-2 waited for
     store_patch8(stage, q, kq, va, three);
     if (!same) store_patch8(stage + 3 * kPiece, q, kq, vb, three);
+    tc::fence_async_smem();
+    tc::tc_fence_before();
+    __syncthreads();
+    // (after the fence, which waits for every access before it)
     if (s + 1 < nslab) {
       const long long r = r0 + (long long)(s + 1) * kKSb + 8 * kq;
       load_patch8(A, r, r1, ca + 4 * q, ld, va);
       if (!same) load_patch8(B, r, r1, cb + 4 * q, ld, vb);
     }
-    tc::fence_async_smem();
-    tc::tc_fence_before();
-    __syncthreads();
     if (t == 0) {
       tc::tc_fence_after();
       const uint32_t base = tc::smem_u32(stage);

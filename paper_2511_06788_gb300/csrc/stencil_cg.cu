@@ -450,80 +450,107 @@ __global__ void __launch_bounds__(256, 4) k_cg_wr(Geom g, const T *__restrict__ 
   block_colsum<T, NC>(acc, ld, part);
 }
 
-// ---- finalisers: one warp per column, lanes stride over the CTA partials ----------
-__device__ __forceinline__ double warp_sum_blocks(const double *part, int nblk, int stride, int e) {
-  const int lane = threadIdx.x & 31;
-  double s = 0.0;
-  for (int b = lane; b < nblk; b += 32) s += part[(long long)b * stride + e];
+// ---- finalisers over the CTA partials of a row kernel: blocks of 256 threads take four columns,
+// 64 interleaved sums each (rows of four consecutive doubles: whole sectors), joined by shuffles
+// and one pass through shared memory, in a fixed order.  A warp a column read one double per
+// sector and left the sums to a few SMs' FP64 pipes (two additions a clock each): k_cg_fin_beta of
+// 608 x 104 x 2 partials from 13.9 to 8.6 us (cold).
+constexpr int kFinCols = 4;
+template <int NC>
+__device__ __forceinline__ bool fin_sums(const double *__restrict__ part, int nblk, int stride,
+                                         const int (&off)[NC], double (&s)[NC]) {
+  __shared__ double red[NC][8][kFinCols];
+  const int c = threadIdx.x & (kFinCols - 1), g = threadIdx.x / kFinCols;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
+  for (int q = 0; q < NC; ++q) s[q] = 0.0;
+#pragma unroll 4
+  for (int b = g; b < nblk; b += 256 / kFinCols)
+#pragma unroll
+    for (int q = 0; q < NC; ++q) s[q] += part[(long long)b * stride + off[q] + c];
+#pragma unroll
+  for (int o = kFinCols; o < 32; o <<= 1)
+#pragma unroll
+    for (int q = 0; q < NC; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+  if ((threadIdx.x & 31) < kFinCols)
+#pragma unroll
+    for (int q = 0; q < NC; ++q) red[q][threadIdx.x >> 5][c] = s[q];
+  __syncthreads();
+  if (threadIdx.x >= kFinCols) return false;
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    s[q] = red[q][0][c];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s[q] += red[q][w][c];
+  }
+  return true;  // this thread holds the sums of column 4 blockIdx.x + threadIdx.x
 }
 
 // state rows: 0 rho (r.r, or r.z with the Jacobi preconditioner), 1 target, 2 alpha,
 // 3 beta, 4 ||b||^2.  ncomp = 2: partials (r.r, b.b); 3: (r.z, b.b, r.r).  A column
 // stays active while its unpreconditioned ||r||^2 is above rtol^2 ||b||^2.
-__global__ void k_cg_fin_init(const double *part, int nblk, int ncomp, int ld, int p,
-                              double rtol2, double *state, int *active, int *ctl) {
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= ld) return;
-  const double rho = warp_sum_blocks(part, nblk, ncomp * ld, j);
-  const double bb = warp_sum_blocks(part, nblk, ncomp * ld, ld + j);
-  const double rr = ncomp == 3 ? warp_sum_blocks(part, nblk, ncomp * ld, 2 * ld + j) : rho;
-  if ((threadIdx.x & 31) == 0) {
-    state[0 * ld + j] = rho;
-    state[1 * ld + j] = rtol2 * bb;
-    state[2 * ld + j] = 0.0;
-    state[3 * ld + j] = 0.0;
-    state[4 * ld + j] = bb;
-    const int a = (j < p) && (rr > rtol2 * bb) && (bb > 0.0);
-    active[j] = a;
-    if (a) atomicAdd(&ctl[1], 1);
-  }
+__global__ void __launch_bounds__(256)
+    k_cg_fin_init(const double *part, int nblk, int ncomp, int ld, int p, double rtol2,
+                  double *state, int *active, int *ctl) {
+  const int j0 = blockIdx.x * kFinCols, j = j0 + (int)threadIdx.x;
+  const int off[3] = {j0, ld + j0, ncomp == 3 ? 2 * ld + j0 : j0};
+  double s[3];
+  if (!fin_sums<3>(part, nblk, ncomp * ld, off, s)) return;
+  const double rho = s[0], bb = s[1], rr = s[2];
+  state[0 * ld + j] = rho;
+  state[1 * ld + j] = rtol2 * bb;
+  state[2 * ld + j] = 0.0;
+  state[3 * ld + j] = 0.0;
+  state[4 * ld + j] = bb;
+  const int a = (j < p) && (rr > rtol2 * bb) && (bb > 0.0);
+  active[j] = a;
+  if (a) atomicAdd(&ctl[1], 1);
 }
 
-__global__ void k_cg_fin_alpha(const double *part, int nblk, int ld, double *state,
-                               const int *active, const int *nact_prev, int *nact_next) {
+__global__ void __launch_bounds__(256)
+    k_cg_fin_alpha(const double *part, int nblk, int ld, double *state, const int *active,
+                   const int *nact_prev, int *nact_next) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *nact_next = 0;
   if (*nact_prev == 0) return;
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= ld) return;
-  const double pq = warp_sum_blocks(part, nblk, ld, j);
-  if ((threadIdx.x & 31) == 0) {
-    const double rr = state[j];
-    state[2 * ld + j] = (active[j] && pq > 0.0) ? rr / pq : 0.0;
-  }
+  const int j0 = blockIdx.x * kFinCols, j = j0 + (int)threadIdx.x;
+  const int off[1] = {j0};
+  double s[1];
+  if (!fin_sums<1>(part, nblk, ld, off, s)) return;
+  const double pq = s[0], rr = state[j];
+  state[2 * ld + j] = (active[j] && pq > 0.0) ? rr / pq : 0.0;
 }
 
 // ncomp = 1: partials (r.r); 2: (r.z, r.r) with the Jacobi preconditioner.
-__global__ void k_cg_fin_beta(const double *part, int nblk, int ncomp, int ld, double *state,
-                              int *active, const int *nact_prev, int *nact_next, int *iters) {
+template <int NCOMP>
+__global__ void __launch_bounds__(256)
+    k_cg_fin_beta(const double *part, int nblk, int ld, double *state, int *active,
+                  const int *nact_prev, int *nact_next, int *iters) {
   if (*nact_prev == 0) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) *iters += 1;
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= ld) return;
-  const double rhon = warp_sum_blocks(part, nblk, ncomp * ld, j);
-  const double rrn = ncomp == 2 ? warp_sum_blocks(part, nblk, ncomp * ld, ld + j) : rhon;
-  if ((threadIdx.x & 31) == 0) {
-    const double rho = state[j];
-    int a = active[j];
-    state[3 * ld + j] = (a && rho > 0.0) ? rhon / rho : 0.0;
-    if (a) {
-      state[j] = rhon;
-      a = rrn > state[ld + j];
-      active[j] = a;
-    }
-    if (a) atomicAdd(nact_next, 1);
+  const int j0 = blockIdx.x * kFinCols, j = j0 + (int)threadIdx.x;
+  int off[NCOMP];
+#pragma unroll
+  for (int q = 0; q < NCOMP; ++q) off[q] = q * ld + j0;
+  double s[NCOMP];
+  if (!fin_sums<NCOMP>(part, nblk, NCOMP * ld, off, s)) return;
+  const double rhon = s[0], rrn = s[NCOMP - 1], rho = state[j];
+  int a = active[j];
+  state[3 * ld + j] = (a && rho > 0.0) ? rhon / rho : 0.0;
+  if (a) {
+    state[j] = rhon;
+    a = rrn > state[ld + j];
+    active[j] = a;
   }
+  if (a) atomicAdd(nact_next, 1);
 }
 
-// colsum[e] = sum_b part[b][e] for e < ncomp*ld: one warp per entry, fixed order.
-__global__ void k_fin_cols(const double *__restrict__ part, int nblk, int ncomp, int ld,
-                           double *__restrict__ colsum) {
-  const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (e >= ncomp * ld) return;
-  const double s = warp_sum_blocks(part, nblk, ncomp * ld, e);
-  if ((threadIdx.x & 31) == 0) colsum[e] = s;
+// colsum[e] = sum_b part[b][e] for e < ncomp*ld, fixed order.
+__global__ void __launch_bounds__(256)
+    k_fin_cols(const double *__restrict__ part, int nblk, int ncomp, int ld,
+               double *__restrict__ colsum) {
+  const int e0 = blockIdx.x * kFinCols;
+  const int off[1] = {e0};
+  double s[1];
+  if (fin_sums<1>(part, nblk, ncomp * ld, off, s)) colsum[e0 + threadIdx.x] = s[0];
 }
 
 // out[c] = sum_j colsum[c][j], c < ncomp (one CTA, fixed order).
@@ -577,8 +604,6 @@ int grid_blocks(long long n, int rows) {
   return (int)want;
 }
 
-int warp_blocks(int warps) { return (warps * 32 + 255) / 256; }
-
 // The CTA partials buffer holds up to num_sms()*8 x 2 x ld doubles; per-column sums follow.
 double *colsum_area(double *part, int ld) { return part + (size_t)num_sms() * 8 * 2 * ld; }
 
@@ -618,7 +643,7 @@ op_status launch_quad(const Geom &g, const T *Vt, double sigma, const T *X, int 
     k_quad<T><<<dim3(nb, s.gy), s.block, 0, st>>>(g, Vt, (T)(g.cdiag + sigma), X, ld, part);
     count_launch();
   }
-  k_fin_cols<<<warp_blocks(2 * ld), 256, 0, st>>>(part, nb, 2, ld, colsum_area(part, ld));
+  k_fin_cols<<<2 * ld / kFinCols, 256, 0, st>>>(part, nb, 2, ld, colsum_area(part, ld));
   count_launch();
   k_fin_total<<<1, 256, 0, st>>>(colsum_area(part, ld), 2, ld, out);
   count_launch();
@@ -633,7 +658,7 @@ op_status launch_sumsq(long long n, int ld, const T *X, double *part, double *ou
   const int nb = grid_blocks(n, s.rows);
   k_sumsq<T><<<dim3(nb, s.gy), s.block, 0, st>>>(n, ld, X, part);
   count_launch();
-  k_fin_cols<<<warp_blocks(ld), 256, 0, st>>>(part, nb, 1, ld, colsum_area(part, ld));
+  k_fin_cols<<<ld / kFinCols, 256, 0, st>>>(part, nb, 1, ld, colsum_area(part, ld));
   count_launch();
   k_fin_total<<<1, 256, 0, st>>>(colsum_area(part, ld), 1, ld, out);
   count_launch();
@@ -677,7 +702,7 @@ op_status cg_solve(const Geom &g, const T *Vt, double sigma, const T *U, T *W, i
   RowShape s = row_shape(ld, Pack<T>::N);
   const int nb = grid_blocks(g.n, s.rows);
   const dim3 grid(nb, s.gy);
-  const int fb = warp_blocks(ld);
+  const int fb = ld / kFinCols;
   T *R = (T *)w.R, *P = (T *)w.P, *Q = (T *)w.Q;
   double *alpha = w.state + 2 * ld, *beta = w.state + 3 * ld;
   int *ctl = w.ctl;
@@ -759,8 +784,12 @@ op_status cg_solve(const Geom &g, const T *Vt, double sigma, const T *U, T *W, i
         count_launch();
         prof_end(w.prof, st);
         prof_begin(w.prof, PK_CG_FIN, st);
-        k_cg_fin_beta<<<fb, 256, 0, st>>>(w.part, nb, jac ? 2 : 1, ld, w.state, w.active, nprev,
-                                           nnext, ctl + 2);
+        if (jac)
+          k_cg_fin_beta<2><<<fb, 256, 0, st>>>(w.part, nb, ld, w.state, w.active, nprev, nnext,
+                                               ctl + 2);
+        else
+          k_cg_fin_beta<1><<<fb, 256, 0, st>>>(w.part, nb, ld, w.state, w.active, nprev, nnext,
+                                               ctl + 2);
         count_launch();
         prof_end(w.prof, st);
       } else {
@@ -782,8 +811,12 @@ op_status cg_solve(const Geom &g, const T *Vt, double sigma, const T *U, T *W, i
         count_launch();
         prof_end(w.prof, st);
         prof_begin(w.prof, PK_CG_FIN, st);
-        k_cg_fin_beta<<<fb, 256, 0, st>>>(w.part, nb, jac ? 2 : 1, ld, w.state, w.active, nprev,
-                                           nnext, ctl + 2);
+        if (jac)
+          k_cg_fin_beta<2><<<fb, 256, 0, st>>>(w.part, nb, ld, w.state, w.active, nprev, nnext,
+                                               ctl + 2);
+        else
+          k_cg_fin_beta<1><<<fb, 256, 0, st>>>(w.part, nb, ld, w.state, w.active, nprev, nnext,
+                                               ctl + 2);
         count_launch();
         prof_end(w.prof, st);
         prof_begin(w.prof, PK_CG_DIR, st);
@@ -880,7 +913,7 @@ op_status cg_refine(const Geom &g, const double *Vt, const float *Vt32, double s
   RowShape s = row_shape(ld, Pack<double>::N);
   const int nb = grid_blocks(g.n, s.rows);
   const dim3 grid(nb, s.gy);
-  const int fb = warp_blocks(ld);
+  const int fb = ld / kFinCols;
   const double sg = g.cdiag + sigma;
   const long long total = g.n * ld;
   const int eb = (int)std::min<long long>((total / 4 + 255) / 256, (long long)num_sms() * 32);
@@ -1038,27 +1071,24 @@ __global__ void __launch_bounds__(256) k_b_cg_init(const BatchProb *__restrict__
   flat_colsum<3>(acc, m, ld, pb.part + (long long)it.local * 3 * ld);
 }
 
-// Finalisers: grid (column warps, problems).
-__global__ void k_b_fin_init(const BatchProb *__restrict__ B) {
+// Finalisers: grid (groups of kFinCols columns, problems).
+__global__ void __launch_bounds__(256) k_b_fin_init(const BatchProb *__restrict__ B) {
   const BatchProb &pb = B[blockIdx.y];
-  const int ld = pb.ld;
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= ld || *pb.frozen) return;
-  const double rho = warp_sum_blocks(pb.part, pb.n_row_items, 3 * ld, j);
-  const double bb = warp_sum_blocks(pb.part, pb.n_row_items, 3 * ld, ld + j);
-  const double rr = warp_sum_blocks(pb.part, pb.n_row_items, 3 * ld, 2 * ld + j);
-  if ((threadIdx.x & 31) == 0) {
-    const double rtol2 = *pb.cg_rtol2;
-    double *state = pb.state;
-    state[0 * ld + j] = rho;
-    state[1 * ld + j] = rtol2 * bb;
-    state[2 * ld + j] = 0.0;
-    state[3 * ld + j] = 0.0;
-    state[4 * ld + j] = bb;
-    const int a = (j < pb.p) && (rr > rtol2 * bb) && (bb > 0.0);
-    pb.active[j] = a;
-    if (a) atomicAdd(&pb.ctl[1], 1);
-  }
+  const int ld = pb.ld, j0 = blockIdx.x * kFinCols, j = j0 + (int)threadIdx.x;
+  if (j0 >= ld || *pb.frozen) return;
+  const int off[3] = {j0, ld + j0, 2 * ld + j0};
+  double s[3];
+  if (!fin_sums<3>(pb.part, pb.n_row_items, 3 * ld, off, s)) return;
+  const double rho = s[0], bb = s[1], rr = s[2], rtol2 = *pb.cg_rtol2;
+  double *state = pb.state;
+  state[0 * ld + j] = rho;
+  state[1 * ld + j] = rtol2 * bb;
+  state[2 * ld + j] = 0.0;
+  state[3 * ld + j] = 0.0;
+  state[4 * ld + j] = bb;
+  const int a = (j < pb.p) && (rr > rtol2 * bb) && (bb > 0.0);
+  pb.active[j] = a;
+  if (a) atomicAdd(&pb.ctl[1], 1);
 }
 
 template <bool FIRST>
@@ -1094,18 +1124,16 @@ __global__ void __launch_bounds__(256, 4) k_b_cg_p(const BatchProb *__restrict__
   flat_colsum<1>(acc, m, ld, pb.part + (long long)it.local * ld);
 }
 
-__global__ void k_b_fin_alpha(const BatchProb *__restrict__ B, int k) {
+__global__ void __launch_bounds__(256) k_b_fin_alpha(const BatchProb *__restrict__ B, int k) {
   const BatchProb &pb = B[blockIdx.y];
   if (blockIdx.x == 0 && threadIdx.x == 0) pb.ctl[k & 1] = 0;
-  if (*pb.frozen || pb.ctl[(k + 1) & 1] == 0) return;
-  const int ld = pb.ld;
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= ld) return;
-  const double pq = warp_sum_blocks(pb.part, pb.n_row_items, ld, j);
-  if ((threadIdx.x & 31) == 0) {
-    const double rr = pb.state[j];
-    pb.state[2 * ld + j] = (pb.active[j] && pq > 0.0) ? rr / pq : 0.0;
-  }
+  const int ld = pb.ld, j0 = blockIdx.x * kFinCols, j = j0 + (int)threadIdx.x;
+  if (j0 >= ld || *pb.frozen || pb.ctl[(k + 1) & 1] == 0) return;
+  const int off[1] = {j0};
+  double s[1];
+  if (!fin_sums<1>(pb.part, pb.n_row_items, ld, off, s)) return;
+  const double pq = s[0], rr = pb.state[j];
+  pb.state[2 * ld + j] = (pb.active[j] && pq > 0.0) ? rr / pq : 0.0;
 }
 
 __global__ void __launch_bounds__(256, 4) k_b_cg_wr(const BatchProb *__restrict__ B,
@@ -1154,27 +1182,25 @@ __global__ void __launch_bounds__(256, 4) k_b_cg_wr(const BatchProb *__restrict_
   flat_colsum<2>(acc, m, ld, pb.part + (long long)it.local * 2 * ld);
 }
 
-__global__ void k_b_fin_beta(const BatchProb *__restrict__ B, int k) {
+__global__ void __launch_bounds__(256) k_b_fin_beta(const BatchProb *__restrict__ B, int k) {
   const BatchProb &pb = B[blockIdx.y];
-  if (*pb.frozen || pb.ctl[(k + 1) & 1] == 0) return;
+  const int ld = pb.ld, j0 = blockIdx.x * kFinCols, j = j0 + (int)threadIdx.x;
+  if (j0 >= ld || *pb.frozen || pb.ctl[(k + 1) & 1] == 0) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) pb.ctl[2] += 1;
-  const int ld = pb.ld;
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= ld) return;
-  const double rhon = warp_sum_blocks(pb.part, pb.n_row_items, 2 * ld, j);
-  const double rrn = warp_sum_blocks(pb.part, pb.n_row_items, 2 * ld, ld + j);
-  if ((threadIdx.x & 31) == 0) {
-    double *state = pb.state;
-    const double rho = state[j];
-    int a = pb.active[j];
-    state[3 * ld + j] = (a && rho > 0.0) ? rhon / rho : 0.0;
-    if (a) {
-      state[j] = rhon;
-      a = rrn > state[ld + j];
-      pb.active[j] = a;
-    }
-    if (a) atomicAdd(&pb.ctl[k & 1], 1);
+  const int off[2] = {j0, ld + j0};
+  double s[2];
+  if (!fin_sums<2>(pb.part, pb.n_row_items, 2 * ld, off, s)) return;
+  const double rhon = s[0], rrn = s[1];
+  double *state = pb.state;
+  const double rho = state[j];
+  int a = pb.active[j];
+  state[3 * ld + j] = (a && rho > 0.0) ? rhon / rho : 0.0;
+  if (a) {
+    state[j] = rhon;
+    a = rrn > state[ld + j];
+    pb.active[j] = a;
   }
+  if (a) atomicAdd(&pb.ctl[k & 1], 1);
 }
 
 // Energy of the new U: part[item][0][j] = u_j . (H u)_j, part[item][1][j] = u_j . u_j.
@@ -1242,7 +1268,7 @@ op_status launch_b_cg_init(const BatchProb *B, const RowItem *items, int nitems,
 }
 
 op_status launch_b_fin_init(const BatchProb *B, int nprob, int max_ld, cudaStream_t st) {
-  k_b_fin_init<<<dim3(warp_blocks(max_ld), nprob), 256, 0, st>>>(B);
+  k_b_fin_init<<<dim3(max_ld / kFinCols, nprob), 256, 0, st>>>(B);
   count_launch();
   OP_LAUNCH("k_b_fin_init");
   return OP_OK;
@@ -1250,7 +1276,7 @@ op_status launch_b_fin_init(const BatchProb *B, int nprob, int max_ld, cudaStrea
 
 op_status launch_b_cg_iter(const BatchProb *B, const RowItem *items, int nitems, int nprob,
                            int max_ld, int k, cudaStream_t st) {
-  const dim3 fg(warp_blocks(max_ld), nprob);
+  const dim3 fg(max_ld / kFinCols, nprob);
   if (k == 0)
     k_b_cg_p<true><<<nitems, 256, 0, st>>>(B, items, k);
   else

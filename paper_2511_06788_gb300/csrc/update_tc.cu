@@ -134,10 +134,10 @@ __device__ __forceinline__ void update_tc_body(long long n, int ld, const float 
         *reinterpret_cast<float4 *>(stage + 2 * kPieceA + kPieceB + off) = vl[j];
       }
     }
-    if (s + 1 < nslab) load(s + 1);
     tc::fence_async_smem();
     tc::tc_fence_before();
     __syncthreads();
+    if (s + 1 < nslab) load(s + 1);  // (after the fence, which waits for every access before it)
     if (t == 0) {
       tc::tc_fence_after();
       const uint32_t base = tc::smem_u32(stage);
@@ -594,10 +594,10 @@ __global__ void __launch_bounds__(256, 1)
       for (int r = 0; r < 3; ++r)
         *reinterpret_cast<uint4 *>(stage + (3 + r) * kPieceA + off) = vb[j][r];
     }
-    if (s + 1 < nslab) load(s + 1);
     tc::fence_async_smem();
     tc::tc_fence_before();
     __syncthreads();
+    if (s + 1 < nslab) load(s + 1);
     if (t == 0) {
       tc::tc_fence_after();
       const uint32_t base = tc::smem_u32(stage);
