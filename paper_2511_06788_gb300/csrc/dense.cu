@@ -29,10 +29,13 @@ constexpr int kT = 8;  // tile of the small GEMM (8 x 8 outputs per CTA: many CT
 // (op = transpose when ta / tb is set); zero elsewhere in ld x ld.  X, Y may be
 // null.  tout (may be null) gets a T copy.  When *status is set (a failed
 // factorisation upstream) the result is the identity.
-// One CTA of kT x kT threads per kT x kT output tile; the kT-row panel of op(A)
+// One CTA of kT x kT x kKW threads per kT x kT output tile; the kT-row panel of op(A)
 // and the kT-column panel of op(B) are loaded for KC values of k at a time, all
-// loads in flight together (one L2 round trip per chunk).
+// loads in flight together (one L2 round trip per chunk) and along the stored rows.  The
+// kKW threads of an output take every kKW-th k: a chain of p dependent FP64 FMAs was longer
+// than the SM's share of them.  9.0 us at p = 128 and 6.6 at p = 84, by one thread an output 10.6.
 constexpr int kKC = 128;
+constexpr int kKW = 4;
 template <typename T>
 __device__ __forceinline__ void small_gemm_body(int p, int ld, double alpha,
                                                 const double *__restrict__ A, int ta,
@@ -42,24 +45,33 @@ __device__ __forceinline__ void small_gemm_body(int p, int ld, double alpha,
                                                 double *__restrict__ out, T *__restrict__ tout,
                                                 const int *__restrict__ status) {
   __shared__ double As[kT][kKC + 1], Bs[kKC][kT + 1];
-  const int tx = threadIdx.x, ty = threadIdx.y, t = ty * kT + tx;
+  __shared__ double part[kKW - 1][kT][kT];
+  const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z, t = (tz * kT + ty) * kT + tx;
   const int i0 = blockIdx.y * kT, j0 = blockIdx.x * kT;
   const int i = i0 + ty, j = j0 + tx;
   double s = 0.0;
   for (int k0 = 0; k0 < p; k0 += kKC) {
-    for (int e = t; e < kT * kKC; e += kT * kT) {
-      const int r = e / kKC, k = k0 + e % kKC, ii = i0 + r;
-      As[r][e % kKC] = (ii < p && k < p) ? (ta ? A[(long long)k * ld + ii] : A[(long long)ii * ld + k])
-                                         : 0.0;
-      const int c = e % kT, kb = k0 + e / kT, jj = j0 + c;
-      Bs[e / kT][c] = (kb < p && jj < p) ? (tb ? B[(long long)jj * ld + kb] : B[(long long)kb * ld + jj])
-                                         : 0.0;
+#pragma unroll
+    for (int e = t; e < kT * kKC; e += kT * kT * kKW) {
+      const int a = e % kKC, b = e / kKC, c = e % kT, d = e / kT;  // a, d: k; b, c: row or column
+      const int ra = ta ? c : b, ka = ta ? d : a, cb = tb ? b : c, kb = tb ? a : d;
+      As[ra][ka] = (i0 + ra < p && k0 + ka < p)
+                       ? A[ta ? (long long)(k0 + ka) * ld + i0 + ra : (long long)(i0 + ra) * ld + k0 + ka]
+                       : 0.0;
+      Bs[kb][cb] = (k0 + kb < p && j0 + cb < p)
+                       ? B[tb ? (long long)(j0 + cb) * ld + k0 + kb : (long long)(k0 + kb) * ld + j0 + cb]
+                       : 0.0;
     }
     __syncthreads();
     const int kn = (p - k0) < kKC ? (p - k0) : kKC;
-    for (int k = 0; k < kn; ++k) s = fma(As[ty][k], Bs[k][tx], s);
+    for (int k = tz; k < kn; k += kKW) s = fma(As[ty][k], Bs[k][tx], s);
     __syncthreads();
   }
+  if (tz) part[tz - 1][ty][tx] = s;
+  __syncthreads();
+  if (tz) return;
+#pragma unroll
+  for (int q = 0; q < kKW - 1; ++q) s += part[q][ty][tx];
   if (i >= ld || j >= ld) return;
   double v = 0.0;
   if (i < p && j < p) {
@@ -209,78 +221,119 @@ __global__ void k_tri_cols(int p, int ld, const double *__restrict__ L, int mode
   for (int i = t; i < ld; i += nt) out[(long long)i * ld + j] = (i < p) ? y[i] : 0.0;
 }
 
+// FP64 <-> FP32 on the integer pipe: the conversion instructions run at the FP64 rate, 2 a clock
+// and SM, so the 2 x 16384 of one CTA's 128 x 128 block took 10 us of k_gj32.  narrow rounds to
+// nearest even and widen is exact, both as the instructions do, which take what is not zero or
+// normal in FP32.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const unsigned long long m = u & 0x7fffffffffffffffull;
+  const unsigned e = (unsigned)(m >> 52);
+  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+  if (m == 0) return __uint_as_float(sign);
+  if (e - 897u > 253u) return (float)x;
+  const unsigned long long r = m + 0x0fffffffull + ((m >> 29) & 1);
+  return __uint_as_float(((unsigned)(r >> 29) - (896u << 23)) | sign);
+}
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  if (m == 0) return __hiloint2double((int)u, 0);
+  if ((m >> 23) - 1u > 253u) return (double)x;
+  return __hiloint2double((int)(((m >> 3) + (896u << 20)) | (u & 0x80000000u)), (int)(m << 29));
+}
+
 // Inverse of the p x p matrix M (stride ld, p <= 128) in FP32 by blocked Gauss-Jordan
-// elimination without pivoting, one CTA of 32 x 32 threads.  [M | I] is padded to
-// 128 x 256 with an identity block and held in registers: thread (tx, ty) owns rows
-// ty + 32a (a < 4) and columns tx + 32b (b < 8).  The 128 pivots are taken in 16
-// groups K of kG = 8.  For a group, with P = A[K, K]:
-//   A[K, :] <- P^-1 A[K, :]                       (the pivot rows, Z)
-//   A[i, :] <- A[i, :] - A[i, K] Z    (i not in K)
-// which equals kG single-pivot steps in exact arithmetic.  Per group the pivot rows and
-// columns are published to shared memory, 256 threads form Z column by column (each
-// Gauss-Jordan on the kG x 256 panel), and every thread applies the rank-kG update to
-// its 32 entries.  The panel elimination synchronises only the 8 warps that hold it.
+// elimination without pivoting, in place, one CTA of 256 threads.  M is padded to 128 x 128
+// with an identity block and held in registers.  The pivots are taken in groups K of kG = 8.
+// For a group, with P = A[K, K]:
+//   Z = P^-1 A[K, :], but P^-1 itself in the columns K
+//   A[i, :] <- A[i, :] - A[i, K] Z    (i not in K; the columns K from zero)
+//   A[K, :] <- Z
+// which equals kG single-pivot steps of the elimination of [M | I] in exact arithmetic: the
+// columns that [M | I] still holds as identity, and those already reduced to it, are not
+// carried.  Per group: the owners publish the pivot rows and columns to shared memory; the
+// first four warps form Z, one column per lane, each warp eliminating P for itself in eight
+// more registers, so that a step is eight shuffles and no barrier; every thread then applies
+// the rank-kG update to its 8 x 8 entries.  A warp owns 64 rows x 32 columns, lane (lr, lc)
+// the rows lr + 8a and the columns 4 lc + 16 h + b: a group of pivot rows is one register row
+// of four warps, and an update reads 128 values of Z and of A[:, K] per 512 FMA, all as
+// conflict-free 16-byte loads (rows of colblk are padded to 12 floats).  Bound by the serial
+// chain of p pivots (a division and a few dependent operations each) and by shared memory
+// bandwidth in the updates.  54 us at p = 128, 42 at p = 84; with [M | I] held and a barrier a
+// step it took 106 and 101.
 // The result seeds the FP64 Newton-Schulz refinement in core(); on GB300 an FP64
 // factorisation on one SM costs ~p^3/3 / (2 FMA/clk), while FP32 runs 64x faster.
 // status <- 1 on a zero or non-finite pivot.
 constexpr int kG = 8;
+constexpr int kGjThreads = 256;
 __device__ __forceinline__ void gj32_body(int p, int ld, const double *__restrict__ M,
                                           double *__restrict__ X, int *status) {
-  __shared__ float rowblk[kG][256];  // A[K, :]
-  __shared__ float colblk[128][kG];  // A[:, K]
-  __shared__ float zblk[kG][256];    // P^-1 A[K, :]
-  __shared__ float pcol[2][kG];      // pivot column of the panel elimination (double-buffered)
-  const int tx = threadIdx.x, ty = threadIdx.y, t = ty * 32 + tx;
-  float v[4][8];
+  __shared__ __align__(16) float rowblk[kG][128];     // A[K, :]
+  __shared__ __align__(16) float colblk[2][128][12];  // A[:, K], double-buffered
+  __shared__ __align__(16) float zblk[kG][128];       // Z
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int lr = lane >> 2;
+  const int i0 = 64 * (w >> 2) + lr;             // rows i0 + 8 a
+  const int j0 = 32 * (w & 3) + 4 * (lane & 3);  // columns j0 + 16 h + b
+  float v[8][2][4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 8; ++a)
 #pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const int i = ty + 32 * a, j = tx + 32 * b;
-      float x;
-      if (j < 128) x = (i < p && j < p) ? (float)M[(long long)i * ld + j] : (i == j ? 1.f : 0.f);
-      else x = (j - 128 == i) ? 1.f : 0.f;
-      v[a][b] = x;
-    }
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int i = i0 + 8 * a, j = j0 + 16 * h + b;
+        v[a][h][b] = (i < p && j < p) ? narrow(M[(long long)i * ld + j]) : (i == j ? 1.f : 0.f);
+      }
   bool bad = false;
 #pragma unroll 1
   for (int k0 = 0; k0 < p; k0 += kG) {  // (the padding is an identity block: its pivots do nothing)
-    const int ak = k0 >> 5, r0 = k0 & 31;
-    // publish the pivot rows (owners: a == ak, ty in [r0, r0 + kG)) and columns
-    // (owners: b == ak, tx in [r0, r0 + kG))
+    float(*cb)[12] = colblk[(k0 >> 3) & 1];
+    const int ak = (k0 >> 3) & 7;  // the pivot rows are register row ak of these warps
+    const bool own = (w >> 2) == (k0 >> 6);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-      if (a == ak && ty >= r0 && ty < r0 + kG) {
+    for (int a = 0; a < 8; ++a)
+      if (own && a == ak) {
 #pragma unroll
-        for (int b = 0; b < 8; ++b) rowblk[ty - r0][tx + 32 * b] = v[a][b];
+        for (int h = 0; h < 2; ++h)
+          *reinterpret_cast<float4 *>(&rowblk[lr][j0 + 16 * h]) =
+              make_float4(v[a][h][0], v[a][h][1], v[a][h][2], v[a][h][3]);
       }
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
-      if (b == ak && tx >= r0 && tx < r0 + kG) {
+    for (int h = 0; h < 2; ++h)
+      if (((j0 + 16 * h) & ~7) == k0) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a) colblk[ty + 32 * a][tx - r0] = v[a][b];
+        for (int a = 0; a < 8; ++a) {
+          *reinterpret_cast<float4 *>(&cb[i0 + 8 * a][j0 & 7]) =
+              make_float4(v[a][h][0], v[a][h][1], v[a][h][2], v[a][h][3]);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) v[a][h][b] = 0.f;
+        }
       }
     __syncthreads();
-    // Z = P^-1 A[K, :]: Gauss-Jordan on the kG x 256 panel A[K, :], thread t < 256
-    // holding column t; the pivot column of step c is column k0 + c, published by its
-    // owner (warps 0..7 synchronise among themselves with barrier 1)
     bool fail = false;
-    if (t < 256) {
-      float z[kG];
+    if (w < 4) {  // column t of Z; lane l also holds column l & 7 of P
+      float z[kG], zp[kG];
 #pragma unroll
-      for (int r = 0; r < kG; ++r) z[r] = rowblk[r][t];
+      for (int r = 0; r < kG; ++r) {
+        zp[r] = rowblk[r][k0 + (lane & 7)];
+        z[r] = (t & ~7) == k0 ? (t - k0 == r ? 1.f : 0.f) : rowblk[r][t];
+      }
 #pragma unroll
       for (int c = 0; c < kG; ++c) {
-        if (t == k0 + c) {
+        float m[kG];
 #pragma unroll
-          for (int r = 0; r < kG; ++r) pcol[c & 1][r] = z[r];
-        }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        const float d = pcol[c & 1][c];
-        if (!(fabsf(d) > 1e-30f) || !isfinite(d)) fail = true;  // uniform
-        const float zc = z[c] / d;
+        for (int r = 0; r < kG; ++r) m[r] = __shfl_sync(0xffffffffu, zp[r], c);
+        if (!(fabsf(m[c]) > 1e-30f) || !isfinite(m[c])) fail = true;  // uniform
+        const float inv = 1.f / m[c];
+        z[c] *= inv;
+        zp[c] *= inv;
 #pragma unroll
-        for (int r = 0; r < kG; ++r) z[r] = (r == c) ? zc : fmaf(-pcol[c & 1][r], zc, z[r]);
+        for (int r = 0; r < kG; ++r)
+          if (r != c) {
+            z[r] = fmaf(-m[r], z[c], z[r]);
+            zp[r] = fmaf(-m[r], zp[c], zp[r]);
+          }
       }
 #pragma unroll
       for (int r = 0; r < kG; ++r) zblk[r][t] = z[r];
@@ -289,47 +342,56 @@ __device__ __forceinline__ void gj32_body(int p, int ld, const double *__restric
       bad = true;
       break;
     }
-    // rank-kG update of this thread's entries (one multiplier and one Z value per load,
-    // applied to all four rows); the pivot rows become Z
-    const bool own = ty >= r0 && ty < r0 + kG;
 #pragma unroll
-    for (int g = 0; g < kG; ++g) {
-      float c[4];
+    for (int q = 0; q < kG; q += 4) {
+      float4 c[8];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) c[a] = (a == ak && own) ? 0.f : colblk[ty + 32 * a][g];
+      for (int a = 0; a < 8; ++a) c[a] = *reinterpret_cast<const float4 *>(&cb[i0 + 8 * a][q]);
 #pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const float zv = zblk[g][tx + 32 * b];
+      for (int g = 0; g < 4; ++g)
 #pragma unroll
-        for (int a = 0; a < 4; ++a) v[a][b] = fmaf(-c[a], zv, v[a][b]);
-      }
+        for (int h = 0; h < 2; ++h) {
+          const float4 z = *reinterpret_cast<const float4 *>(&zblk[q + g][j0 + 16 * h]);
+#pragma unroll
+          for (int a = 0; a < 8; ++a) {
+            const float m = g == 0 ? c[a].x : g == 1 ? c[a].y : g == 2 ? c[a].z : c[a].w;
+            v[a][h][0] = fmaf(-m, z.x, v[a][h][0]);
+            v[a][h][1] = fmaf(-m, z.y, v[a][h][1]);
+            v[a][h][2] = fmaf(-m, z.z, v[a][h][2]);
+            v[a][h][3] = fmaf(-m, z.w, v[a][h][3]);
+          }
+        }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-      if (a == ak && own) {
+    for (int a = 0; a < 8; ++a)
+      if (own && a == ak) {
 #pragma unroll
-        for (int b = 0; b < 8; ++b) v[a][b] = zblk[ty - r0][tx + 32 * b];
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) v[a][h][b] = zblk[lr][j0 + 16 * h + b];
       }
-    __syncthreads();  // rowblk / colblk / zblk are rewritten by the next group
+    // the next group writes rowblk (last read before the barrier above), the other half of
+    // colblk, and zblk only after its own first barrier
   }
   if (bad) {
-    if (tx == 0 && ty == 0) *status = 1;
+    if (t == 0) *status = 1;
     return;
   }
-  // right half: M^-1 (rows and columns >= p are the padding identity)
+  // M^-1 (rows and columns >= p are the padding identity; p <= 128 gives ld <= 128)
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 8; ++a)
 #pragma unroll
-    for (int b = 4; b < 8; ++b) {
-      const int i = ty + 32 * a, j = tx + 32 * b - 128;
-      if (i < ld && j < ld) X[(long long)i * ld + j] = (i < p && j < p) ? (double)v[a][b] : 0.0;
-    }
-  // entries of X beyond the 128 x 128 block (ld > 128 cannot occur here: p <= 128 gives
-  // ld <= 128)
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int i = i0 + 8 * a, j = j0 + 16 * h + b;
+        if (i < ld && j < ld)
+          X[(long long)i * ld + j] = (i < p && j < p) ? widen(v[a][h][b]) : 0.0;
+      }
 }
 
-__global__ void __launch_bounds__(1024) k_gj32(int p, int ld, const double *__restrict__ M,
-                                               double *__restrict__ X, int *status) {
+__global__ void __launch_bounds__(kGjThreads) k_gj32(int p, int ld, const double *__restrict__ M,
+                                                     double *__restrict__ X, int *status) {
   gj32_body(p, ld, M, X, status);
 }
 
@@ -549,7 +611,7 @@ __global__ void k_b_core_gemm(const BatchProb *__restrict__ Bp, int op) {
   }
 }
 
-__global__ void __launch_bounds__(1024) k_b_gj32(const BatchProb *__restrict__ Bp) {
+__global__ void __launch_bounds__(kGjThreads) k_b_gj32(const BatchProb *__restrict__ Bp) {
   const BatchProb &pb = Bp[blockIdx.x];
   if (*pb.frozen) return;
   gj32_body(pb.p, pb.ld, pb.core_M, pb.core_X, pb.core_status);
@@ -775,9 +837,8 @@ __global__ void k_ns_resid(int p, int ld, const double *__restrict__ T, double *
 __global__ void k_maxabs(int p, int ld, const double *__restrict__ R,
                          unsigned long long *err_bits) {
   double mx = 0.0;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)p * p;
-       e += (long long)gridDim.x * blockDim.x)
-    mx = fmax(mx, fabs(R[(e / p) * ld + e % p]));
+  for (int i = blockIdx.x; i < p; i += gridDim.x)
+    for (int j = threadIdx.x; j < p; j += blockDim.x) mx = fmax(mx, fabs(R[(long long)i * ld + j]));
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0 && mx > 0.0)
     atomicMax(err_bits, (unsigned long long)__double_as_longlong(mx));
@@ -834,7 +895,7 @@ op_status core(int p, int ld, double tau, const double *C, const double *S, doub
   double *B = L + (size_t)ld * ld;
   double *R = B + (size_t)ld * ld;
   double *E = R + (size_t)ld * ld;
-  const dim3 tb(kT, kT), tg((ld + kT - 1) / kT, (ld + kT - 1) / kT);
+  const dim3 tb(kT, kT, kKW), tg((ld + kT - 1) / kT, (ld + kT - 1) / kT);
   const double q = 0.25 * tau * tau;
   OP_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
   // Step 2 matrix, solving (4.1) without assuming C = <W,U> symmetric:
@@ -845,7 +906,7 @@ op_status core(int p, int ld, double tau, const double *C, const double *S, doub
   if (p <= 128) {
     // B = M^-1: FP32 Gauss-Jordan, then Newton-Schulz X <- X + X (I - M X) in FP64
     // (each step squares the residual: 1e-7 -> 1e-14 -> roundoff)
-    k_gj32<<<1, dim3(32, 32), 0, st>>>(p, ld, M, L, status);
+    k_gj32<<<1, kGjThreads, 0, st>>>(p, ld, M, L, status);
     count_launch();
     const int nref = std::is_same<T, double>::value ? 2 : 1;
     double *X = L, *Xn = B;
@@ -871,7 +932,7 @@ op_status core(int p, int ld, double tau, const double *C, const double *S, doub
                                             (double *)nullptr, (const int *)nullptr);
     count_launch();
     OP_CUDA(cudaMemsetAsync(err_bits, 0, sizeof(unsigned long long), st));
-    k_maxabs<<<8, 256, 0, st>>>(p, ld, R, err_bits);
+    k_maxabs<<<p, 128, 0, st>>>(p, ld, R, err_bits);
     count_launch();
     // FP64 contexts refine twice (residual ~1e-15); FP32 contexts once (their blocks carry
     // 6e-8 anyway): fall back beyond 1e-12 and 1e-6 respectively
@@ -978,12 +1039,12 @@ op_status launch_paper_lams(int p, const double *mu, double sigma, double *lam, 
 }
 
 op_status launch_b_core(const BatchProb *B, int nprob, int max_ld, cudaStream_t st) {
-  const dim3 tb(kT, kT), tg((max_ld + kT - 1) / kT, (max_ld + kT - 1) / kT, nprob);
+  const dim3 tb(kT, kT, kKW), tg((max_ld + kT - 1) / kT, (max_ld + kT - 1) / kT, nprob);
   k_b_core_misc<<<nprob, 1024, 0, st>>>(B, 0);
   count_launch();
   k_b_core_gemm<<<tg, tb, 0, st>>>(B, BC_M);
   count_launch();
-  k_b_gj32<<<nprob, dim3(32, 32), 0, st>>>(B);
+  k_b_gj32<<<nprob, kGjThreads, 0, st>>>(B);
   count_launch();
   k_b_core_gemm<<<tg, tb, 0, st>>>(B, BC_R);
   count_launch();

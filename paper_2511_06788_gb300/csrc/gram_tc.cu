@@ -35,8 +35,8 @@ namespace opevo {
 namespace {
 
 constexpr int kTM = 128;                      // output tile (rows and columns)
-// reduce grid: one thread per output element of a tile (the split sums stay in order)
-constexpr int kReduceSlices = kTM * kTM / 256;
+constexpr int kRedLanes = 64, kRedGroups = 4;  // reduce: elements x split groups of a CTA
+constexpr int kReduceSlices = kTM * kTM / kRedLanes;
 constexpr int kKS = 32;                       // grid points per slab (one 128-byte K row)
 constexpr int kPiece = kTM * 128;             // bytes of one operand piece (128 rows x 128 B)
 constexpr int kStage = 4 * kPiece;            // A_hi, A_lo, B_hi, B_lo
@@ -544,36 +544,58 @@ __global__ void __launch_bounds__(256, 1)
                  three != 0);
 }
 
-// Sum over the splits of element e of a partial tile, in order: FP32 partials as an error-free
-// pair of floats (two-sum; the FP64 pipe would take longer than reading them), or FP64.
-__device__ __forceinline__ double sum_splits(const float *p, long long stride, int nsplit) {
+// A running sum of partials: FP32 ones as an error-free pair of floats (two-sum; the FP64 pipe
+// would take longer than reading them), or FP64.
+template <typename P> struct SplitSum;
+template <> struct SplitSum<float> {
   float h = 0.f, l = 0.f;
-#pragma unroll 8
-  for (int sp = 0; sp < nsplit; ++sp) {
-    const float v = p[sp * stride], s = __fadd_rn(h, v), b = __fsub_rn(s, h);
+  __device__ __forceinline__ void add(float v) {
+    const float s = __fadd_rn(h, v), b = __fsub_rn(s, h);
     l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b)));
     h = s;
   }
-  return l == l ? (double)h + (double)l : (double)h;  // (an overflowed sum has no low part)
-}
-__device__ __forceinline__ double sum_splits(const double *p, long long stride, int nsplit) {
+  __device__ __forceinline__ void merge(const SplitSum &o) {
+    add(o.h);
+    l = __fadd_rn(l, o.l);
+  }
+  __device__ __forceinline__ double value() const {
+    return l == l ? (double)h + (double)l : (double)h;  // (an overflowed sum has no low part)
+  }
+};
+template <> struct SplitSum<double> {
   double s = 0.0;
-  for (int sp = 0; sp < nsplit; ++sp) s += p[sp * stride];
-  return s;
-}
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void merge(const SplitSum &o) { s += o.s; }
+  __device__ __forceinline__ double value() const { return s; }
+};
 
 // out(i, j) = the summed tile element, zero outside p x p, both triangles of S and D.
+// A CTA of kRedLanes x kRedGroups threads: group g sums every kRedGroups-th split, the first
+// group adds the sums up.  One thread per element and all its splits was a serial chain of up to
+// 228 loads and two-sums: 24 us at 262144 x 128, now 13.
 template <typename P>
 __device__ __forceinline__ void reduce_tile(int prod, int ti, int tj, int slice, int slices,
                                             const P *part, long long stride, int nsplit, int p,
                                             int ld, double *out) {
-  for (int e = slice * blockDim.x + threadIdx.x; e < kTM * kTM; e += slices * blockDim.x) {
-    const int i = ti * kTM + e % kTM, j = tj * kTM + e / kTM;
-    if (i >= ld || j >= ld) continue;
-    const double s = sum_splits(part + e, stride, nsplit);
-    const double v = (i < p && j < p) ? s : 0.0;
-    out[(long long)i * ld + j] = v;
-    if (prod != PROD_C && ti != tj) out[(long long)j * ld + i] = v;
+  __shared__ SplitSum<P> sh[kRedGroups - 1][kRedLanes];
+  const int lane = threadIdx.x % kRedLanes, g = threadIdx.x / kRedLanes;
+  for (int e0 = slice * kRedLanes; e0 < kTM * kTM; e0 += slices * kRedLanes) {
+    const int e = e0 + lane, i = ti * kTM + e % kTM, j = tj * kTM + e / kTM;
+    SplitSum<P> s;
+    if (i < p && j < p) {
+#pragma unroll 8
+      for (int sp = g; sp < nsplit; sp += kRedGroups) s.add(part[e + sp * stride]);
+    }
+    if (g) sh[g - 1][lane] = s;
+    __syncthreads();
+    if (g == 0 && i < ld && j < ld) {
+#pragma unroll
+      for (int q = 0; q < kRedGroups - 1; ++q) s.merge(sh[q][lane]);
+      const double v = (i < p && j < p) ? s.value() : 0.0;
+      out[(long long)i * ld + j] = v;
+      if (prod != PROD_C && ti != tj) out[(long long)j * ld + i] = v;
+    }
+    __syncthreads();
   }
 }
 
@@ -666,7 +688,7 @@ op_status gram_tc(long long n, int p, int ld, const float *U, const float *W, do
     OP_TRY(launch_gram_ws(GramSrc{n, rps, (long long)nj * nsplit, ld, mask, nt, nj, U, W, part,
                                   nullptr, err}, split, st));
   }
-  k_gram_tc_reduce<float><<<dim3(nj, kReduceSlices), 256, 0, st>>>(mask, nt, nj, nsplit, part, p, ld,
+  k_gram_tc_reduce<float><<<dim3(nj, kReduceSlices), kRedLanes * kRedGroups, 0, st>>>(mask, nt, nj, nsplit, part, p, ld,
                                                              C, S, D);
   count_launch();
   OP_LAUNCH("k_gram_tc_reduce");
@@ -700,7 +722,7 @@ op_status gram_tc_fixed_scratch(long long n, int p, int ld, const float *U, cons
   OP_CUDA(cudaMemsetAsync(part, 0, (size_t)nj * tile_bytes, st));
   OP_TRY(launch_gram_ws(GramSrc{n, rps, (long long)nj * nsplit, ld, mask, nt, nj, U, W, nullptr,
                                 (double *)part, err}, 1, st));
-  k_gram_tc_reduce<double><<<dim3(nj, kReduceSlices), 256, 0, st>>>(mask, nt, nj, 1, (const double *)part,
+  k_gram_tc_reduce<double><<<dim3(nj, kReduceSlices), kRedLanes * kRedGroups, 0, st>>>(mask, nt, nj, 1, (const double *)part,
                                                              p, ld, C, S, D);
   count_launch();
   OP_LAUNCH("k_gram_tc_reduce");
@@ -711,7 +733,7 @@ op_status launch_b_gram(const BatchProb *B, const GramItem *items, int nitems, i
                         int parity, cudaStream_t st) {
   OP_TRY(launch_gram_ws(GramBatchSrc{nitems, B, items, parity}, 1, st));
   // at most 3 * 8 * 8 + ... jobs for ld <= 1024: grid x covers the largest job count
-  k_b_gram_tc_reduce<<<dim3(tc_jobs(8, 7), nprob, 4), 256, 0, st>>>(B);
+  k_b_gram_tc_reduce<<<dim3(tc_jobs(8, 7), nprob, 8), kRedLanes * kRedGroups, 0, st>>>(B);
   count_launch();
   OP_LAUNCH("k_b_gram_tc_reduce");
   return OP_OK;
