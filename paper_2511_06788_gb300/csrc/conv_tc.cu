@@ -7,19 +7,23 @@
 // with X channels-last [point][ci] on an N^3 grid, taps t = (dz+1) 9 + (dy+1) 3 + (dx+1)
 // (27 taps, zero outside the grid) or the point itself (1 tap).
 //
-// Tiling: one CTA per 128 grid points (the MMA's M), all output channels at once
-// (N = Cout rounded up to 16, at most 128), one FP32 accumulator, K in order.  Two kernels with
+// Tiling: tiles of 128 grid points (the MMA's M), all output channels at once
+// (N = Cout rounded up to 16, at most 128), one FP32 accumulator a tile, K in order.  Two kernels with
 // the same products in the same order (bit-identical results):
 //
 // k_conv_tma (Cin a multiple of 8, or few K values).  A first pass rounds X to BF16 once, into a copy with one
 // point of zeros around the grid, so a tap of a run of points is the same run shifted by a
 // constant number of rows: TMA loads A as boxes of 128 rows, 64, 32 or 16 channels wide, and two
-// 8-wide boxes for a K step that straddles two taps.  No value is gathered or converted again;
-// the tiles run over the padded points between the first and the last grid point (about 9 %
-// more at 48^3).  A stage of the ring holds up to 64 K values (as many pieces as fit).  One thread
-// loads, one issues the MMAs, four warps write the outputs.  What is left is the issue of the
-// copies and MMAs, 500 to 700 clocks a piece for one thread each.  The 11 layers at 48^3, widths
-// 24, 48, 96, p = 64: 0.50 ms and 0.10 ms for the copies, by k_conv_tc 1.37 ms.
+// 8-wide boxes for a K step that straddles two taps.  A narrow box takes as long as a wide one, so
+// where it saves a third of them the copy holds the three taps along x of a point side by side
+// (merge_x).  No value is gathered or converted again; the tiles run over the padded points
+// between the first and the last grid point (about 9 % more at 48^3).  Up to three persistent
+// CTAs an SM: one thread loads A, one B (a box of 64 K values a stage, whatever pieces A comes
+// in), one issues the MMAs into two accumulators in turn, four warps write the outputs of the
+// other.  With one CTA a tile the first loads and the outputs stood beside nothing, and 937 tiles
+// made four waves where three and a bit were work.  Bound by the copies: 27 taps of narrow rows.
+// The 11 layers at 48^3, widths 24, 48, 96, p = 64: 0.39 ms and 0.12 ms for the BF16 copies; one
+// CTA a tile and a box per tap 0.51 and 0.10, by k_conv_tc 1.37 ms.
 //
 // k_conv_tc (other layers).  K in slabs of 64; the 256 threads gather a slab of A from FP32 (27
 // taps, zero padding) and convert it, one thread issues the slab's MMAs; the gather of slab
@@ -242,17 +246,18 @@ __global__ void __launch_bounds__(256) k_conv_tc(const ConvTc a) {
 }
 
 // ---- TMA-fed kernel -------------------------------------------------------------------
-constexpr int kTmaThreads = 192;           // producer, MMA and four epilogue warps
+constexpr int kTmaThreads = 224;           // A copies, MMA, four epilogue warps, B copies
 constexpr int kMaxStages = 8;
 constexpr uint64_t kWaitNs = 2000000000ull;
 
 // BF16 weights as k_conv_wt, and the BF16 copy of X: rows of cin values, the grid points with
 // one point of zeros around them (pad = 1, row ((z + 1) Np + y + 1) Np + x + 1, Np = N + 2) or
-// as they are (pad = 0); or (gcin > 0) the gathered rows themselves, cin = K rounded up values of
-// the taps of gcin channels.  One thread per 8 values.
+// as they are (pad = 0), with the xcin = cin channels of the point or (cin = 3 xcin) those of the
+// point and its neighbours along x; or (gcin > 0) the gathered rows themselves, cin = K rounded up
+// values of the taps of gcin channels.  One thread per 8 values.
 __global__ void k_conv_prep(const float *__restrict__ W, int K, int cout, int Kp, int coutp,
                             uint16_t *__restrict__ Wt, const float *__restrict__ X, int N, int cin,
-                            int pad, int gcin, uint16_t *__restrict__ Xb) {
+                            int xcin, int pad, int gcin, uint16_t *__restrict__ Xb) {
   const long long wtot = (long long)coutp * Kp, step = (long long)gridDim.x * blockDim.x;
   const long long e0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   for (long long e = e0; e < wtot; e += step) {
@@ -275,11 +280,14 @@ __global__ void k_conv_prep(const float *__restrict__ W, int K, int cout, int Kp
       a.K = K;
       o = gather8(a, x, y, z, true, 8 * (int)v);
     } else if (x >= 0 && x < N && y >= 0 && y < N && z >= 0 && z < N) {
-      const float4 *src = reinterpret_cast<const float4 *>(
-          X + (((long long)z * N + y) * N + x) * cin + 8 * v);
-      const float4 a = __ldg(src), b = __ldg(src + 1);
-      o = make_uint4(bf16_bits(a.x) | (bf16_bits(a.y) << 16), bf16_bits(a.z) | (bf16_bits(a.w) << 16),
-                     bf16_bits(b.x) | (bf16_bits(b.y) << 16), bf16_bits(b.z) | (bf16_bits(b.w) << 16));
+      const int d = 8 * (int)v / xcin, xx = xcin < cin ? x + d - 1 : x;
+      if (xx >= 0 && xx < N) {
+        const float4 *src = reinterpret_cast<const float4 *>(
+            X + (((long long)z * N + y) * N + xx) * xcin + (8 * (int)v - d * xcin));
+        const float4 a = __ldg(src), b = __ldg(src + 1);
+        o = make_uint4(bf16_bits(a.x) | (bf16_bits(a.y) << 16), bf16_bits(a.z) | (bf16_bits(a.w) << 16),
+                       bf16_bits(b.x) | (bf16_bits(b.y) << 16), bf16_bits(b.z) | (bf16_bits(b.w) << 16));
+      }
     }
     *reinterpret_cast<uint4 *>(Xb + e * 8) = o;
   }
@@ -303,7 +311,7 @@ struct KPieces {
 struct ConvTma {
   const float *bias;
   float *Z, *A;
-  int N, pad, cout, coutp, stages;
+  int N, pad, cout, coutp, stages, tiles;
   int q0, q1;            // first output row and one past the last
   int *err;
 };
@@ -319,27 +327,28 @@ __device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr, int lead, int st
 __global__ void __launch_bounds__(kTmaThreads)
     k_conv_tma(const __grid_constant__ CUtensorMap a64, const __grid_constant__ CUtensorMap a32,
                const __grid_constant__ CUtensorMap a16, const __grid_constant__ CUtensorMap a8,
-               const __grid_constant__ CUtensorMap b64, const __grid_constant__ CUtensorMap b32,
-               const __grid_constant__ CUtensorMap b16, const __grid_constant__ KPieces pc,
+               const __grid_constant__ CUtensorMap b64, const __grid_constant__ KPieces pc,
                const ConvTma c) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t full[kMaxStages], empty[kMaxStages], fin;
+  __shared__ uint64_t full[kMaxStages], empty[kMaxStages], fin[2], freed[2];
   __shared__ uint32_t tmem_sh;
   __shared__ int abort_sh;
   __shared__ KPiece piece[kMaxPieces];
   for (int i = threadIdx.x; i < pc.count; i += kTmaThreads) piece[i] = pc.p[i];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q0 = c.q0 + blockIdx.x * kCM;
   const uint32_t ncols = c.coutp <= 32 ? 32u : (c.coutp <= 64 ? 64u : 128u);
   const int stage_bytes = kAPiece + c.coutp * 128;
-  if (warp == 1) tc::tmem_alloc(&tmem_sh, ncols);
+  if (warp == 1) tc::tmem_alloc(&tmem_sh, 2 * ncols);
   if (threadIdx.x == 0) {
     for (int s = 0; s < c.stages; ++s) {
-      tc::mbar_init(&full[s], 1);
+      tc::mbar_init(&full[s], 2);
       tc::mbar_init(&empty[s], 1);
     }
-    tc::mbar_init(&fin, 1);
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&fin[i], 1);
+      tc::mbar_init(&freed[i], 4);
+    }
     tc::fence_mbar_init();
     abort_sh = 0;
   }
@@ -351,102 +360,143 @@ __global__ void __launch_bounds__(kTmaThreads)
 
   if (warp == 0) {
     if (lane == 0) {
-      int it = 0, slot = 0, o = 0, k = 0;
+      int it = 0, slot = 0, o = 0;
       uint32_t phase = 1;  // of the slot's last release (the first use of a slot passes)
       uint8_t *as = smem;
-      for (int i = 0; i < pc.count; ++i) {
-        const KPiece s = piece[i];
-        if (s.stage) {  // a new stage
-          if (it > 0 && ++slot == c.stages) {
-            slot = 0;
-            phase ^= 1;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < c.tiles && ok; tile += gridDim.x) {
+        const int q0 = c.q0 + tile * kCM;
+        for (int i = 0; i < pc.count; ++i) {
+          const KPiece s = piece[i];
+          if (s.stage) {  // a new stage
+            if (it > 0 && ++slot == c.stages) {
+              slot = 0;
+              phase ^= 1;
+            }
+            if (it >= c.stages && !tc::wait_or_abort(&empty[slot], phase, abort, kWaitNs)) {
+              ok = false;
+              break;
+            }
+            as = smem + slot * stage_bytes;
+            o = 0;
+            tma::bar_expect(&full[slot], (uint32_t)(s.stage * 2 * kCM));
+            ++it;
           }
-          if (it >= c.stages && !tc::wait_or_abort(&empty[slot], phase, abort, kWaitNs)) break;
-          as = smem + slot * stage_bytes;
-          o = 0;
-          tma::bar_expect(&full[slot], (uint32_t)(s.stage * (2 * kCM + 2 * c.coutp)));
-          ++it;
-        }
-        uint64_t *bar = &full[slot];
-        uint8_t *ap = as + o * 2 * kCM, *bp = as + kAPiece + o * 2 * c.coutp;
-        const int r = q0 + s.row;
-        int len = s.width;
-        if (s.width == 64) {
-          tma::load_2d(ap, &a64, s.off, r, bar);
-          tma::load_2d(bp, &b64, k, 0, bar);
-        } else if (s.width == 32) {
-          tma::load_2d(ap, &a32, s.off, r, bar);
-          tma::load_2d(bp, &b32, k, 0, bar);
-        } else {
-          if (s.width == 16) {
+          uint64_t *bar = &full[slot];
+          uint8_t *ap = as + o * 2 * kCM;
+          const int r = q0 + s.row;
+          if (s.width == 64) {
+            tma::load_2d(ap, &a64, s.off, r, bar);
+          } else if (s.width == 32) {
+            tma::load_2d(ap, &a32, s.off, r, bar);
+          } else if (s.width == 16) {
             tma::load_2d(ap, &a16, s.off, r, bar);
           } else {
             tma::load_2d(ap, &a8, s.off, r, bar);
             tma::load_2d(ap + 16 * kCM, &a8, 0, q0 + s.row2, bar);
-            len = 16;
           }
-          tma::load_2d(bp, &b16, k, 0, bar);
+          o += s.width == 8 ? 16 : s.width;
         }
-        o += len;
-        k += len;
       }
       // the copies issued last land before the CTA may exit
+      for (int u = it - 1; u >= 0 && u >= it - c.stages; --u)
+        tma::bar_wait(&full[u % c.stages], (uint32_t)((u / c.stages) & 1), kWaitNs);
+    }
+  } else if (warp == kTmaThreads / 32 - 1) {
+    if (lane == 0) {  // B: one box of 64 K values a stage, whatever pieces its A comes in
+      int it = 0, slot = 0;
+      uint32_t phase = 1;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < c.tiles && ok; tile += gridDim.x) {
+        int k = 0;
+        for (int i = 0; i < pc.count; ++i) {
+          const int len = piece[i].stage;
+          if (!len) continue;
+          if (it > 0 && ++slot == c.stages) {
+            slot = 0;
+            phase ^= 1;
+          }
+          if (it >= c.stages && !tc::wait_or_abort(&empty[slot], phase, abort, kWaitNs)) {
+            ok = false;
+            break;
+          }
+          tma::bar_expect(&full[slot], (uint32_t)(kCK * 2 * c.coutp));
+          tma::load_2d(smem + slot * stage_bytes + kAPiece, &b64, k, 0, &full[slot]);
+          k += len;
+          ++it;
+        }
+      }
       for (int u = it - 1; u >= 0 && u >= it - c.stages; --u)
         tma::bar_wait(&full[u % c.stages], (uint32_t)((u / c.stages) & 1), kWaitNs);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = tc::idesc_bf16(kCM, c.coutp);
-      int it = 0, slot = 0, o = 0;
-      uint32_t acc = 0, phase = 0, as = 0;
-      for (int i = 0; i < pc.count; ++i) {
-        const KPiece s = piece[i];
-        if (s.stage) {
-          if (it > 0) {
-            tc::mma_commit(&empty[slot]);
-            if (++slot == c.stages) {
-              slot = 0;
-              phase ^= 1;
+      int slot = 0, o = 0, j = 0;  // j: tiles begun
+      uint32_t phase = 0, as = 0;
+      uint64_t bs = 0;
+      bool ok = true, open = false;  // open: a stage whose MMAs are not committed yet
+      for (int tile = blockIdx.x; tile < c.tiles && ok; tile += gridDim.x, ++j) {
+        // two accumulators in turn: the read-out of a tile runs beside the next one
+        if (j >= 2 && !tc::wait_or_abort(&freed[j & 1], (uint32_t)((j >> 1) - 1) & 1, abort, kWaitNs))
+          break;
+        const uint32_t d = tmem + (uint32_t)(j & 1) * ncols;
+        uint32_t acc = 0;
+        for (int i = 0; i < pc.count; ++i) {
+          const KPiece s = piece[i];
+          if (s.stage) {
+            if (open) {
+              tc::mma_commit(&empty[slot]);
+              if (++slot == c.stages) {
+                slot = 0;
+                phase ^= 1;
+              }
             }
+            if (!tc::wait_or_abort(&full[slot], phase, abort, kWaitNs)) {
+              ok = false;
+              break;
+            }
+            tc::tc_fence_after();
+            as = tc::smem_u32(smem + slot * stage_bytes);
+            bs = desc_kmajor(as + kAPiece, 16, 1024, 2);
+            o = 0;
+            open = true;
           }
-          if (!tc::wait_or_abort(&full[slot], phase, abort, kWaitNs)) break;
-          tc::tc_fence_after();
-          as = tc::smem_u32(smem + slot * stage_bytes);
-          o = 0;
-          ++it;
-        }
-        const uint32_t ap = as + o * 2 * kCM, bp = as + kAPiece + o * 2 * c.coutp;
-        if (s.width == 64) {
-          const uint64_t ad = desc_kmajor(ap, 16, 1024, 2), bd = desc_kmajor(bp, 16, 1024, 2);
+          const uint32_t ap = as + o * 2 * kCM;
+          const uint64_t bd = bs + (uint64_t)(o / 8);  // o K values along the 128-byte rows
+          if (s.width == 64) {
+            const uint64_t ad = desc_kmajor(ap, 16, 1024, 2);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks, acc = 1)
-            tc::mma_bf16(tmem, ad + 2 * ks, bd + 2 * ks, idesc, acc);
-          o += 64;
-        } else if (s.width == 32) {
-          const uint64_t ad = desc_kmajor(ap, 16, 512, 4), bd = desc_kmajor(bp, 16, 512, 4);
+            for (int ks = 0; ks < 4; ++ks, acc = 1)
+              tc::mma_bf16(d, ad + 2 * ks, bd + 2 * ks, idesc, acc);
+            o += 64;
+          } else if (s.width == 32) {
+            const uint64_t ad = desc_kmajor(ap, 16, 512, 4);
 #pragma unroll
-          for (int ks = 0; ks < 2; ++ks, acc = 1)
-            tc::mma_bf16(tmem, ad + 2 * ks, bd + 2 * ks, idesc, acc);
-          o += 32;
-        } else {
-          const uint64_t ad =
-              s.width == 16 ? desc_kmajor(ap, 16, 256, 6) : desc_kmajor(ap, 16 * kCM, 128, 0);
-          tc::mma_bf16(tmem, ad, desc_kmajor(bp, 16, 256, 6), idesc, acc);
-          acc = 1;
-          o += 16;
+            for (int ks = 0; ks < 2; ++ks, acc = 1)
+              tc::mma_bf16(d, ad + 2 * ks, bd + 2 * ks, idesc, acc);
+            o += 32;
+          } else {
+            const uint64_t ad =
+                s.width == 16 ? desc_kmajor(ap, 16, 256, 6) : desc_kmajor(ap, 16 * kCM, 128, 0);
+            tc::mma_bf16(d, ad, bd, idesc, acc);
+            acc = 1;
+            o += 16;
+          }
         }
+        tc::mma_commit(&fin[j & 1]);  // (also after a failed wait: the MMAs end before the CTA does)
       }
-      if (it > 0) tc::mma_commit(&fin);
-      else tc::mbar_arrive(&fin);
-      tma::bar_wait(&fin, 0u, kWaitNs);
+      if (j > 0) tma::bar_wait(&fin[(j - 1) & 1], (uint32_t)((j - 1) >> 1) & 1, kWaitNs);
     }
   } else {
-    int ok = 0;
-    if (lane == 0) ok = tc::wait_or_abort(&fin, 0u, abort, kWaitNs) && !*abort;
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    if (ok) {
+    int j = 0;
+    for (int tile = blockIdx.x; tile < c.tiles; tile += gridDim.x, ++j) {
+      int ok = 0;
+      if (lane == 0)
+        ok = tc::wait_or_abort(&fin[j & 1], (uint32_t)(j >> 1) & 1, abort, kWaitNs) && !*abort;
+      if (!__shfl_sync(0xffffffffu, ok, 0)) break;
       tc::tc_fence_after();
-      const int quarter = warp & 3, q = q0 + quarter * 32 + lane;
+      const int quarter = warp & 3, q = c.q0 + tile * kCM + quarter * 32 + lane;
       long long m = q;
       bool in = q < c.q1;
       if (c.pad) {
@@ -455,7 +505,7 @@ __global__ void __launch_bounds__(kTmaThreads)
         in = in && x >= 0 && x < c.N && y >= 0 && y < c.N && z >= 0 && z < c.N;
         m = ((long long)z * c.N + y) * c.N + x;
       }
-      const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16);
+      const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(j & 1) * ncols;
       for (int c0 = 0; c0 < c.coutp; c0 += 8) {
         float v[8];
         tmem_ld8(tb + (uint32_t)c0, v);
@@ -490,15 +540,31 @@ __global__ void __launch_bounds__(kTmaThreads)
           }
         }
       }
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&freed[j & 1]);
     }
   }
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc::tc_fence_after();
-    tc::tmem_dealloc(tmem, ncols);
+    tc::tmem_dealloc(tmem, 2 * ncols);
   }
   if (threadIdx.x == 0 && abort_sh) atomicExch(c.err, 1);
+}
+
+// Copies of 128 rows that a group of `cin` K values takes.
+int boxes(int cin) { return cin / 64 + ((cin & 32) != 0) + ((cin & 16) != 0) + ((cin & 8) != 0); }
+// Whether the copy holds the three taps along x side by side (rows of 3 cin values, 9 groups of
+// taps): where that takes at most two thirds of the boxes and the copy stays within 8 GiB.  The K
+// order, and so every sum, is the same.  48^3, one CTA a tile: 24 -> 24 channels 70 -> 51 us,
+// 48 -> 48 97 -> 83; for 72 channels (5 boxes instead of 6) the three times larger copy would
+// cost what it saves.
+bool merge_x(int N, int taps, int cin) {
+  const long long m = N + 2;
+  return taps == 27 && cin % 8 == 0 && boxes(3 * cin) <= 2 * boxes(cin) &&
+         m * m * m * 3 * cin * 2 <= (8ll << 30);
 }
 
 // Rows and row length of the BF16 copy (0: the layer is left to k_conv_tc).  Channels in 16-byte
@@ -510,6 +576,7 @@ long long copy_rows(int N, int taps, int cin) {
   return m * m * m;
 }
 int copy_len(int N, int taps, int cin) {
+  if (merge_x(N, taps, cin)) return 3 * cin;
   const int len = cin % 8 == 0 ? cin : (taps * cin <= 256 ? (taps * cin + 15) / 16 * 16 : 0);
   return copy_rows(N, taps, cin) * len * 2 <= (8ll << 30) ? len : 0;
 }
@@ -517,6 +584,7 @@ int copy_len(int N, int taps, int cin) {
 void list_pieces(int taps, int cin, int Np, long long rows, KPieces *out) {
   auto shift = [&](int t) -> int {
     if (t >= taps) return (int)rows;  // past the last row: zeros
+    if (taps == 9) return ((t / 3 - 1) * Np + t % 3 - 1) * Np;
     return taps == 1 ? 0 : ((t / 9 - 1) * Np + (t / 3) % 3 - 1) * Np + t % 3 - 1;
   };
   int n = 0, used = kCK, first = 0, off = 0;
@@ -583,7 +651,7 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
     const long long rows = copy_rows(N, taps, cin);
     const long long work = std::max(rows * (clen / 8), (long long)coutp * Kp);
     k_conv_prep<<<(unsigned)std::min<long long>((work + 255) / 256, 16LL * num_sms()), 256, 0, st>>>(
-        W, K, cout, Kp, coutp, Wt, X, N, clen, pad, gcin, Xb);
+        W, K, cout, Kp, coutp, Wt, X, N, clen, gcin ? clen : cin, pad, gcin, Xb);
     count_launch();
     OP_LAUNCH("k_conv_prep");
     ConvTma c;
@@ -598,22 +666,28 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
     const int Np = N + 2;
     c.q0 = pad ? Np * Np + Np + 1 : 0;
     c.q1 = (int)rows - c.q0;
-    // with no more tiles than SMs a CTA has the SM to itself and is bound by the latency of its
-    // loads: as many stages as fit; else two CTAs per SM
     const int tiles = (c.q1 - c.q0 + kCM - 1) / kCM, stage = kAPiece + coutp * 128;
-    c.stages = std::min(kMaxStages, ((tiles <= num_sms() ? 215 : 104) * 1024) / stage);
-    CUtensorMap ma[4], mb[3];
+    KPieces pc;
+    list_pieces(gcin ? 1 : (clen > cin ? 9 : taps), clen, Np, rows, &pc);
+    const int ncols = coutp <= 32 ? 32 : (coutp <= 64 ? 64 : 128);
+    // with no more tiles than SMs a CTA has the SM to itself and is bound by the latency of its
+    // loads: as many stages as fit; else CTAs that cover each other's first loads and waits (the
+    // 11 layers by one CTA an SM 0.698 ms, two 0.619, three 0.615, four 0.617)
+    int per_sm = tiles <= num_sms() ? 1 : std::min(3, 256 / ncols);
+    auto ring = [&](int ctas) { return std::min(kMaxStages, (227 / ctas - 9) * 1024 / stage); };
+    while (per_sm > 1 && ring(per_sm) < 2) --per_sm;
+    c.stages = ring(per_sm);
+    c.tiles = tiles;
+    CUtensorMap ma[4], mb;
     const int wid[4] = {64, 32, 16, 8};
     for (int i = 0; i < 4; ++i)
       OP_TRY(tma_map_2d_bf16(&ma[i], Xb, (uint64_t)clen, (uint64_t)rows, wid[i], kCM));
-    for (int i = 0; i < 3; ++i)
-      OP_TRY(tma_map_2d_bf16(&mb[i], Wt, (uint64_t)Kp, (uint64_t)coutp, wid[i], coutp));
-    KPieces pc;
-    list_pieces(gcin ? 1 : taps, clen, Np, rows, &pc);
-    const int smem = c.stages * (kAPiece + coutp * 128) + 1024;
+    OP_TRY(tma_map_2d_bf16(&mb, Wt, (uint64_t)Kp, (uint64_t)coutp, kCK, coutp));
+    // (room for no more CTAs than their TMEM allows)
+    const int smem = std::max(c.stages * stage, 228 * 1024 / (256 / ncols + 1)) + 1024;
     OP_CUDA(cudaFuncSetAttribute(k_conv_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_conv_tma<<<(unsigned)tiles, kTmaThreads, smem, st>>>(
-        ma[0], ma[1], ma[2], ma[3], mb[0], mb[1], mb[2], pc, c);
+    k_conv_tma<<<(unsigned)std::min(tiles, per_sm * num_sms()), kTmaThreads, smem, st>>>(
+        ma[0], ma[1], ma[2], ma[3], mb, pc, c);
     count_launch();
     OP_LAUNCH("k_conv_tma");
     return OP_OK;
