@@ -82,7 +82,7 @@ def digit_flops(group, n, ld):
     return 0
 KERNEL_NAME = {("cg_apply", "fp32"): "k_cg_tma", ("cg_axpy", "fp32"): "k_cg_wr",
                ("cg_apply", "fp64"): "k_cg_apply", ("cg_axpy", "fp64"): "k_cg_axpy",
-               ("cg_dir", "fp64"): "k_cg_dir", ("gram", "fp32"): "k_gram_tc",
+               ("cg_dir", "fp64"): "k_cg_dir", ("gram", "fp32"): "k_gram_ws",
                ("update", "fp32"): "k_update_ws", ("gram", "fp64"): "k_gram<double>",
                ("update", "fp64"): "k_update<double>"}
 # the TF32 mode runs the FP32 mode's kernels (one MMA per product in the Gram and update);

@@ -406,7 +406,8 @@ op_status op_apply_H(const op_problem *pb, int ld, const void *V_t, double sigma
  * from the W passed in, each column to ||u - (H+sigma) w|| <= rtol ||u||, at most
  * max_iter iterations.  V_t as in op_apply_H; U, W: n x ld blocks of T.  Scratch: ws
  * (device) of at least op_cg_workspace() bytes.  *iters (host) receives the iteration
- * count.  Synchronises `stream` once per iteration (convergence checks). */
+ * count.  Synchronises `stream` (every second iteration for its convergence checks; once
+ * where one launch runs the whole solve: blocks that stay in L2). */
 op_status op_cg_solve(const op_problem *pb, int ld, const void *V_t, double sigma,
                       const void *U, void *W, double rtol, int max_iter, void *ws,
                       size_t ws_bytes, int *iters, void *stream);
@@ -416,7 +417,8 @@ size_t op_cg_workspace(const op_problem *pb, int ld);
  * each ld x ld FP64 row-major on the device (entries with i or j >= p are zero).
  * Any of C, S, D may be NULL to skip it.  OP_FP64: FP64 FMA, chunk partials in FP64.
  * OP_FP32: tcgen05 tensor-core MMAs (TF32 inputs split hi + lo, four MMAs per
- * product, FP32 accumulation per chunk of grid points, chunk partials summed in FP64).
+ * product, FP32 accumulation per chunk of grid points, chunk partials summed as error-free
+ * pairs of floats).
  * OP_MIX_BF16X3: FP32 blocks, BF16 inputs split in three, six kind::f16 MMAs per product.
  * ws: device scratch of at least op_gram_workspace() bytes; its first int is set when a
  * bounded device wait gave up (check with op_ws_status). */
