@@ -530,11 +530,11 @@ template <typename T> bool cg_coop_eligible(long long n, int ld) {
 
 template <typename T>
 op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, int p, int ld,
-                  double rtol, int max_iter, CGWork &w, int *iters, cudaStream_t st) {
+                  double rtol, int max_iter, CGWork &w, int *iters, bool *ran, cudaStream_t st) {
   constexpr int N = Pack<T>::N;
   int rows = 0;
   const int G = coop_ctas<T>(g.n, ld, &rows);
-  const bool cluster = G == kCluster;
+  const bool cluster = G == kCluster && ld <= 64;  // (wider partials leave no room beside them)
   CoopArgs a{};
   a.g = g;
   a.Vt = Vt;
@@ -582,9 +582,17 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
   }
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  OP_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
-  count_launch();
+  const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
   prof_end(w.prof, st);
+  // a process confined to a few SMs may not hold the CTAs together: the general path needs no such thing
+  *ran = e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorInvalidClusterSize &&
+         e != cudaErrorLaunchOutOfResources;
+  if (!*ran) {
+    (void)cudaGetLastError();
+    return OP_OK;
+  }
+  OP_CUDA(e);
+  count_launch();
   OP_CUDA(cudaMemcpyAsync(w.host_ctl, w.ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
   OP_CUDA(cudaStreamSynchronize(st));
   prof_harvest(w.prof);
@@ -600,7 +608,7 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
 #define OPEVO_INST(T)                                                                          \
   template bool cg_coop_eligible<T>(long long, int);                                           \
   template op_status cg_coop<T>(const Geom &, const T *, double, const T *, T *, int, int,     \
-                                double, int, CGWork &, int *, cudaStream_t);
+                                double, int, CGWork &, int *, bool *, cudaStream_t);
 OPEVO_INST(float)
 OPEVO_INST(double)
 #undef OPEVO_INST

@@ -146,11 +146,12 @@ op_status cg_solve(const Geom &g, const T *Vt, double sigma, const T *U, T *W, i
                    double rtol, int max_iter, CGWork &w, int *iters, cudaStream_t st);
 
 // The same solve in one cooperative launch for blocks that stay in L2 (cg_coop.cu); cg_solve
-// takes it where cg_coop_eligible.
+// takes it where cg_coop_eligible; *ran = false (and no work done) where the device cannot hold
+// its CTAs together.
 template <typename T> bool cg_coop_eligible(long long n, int ld);
 template <typename T>
 op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, int p, int ld,
-                  double rtol, int max_iter, CGWork &w, int *iters, cudaStream_t st);
+                  double rtol, int max_iter, CGWork &w, int *iters, bool *ran, cudaStream_t st);
 
 // Step 1 in FP64 by iterative refinement around an FP32 CG: each cycle forms the FP64
 // residual R = U - (H + sigma) W and its column norms (w64: FP64 scratch, its R block and

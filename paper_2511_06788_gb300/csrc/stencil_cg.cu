@@ -696,8 +696,11 @@ void cg_carve(void *ws, long long n, int ld, int elem, CGWork *w) {
 template <typename T>
 op_status cg_solve(const Geom &g, const T *Vt, double sigma, const T *U, T *W, int p, int ld,
                    double rtol, int max_iter, CGWork &w, int *iters, cudaStream_t st) {
-  if (cg_coop_eligible<T>(g.n, ld))
-    return cg_coop<T>(g, Vt, sigma, U, W, p, ld, rtol, max_iter, w, iters, st);
+  if (cg_coop_eligible<T>(g.n, ld)) {
+    bool ran = true;
+    OP_TRY(cg_coop<T>(g, Vt, sigma, U, W, p, ld, rtol, max_iter, w, iters, &ran, st));
+    if (ran) return OP_OK;
+  }
   constexpr bool kFused = std::is_same<T, float>::value;
   RowShape s = row_shape(ld, Pack<T>::N);
   const int nb = grid_blocks(g.n, s.rows);
