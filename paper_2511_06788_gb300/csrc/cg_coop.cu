@@ -35,6 +35,10 @@ constexpr int kCoopThreads = 512;
 // here and 2.90 ms by kernels, 56^3 x 64 (45 MB) 3.43 and 3.54, 64^3 x 84 (92 MB) 8.9 and 7.7.
 // FP64: bound by the FP64 pipe either way: 64^3 x 64 (134 MB, the largest tried) 32.9 and 38.1.
 template <typename T> constexpr long long kCoopBytes = (sizeof(T) == 4 ? 48ll : 140ll) << 20;
+// Dynamic shared memory a launch may ask for (the largest any size below takes is 130 KB).  The
+// limit belongs to the kernel on the device, so every call sets this one value: a limit of the
+// call's own size could be lowered by another thread's solve between setting it and the launch.
+constexpr int kCoopSmem = 224 * 1024;
 // polls of the barrier (several hundred clocks each) before a CTA gives up: some seconds
 constexpr int kBarrierPolls = 1 << 23;
 // ctl words (256 bytes): 2 iterations, 3 error, 32 the barrier's arrivals
@@ -563,7 +567,7 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
   int lanes = 1;
   while (lanes < 32 && 2 * lanes * ld <= kSumThreads<T>) lanes *= 2;
   const void *fn = w.jacobi ? coop_kernel<T, true>(lanes) : coop_kernel<T, false>(lanes);
-  OP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  OP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoopSmem));
   prof_begin(w.prof, PK_CG_APPLY, st);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(G);

@@ -248,6 +248,10 @@ __global__ void __launch_bounds__(256) k_conv_tc(const ConvTc a) {
 // ---- TMA-fed kernel -------------------------------------------------------------------
 constexpr int kTmaThreads = 224;           // A copies, MMA, four epilogue warps, B copies
 constexpr int kMaxStages = 8;
+// Limit of the dynamic shared memory (a ring of (227 - 9) KB at most and 1 KB of alignment slack),
+// the same at every call: it belongs to the kernel on the device, where another thread's call
+// with a smaller ring could lower it between setting it and the launch.
+constexpr int kTmaSmem = 219 * 1024;
 constexpr uint64_t kWaitNs = 2000000000ull;
 
 // BF16 weights as k_conv_wt, and the BF16 copy of X: rows of cin values, the grid points with
@@ -685,7 +689,7 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
     OP_TRY(tma_map_2d_bf16(&mb, Wt, (uint64_t)Kp, (uint64_t)coutp, kCK, coutp));
     // (room for no more CTAs than their TMEM allows)
     const int smem = std::max(c.stages * stage, 228 * 1024 / (256 / ncols + 1)) + 1024;
-    OP_CUDA(cudaFuncSetAttribute(k_conv_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    OP_CUDA(cudaFuncSetAttribute(k_conv_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmaSmem));
     k_conv_tma<<<(unsigned)std::min(tiles, per_sm * num_sms()), kTmaThreads, smem, st>>>(
         ma[0], ma[1], ma[2], ma[3], mb, pc, c);
     count_launch();

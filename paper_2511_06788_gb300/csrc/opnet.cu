@@ -290,6 +290,10 @@ struct WgradPadArgs {
   int apitch, bpitch;  // floats of a stage's A window run (per (dz, dy)) and of its B rows
 };
 constexpr int kWP = 32, kWStages = 3;  // points per stage, stages
+// Bound of the stages' bytes (198,576 at most over the widths a net may have), set as the kernel's
+// limit at every call: a limit of the layer's own size could be lowered by another thread's layer
+// between setting it and the launch.
+constexpr int kWSmem = 200 * 1024;
 
 __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool in) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
@@ -838,7 +842,7 @@ op_status back_layer(opnet *net, int i, const float *X, const float *dZ, float *
     auto bytes = [&](int ng) {
       return kWStages * (ng * w.apitch + w.bpitch) * (int)sizeof(float);
     };
-    while (w.ng > 1 && bytes(w.ng) > 200 * 1024) w.ng /= 3;
+    while (w.ng > 1 && bytes(w.ng) > kWSmem) w.ng /= 3;
     const int threads = (per * w.ng + 31) / 32 * 32, gx = groups / w.ng * w.kblocks;
     // runs of at most 2048 points, more of them while CTAs are missing, down to 128 points (four
     // stages; loss and gradient at 48^3: from 96 points 3.85 ms, 128 3.80, 64 3.84), and the
@@ -850,7 +854,7 @@ op_status back_layer(opnet *net, int i, const float *X, const float *dZ, float *
     w.chunk = (int)(((points + want - 1) / want + kWP - 1) / kWP * kWP);
     splits = (int)((points + w.chunk - 1) / w.chunk);
     const int smem = bytes(w.ng);
-    OP_CUDA(cudaFuncSetAttribute(k_wgrad_pad, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    OP_CUDA(cudaFuncSetAttribute(k_wgrad_pad, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem));
     k_wgrad_pad<<<dim3((unsigned)gx, (unsigned)splits), threads, smem, st>>>(w);
   } else {
     long long chunk = 2048;
