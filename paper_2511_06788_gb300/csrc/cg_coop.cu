@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "sums.cuh"
 #include "tc.cuh"
 
 namespace opevo {
@@ -35,7 +36,7 @@ constexpr int kCoopThreads = 512;
 // here and 2.90 ms by kernels, 56^3 x 64 (45 MB) 3.43 and 3.54, 64^3 x 84 (92 MB) 8.9 and 7.7.
 // FP64: bound by the FP64 pipe either way: 64^3 x 64 (134 MB, the largest tried) 32.9 and 38.1.
 template <typename T> constexpr long long kCoopBytes = (sizeof(T) == 4 ? 48ll : 140ll) << 20;
-// Dynamic shared memory a launch may ask for (the largest any size below takes is 130 KB).  The
+// Dynamic shared memory a launch may ask for (the largest any size below takes is 140 KB).  The
 // limit belongs to the kernel on the device, so every call sets this one value: a limit of the
 // call's own size could be lowered by another thread's solve between setting it and the launch.
 constexpr int kCoopSmem = 224 * 1024;
@@ -76,26 +77,23 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Running sum across threads and CTAs.  FP64 blocks: a double.  FP32 blocks: an unevaluated pair
-// of floats (error-free two-sum, 48 bits): the terms are FP32 sums, and a warp's FP64 addition
-// takes 64 clocks of its scheduler on GB300, which made the reductions half of an iteration.
+// Running sum across threads and CTAs.  FP64 blocks: a double.  FP32 blocks: a triple of floats
+// (sums.cuh: with FP64 additions the reductions were half of an iteration).  A sum that leaves the
+// FP32 range is formed again in FP64 (`total` below) and held as the double's bits in h and m,
+// marked by l = NaN.  WIDE: the sums are such doubles.
 template <typename T> struct Sum;
-// Threads that share the sums of the columns: all of them for FP32 pairs, one warp a scheduler
+// Threads that share the sums of the columns: all of them for FP32 blocks, one warp a scheduler
 // for FP64 (its additions queue on the one FP64 pipe, and idle lanes cost as much as busy ones).
 template <typename T> constexpr int kSumThreads = sizeof(T) == 4 ? kCoopThreads : 128;
 template <> struct Sum<double> {
   double h = 0.0;
   __device__ __forceinline__ void add(double x) { h += x; }
   __device__ __forceinline__ void add(const Sum &o) { h += o.h; }
+  __device__ __forceinline__ bool finite() const { return true; }  // (nothing to form again)
   __device__ __forceinline__ double value() const { return h; }
-  __device__ __forceinline__ Sum down(int o) const {
+  __device__ __forceinline__ Sum over(int o) const {
     Sum s;
-    s.h = __shfl_down_sync(0xffffffffu, h, o);
-    return s;
-  }
-  __device__ __forceinline__ Sum from(int lane, int width) const {
-    Sum s;
-    s.h = __shfl_sync(0xffffffffu, h, lane, width);
+    s.h = __shfl_xor_sync(0xffffffffu, h, o);
     return s;
   }
   __device__ __forceinline__ static Sum load(const Sum *p) {
@@ -103,60 +101,71 @@ template <> struct Sum<double> {
     s.h = __ldcg(&p->h);
     return s;
   }
-  __device__ __forceinline__ static double ratio(const Sum &a, const Sum &b) { return a.h / b.h; }
-  __device__ __forceinline__ bool positive() const { return h > 0.0; }
+  // q = a / b, 0 where b <= 0; false: for WIDE
+  template <bool WIDE>
+  __device__ __forceinline__ static bool quotient(const Sum &a, const Sum &b, double *q) {
+    *q = b.h > 0.0 ? a.h / b.h : 0.0;
+    return true;
+  }
+  // 1 or 0: a sum of squares is above t or not (tf: t in the block's type); -1: for WIDE
+  template <bool WIDE> __device__ __forceinline__ int above(double t, double) const { return h > t; }
 };
-template <> struct __align__(8) Sum<float> {
-  float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
-    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
-    h = s;
-  }
-  __device__ __forceinline__ void add(const Sum &o) {
-    add(o.h);
-    l = __fadd_rn(l, o.l);
-  }
-  // (an overflowed sum has no low part)
-  __device__ __forceinline__ double value() const { return l == l ? (double)h + (double)l : (double)h; }
-  __device__ __forceinline__ Sum down(int o) const {
+template <> struct __align__(16) Sum<float> : Sum3 {
+  __device__ __forceinline__ static Sum of(double d) {
     Sum s;
-    s.h = __shfl_down_sync(0xffffffffu, h, o);
-    s.l = __shfl_down_sync(0xffffffffu, l, o);
+    s.h = __int_as_float(__double2loint(d));
+    s.m = __int_as_float(__double2hiint(d));
+    s.l = __int_as_float(0x7fffffff);
     return s;
   }
-  __device__ __forceinline__ Sum from(int lane, int width) const {
+  __device__ __forceinline__ double value() const {
+    return finite() ? Sum3::value() : __hiloint2double(__float_as_int(m), __float_as_int(h));
+  }
+  __device__ __forceinline__ Sum over(int o) const {
     Sum s;
-    s.h = __shfl_sync(0xffffffffu, h, lane, width);
-    s.l = __shfl_sync(0xffffffffu, l, lane, width);
+    s.h = __shfl_xor_sync(0xffffffffu, h, o);
+    s.m = __shfl_xor_sync(0xffffffffu, m, o);
+    s.l = __shfl_xor_sync(0xffffffffu, l, o);
     return s;
   }
   __device__ __forceinline__ static Sum load(const Sum *p) {
-    const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p));
     Sum s;
     s.h = v.x;
-    s.l = v.y;
+    s.m = v.y;
+    s.l = v.z;
     return s;
   }
-  // a / b to about 46 bits, rounded to FP32 (what the FP64 quotient rounds to)
-  __device__ __forceinline__ static float ratio(const Sum &a, const Sum &b) {
-    const float bh = b.h + b.l, bl = __fsub_rn(b.l, __fsub_rn(bh, b.h));
-    const float q = a.h / bh;
-    const float r = fmaf(-q, bh, a.h) + fmaf(-q, bl, a.l);
-    const float c = r / bh;
-    return c == c ? q + c : q;
+  template <bool WIDE>
+  __device__ __forceinline__ static bool quotient(const Sum &a, const Sum &b, float *q) {
+    if constexpr (WIDE) {
+      const double d = b.value();
+      *q = d > 0.0 ? (float)(a.value() / d) : 0.f;
+      return true;
+    }
+    return opevo::quotient(a, b, q);
   }
-  __device__ __forceinline__ bool positive() const { return h + l > 0.f; }
+  // (the FP32 parts decide unless they are within 2^-12: a sum of n squares has |m| < n 2^-24 h)
+  template <bool WIDE> __device__ __forceinline__ int above(double t, float tf) const {
+    if constexpr (WIDE) return value() > t;
+    if (!(tf < 1e30f)) return -1;
+    if (h > fmaxf(tf, 1e-30f) * 1.000245f) return 1;
+    return tf > 1e-30f && h < tf * 0.999755f ? 0 : -1;
+  }
 };
 
 // v into CTA `rank`'s copy of the shared-memory slot p.
 template <typename S> __device__ __forceinline__ void store_cluster(S *p, int rank, const S &v) {
   uint32_t a;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(tc::smem_u32(p)), "r"(rank));
-  unsigned long long bits;
-  static_assert(sizeof(S) == 8, "one 8-byte store");
-  memcpy(&bits, &v, 8);
-  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(bits) : "memory");
+  unsigned long long bits[2] = {0, 0};
+  static_assert(sizeof(S) == 8 || sizeof(S) == 16, "one store");
+  memcpy(bits, &v, sizeof(S));
+  if constexpr (sizeof(S) == 8)
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(bits[0]) : "memory");
+  else
+    asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(a), "l"(bits[0]), "l"(bits[1])
+                 : "memory");
 }
 
 struct CoopArgs {
@@ -212,13 +221,16 @@ __device__ __forceinline__ Pack<T> stencil_sum(const Geom &g, int i, int ld, T d
   return y;
 }
 
+// Sums of the CTAs' partials in shared memory: at most 512 or one row of 3 ld, at an odd pitch.
+__host__ __device__ constexpr int tot_len(int ld) { return kCoopThreads + 3 * ld + 64; }
+
 // L: neighbouring lanes that reduce one column
 template <typename T, bool JAC, int L>
 __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
   constexpr int N = Pack<T>::N;
   constexpr bool kFused = std::is_same<T, float>::value;
   extern __shared__ __align__(16) double sm[];
-  __shared__ int ok_sh, nact_sh;
+  __shared__ int ok_sh, nact_sh, wide_sh;
   const Geom &g = A.g;
   const int ld = A.ld, nv = ld / N, nr = kCoopThreads / nv;
   const int tx = threadIdx.x % nv, ty = threadIdx.x / nv;
@@ -231,16 +243,16 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
   T *W = (T *)A.W, *R = (T *)A.R;
   const T shift = (T)A.shift;
   // shared memory: per-column state, 1 / diag of the CTA's points, the cluster's partials
-  // [2][CTA][3 ld], the threads' sums
+  // [2][CTA][3 ld] (odd pitch), sums of the CTAs' partials, the threads' sums
   using S = Sum<T>;
   double *target = sm;
   S *rho = reinterpret_cast<S *>(target + ld);
-  T *al = reinterpret_cast<T *>(rho + ld), *be = al + ld;
-  int *act = reinterpret_cast<int *>(be + ld);
-  T *inv_sh = reinterpret_cast<T *>(act + ld);
+  T *al = reinterpret_cast<T *>(rho + ld), *be = al + ld, *target_t = be + ld;
+  int *act = reinterpret_cast<int *>(target_t + ld), *wide = act + ld;
+  T *inv_sh = reinterpret_cast<T *>(wide + ld);
   S *xch = reinterpret_cast<S *>(inv_sh + A.inv_rows);
-  T *rows = reinterpret_cast<T *>(xch + (A.cluster ? 6 * G * ld : 0));
-  S *tot = reinterpret_cast<S *>(rows);  // (the threads' sums are read before)
+  S *tot = xch + (A.cluster ? 2 * G * (3 * ld + 1) : 0);
+  T *rows = reinterpret_cast<T *>(tot + tot_len(ld));
   constexpr int jstep = kCoopThreads / L;
   const int lane = threadIdx.x & (L - 1);
   const int jw = (int)(threadIdx.x & ~31u) / L, jl = (int)(threadIdx.x & 31) / L;
@@ -269,11 +281,13 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
   };
 
   // Totals over the grid of the per-thread sums acc[c][k] (column col + k): over the CTA's rows,
-  // then over the CTAs, in the same order in every CTA; one lane a column gets fin(j, sums).
-  // A cluster's partials go straight into every member's shared memory.
+  // then over the CTAs, in the same order in every CTA; one lane a column gets fin(j, sums, WIDE).
+  // A cluster's partials go straight into every member's shared memory.  A column that fin refuses
+  // (a sum outside the FP32 range, or a quotient or comparison that takes FP64: rare) is summed
+  // again in FP64 from the threads' sums: every CTA has the same partials, so all refuse alike.
   auto total = [&](auto &acc, auto &&fin) -> bool {
     constexpr int NC = sizeof(acc) / sizeof(acc[0]);
-    const int w = NC * ld, pitch = w | 1;
+    const int w = NC * ld, pitch = w | 1, pm = w | 1;
     __syncthreads();
     if (ty < nra) {
 #pragma unroll
@@ -282,9 +296,12 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
         for (int k = 0; k < N; ++k) rows[ty * pitch + c * ld + col + k] = acc[c][k];
     }
     __syncthreads();
+    auto last = [&](int j, S *s) {
+      if (!fin(j, s, std::false_type{})) wide[j] = wide_sh = 1;
+    };
     // alternate buffers: a CTA may still read the last totals' partials
     S *part = reinterpret_cast<S *>(A.part) + odd * 3 * G * ld;
-    S *mine = xch + odd * 3 * G * ld;
+    S *mine = xch + odd * G * (3 * ld + 1);
     odd ^= 1;
     for (int jb = jw; jb < ld; jb += jstep) {  // (whole warps)
       const int j = jb + jl;
@@ -297,17 +314,15 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
 #pragma unroll
       for (int o = L >> 1; o > 0; o >>= 1)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) s[c].add(s[c].down(o));
+        for (int c = 0; c < NC; ++c) s[c].add(s[c].over(o));
+      if (j >= ld) continue;
       if (G == 1) {
-        if (lane == 0 && j < ld) fin(j, s);
+        if (lane == 0) last(j, s);
       } else if (A.cluster) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const S v = s[c].from(0, L);
-          if (j < ld)
-            for (int r = lane; r < G; r += L) store_cluster(mine + blockIdx.x * w + c * ld + j, r, v);
-        }
-      } else if (lane == 0 && j < ld) {
+        for (int c = 0; c < NC; ++c)
+          for (int r = lane; r < G; r += L) store_cluster(mine + blockIdx.x * pm + c * ld + j, r, s[c]);
+      } else if (lane == 0) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) part[blockIdx.x * w + c * ld + j] = s[c];
       }
@@ -317,16 +332,15 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
       // the CTAs' partials: a cluster's are here; a grid's come from L2 as whole lines, summed
       // in `gg` interleaved groups first
       const S *from = mine;
-      int terms = G, pitch2 = w;
+      int terms = G;
       if (!A.cluster) {
         const int gg = max(1, min(G, max(kSumThreads<T>, min(kCoopThreads, 4 * w)) / w));
-        pitch2 = w | 1;
         for (int t = threadIdx.x; t < gg * w; t += kCoopThreads) {
           const int q = t / w, e = t - q * w;
           S s;
 #pragma unroll 8
           for (int b = q; b < G; b += gg) s.add(S::load(part + b * w + e));
-          tot[q * pitch2 + e] = s;
+          tot[q * pm + e] = s;
         }
         __syncthreads();
         from = tot;
@@ -339,17 +353,63 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
 #pragma unroll 4
           for (int b = lane; b < terms; b += L)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) s[c].add(from[b * pitch2 + c * ld + j]);
+            for (int c = 0; c < NC; ++c) s[c].add(from[b * pm + c * ld + j]);
 #pragma unroll
         for (int o = L >> 1; o > 0; o >>= 1)
 #pragma unroll
-          for (int c = 0; c < NC; ++c) s[c].add(s[c].down(o));
-        if (lane == 0 && j < ld) fin(j, s);
+          for (int c = 0; c < NC; ++c) s[c].add(s[c].over(o));
+        if (lane == 0 && j < ld) last(j, s);
       }
     }
     __syncthreads();
+    if constexpr (kFused) {
+      if (wide_sh) {
+        part = reinterpret_cast<S *>(A.part) + odd * 3 * G * ld;
+        mine = xch + odd * G * (3 * ld + 1);
+        odd ^= 1;
+#pragma unroll 1
+        for (int e = threadIdx.x; e < w; e += kCoopThreads) {
+          double d = 0.0;
+#pragma unroll 1
+          for (int y = 0; y < nra; ++y) d += (double)rows[y * pitch + e];
+          const S v = S::of(d);
+          if (G == 1) {
+            tot[e] = v;
+          } else if (A.cluster) {
+#pragma unroll 1
+            for (int r = 0; r < G; ++r) store_cluster(mine + blockIdx.x * pm + e, r, v);
+          } else {
+            part[blockIdx.x * w + e] = v;
+          }
+        }
+        if (G > 1) {
+          if (!meet()) return false;
+#pragma unroll 1
+          for (int e = threadIdx.x; e < w; e += kCoopThreads) {
+            double d = 0.0;
+#pragma unroll 1
+            for (int b = 0; b < G; ++b)
+              d += (A.cluster ? mine[b * pm + e] : S::load(part + b * w + e)).value();
+            tot[e] = S::of(d);
+          }
+        }
+        __syncthreads();
+        for (int j = threadIdx.x; j < ld; j += kCoopThreads)
+          if (wide[j]) {
+            S s[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s[c] = tot[c * ld + j];
+            fin(j, s, std::true_type{});
+            wide[j] = 0;
+          }
+        if (threadIdx.x == 0) wide_sh = 0;
+        __syncthreads();
+      }
+    }
     return true;
   };
+  for (int j = threadIdx.x; j < ld; j += kCoopThreads) wide[j] = 0;
+  if (threadIdx.x == 0) wide_sh = 0;
   if (A.cluster) cluster_barrier();  // every member runs before its shared memory is written
 
   // start: R = U - (H + sigma) W (Z = R / d with the Jacobi preconditioner); FP64: P = R
@@ -376,14 +436,17 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
         if (!kFused) r.store((T *)A.P + o);
       }
     if (threadIdx.x == 0) nact_sh = 0;
-    ok = total(acc, [&](int j, S (&s)[3]) {
+    ok = total(acc, [&](int j, S *s, auto wd) {
+      if (!decltype(wd)::value && !(s[0].finite() && s[1].finite() && s[2].finite())) return false;
       const double bb = s[1].value();
       rho[j] = s[0];
       target[j] = A.rtol2 * bb;
+      target_t[j] = (T)target[j];
       al[j] = be[j] = T(0);
       const int a = (j < A.p) && (s[2].value() > A.rtol2 * bb) && (bb > 0.0);
       act[j] = a;
       if (a) atomicAdd(&nact_sh, 1);
+      return true;
     });
   }
   int it = 0;
@@ -425,8 +488,11 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
           for (int k = 0; k < N; ++k) acc[0][k] += pc.v[k] * q.v[k];
         }
       }
-      ok = total(acc, [&](int j, S (&s)[1]) {
-        al[j] = (act[j] && s[0].positive()) ? (T)S::ratio(rho[j], s[0]) : T(0);
+      ok = total(acc, [&](int j, S *s, auto wd) {
+        T q = T(0);
+        if (act[j] && !S::template quotient<decltype(wd)::value>(rho[j], s[0], &q)) return false;
+        al[j] = q;
+        return true;
       });
       if (!ok) break;
       if (threadIdx.x == 0) nact_sh = 0;  // (every thread has read it for this iteration)
@@ -465,15 +531,18 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(const CoopArgs A) {
           r.store(R + o);
         }
       }
-      ok = total(acc, [&](int j, S (&s)[NC]) {
-        int a = act[j];
-        be[j] = (a && rho[j].positive()) ? (T)S::ratio(s[0], rho[j]) : T(0);
-        if (a) {
+      ok = total(acc, [&](int j, S *s, auto wd) {
+        constexpr bool kWide = decltype(wd)::value;
+        T q = T(0);
+        if (act[j]) {
+          const int a = s[NC - 1].template above<kWide>(target[j], target_t[j]);
+          if (a < 0 || !S::template quotient<kWide>(s[0], rho[j], &q)) return false;
           rho[j] = s[0];
-          a = s[NC - 1].value() > target[j];
           act[j] = a;
+          if (a) atomicAdd(&nact_sh, 1);
         }
-        if (a) atomicAdd(&nact_sh, 1);
+        be[j] = q;
+        return true;
       });
       if (!ok) break;
       ++it;
@@ -551,17 +620,18 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
   a.ld = ld;
   a.max_iter = max_iter;
   a.rows_per_cta = rows;
-  a.inv_rows = w.jacobi && rows <= 8192 ? (rows + 1) / 2 * 2 : 0;  // (8-byte alignment after it)
+  a.inv_rows = w.jacobi && rows <= 8192 ? (rows + 3) / 4 * 4 : 0;  // (16-byte alignment after it)
   a.rtol2 = rtol * rtol;
   a.shift = g.cdiag + sigma;
   a.part = w.part;
   a.ctl = w.ctl;
   a.cluster = cluster;
   // as laid out in the kernel; the threads' sums have an odd pitch
-  const size_t smem = (size_t)ld * (2 * sizeof(double) + 2 * sizeof(T) + sizeof(int)) +
-                      (size_t)a.inv_rows * sizeof(T) + (cluster ? (size_t)6 * G * ld * 8 : 0) +
-                      std::max(((size_t)kCoopThreads * N * 3 + kCoopThreads / (ld / N) + 1) * sizeof(T),
-                               (size_t)(2 * kCoopThreads + 3 * ld + 2) * 8);
+  const size_t sum = sizeof(Sum<T>);
+  const size_t smem = (size_t)ld * (sizeof(double) + sum + 3 * sizeof(T) + 2 * sizeof(int)) +
+                      (size_t)a.inv_rows * sizeof(T) +
+                      (cluster ? (size_t)2 * G * (3 * ld + 1) * sum : 0) + tot_len(ld) * sum +
+                      ((size_t)kCoopThreads * N * 3 + kCoopThreads / (ld / N) + 1) * sizeof(T);
   OP_CUDA(cudaMemsetAsync(w.ctl, 0, 256, st));
   void *args[] = {&a};
   int lanes = 1;

@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "sums.cuh"
 
 namespace opevo {
 
@@ -221,10 +222,9 @@ __global__ void k_tri_cols(int p, int ld, const double *__restrict__ L, int mode
   for (int i = t; i < ld; i += nt) out[(long long)i * ld + j] = (i < p) ? y[i] : 0.0;
 }
 
-// FP64 <-> FP32 on the integer pipe: the conversion instructions run at the FP64 rate, 2 a clock
-// and SM, so the 2 x 16384 of one CTA's 128 x 128 block took 10 us of k_gj32.  narrow rounds to
-// nearest even and widen is exact, both as the instructions do, which take what is not zero or
-// normal in FP32.
+// FP64 to FP32 on the integer pipe: the conversion instructions run at the FP64 rate, 2 a clock
+// and SM, so the 2 x 16384 of one CTA's 128 x 128 block (back by widen) took 10 us of k_gj32.
+// Rounds to nearest even, as the instruction does, which takes what is not zero or normal in FP32.
 __device__ __forceinline__ float narrow(double x) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const unsigned long long m = u & 0x7fffffffffffffffull;
@@ -234,12 +234,6 @@ __device__ __forceinline__ float narrow(double x) {
   if (e - 897u > 253u) return (float)x;
   const unsigned long long r = m + 0x0fffffffull + ((m >> 29) & 1);
   return __uint_as_float(((unsigned)(r >> 29) - (896u << 23)) | sign);
-}
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
-  if (m == 0) return __hiloint2double((int)u, 0);
-  if ((m >> 23) - 1u > 253u) return (double)x;
-  return __hiloint2double((int)(((m >> 3) + (896u << 20)) | (u & 0x80000000u)), (int)(m << 29));
 }
 
 // Inverse of the p x p matrix M (stride ld, p <= 128) in FP32 by blocked Gauss-Jordan
