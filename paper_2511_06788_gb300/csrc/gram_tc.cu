@@ -28,6 +28,7 @@
 // clocks beside the staging: both load shared memory).
 #include "common.cuh"
 #include "kernels.cuh"
+#include "sums.cuh"
 #include "tc.cuh"
 
 namespace opevo {
@@ -544,35 +545,23 @@ __global__ void __launch_bounds__(256, 1)
                  three != 0);
 }
 
-// A running sum of partials: FP32 ones as an error-free pair of floats (two-sum; the FP64 pipe
-// would take longer than reading them), or FP64.
+// A running sum of partials: FP32 ones as a triple of floats (sums.cuh; the FP64 pipe would take
+// longer than reading them), or FP64.
 template <typename P> struct SplitSum;
-template <> struct SplitSum<float> {
-  float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(h, v), b = __fsub_rn(s, h);
-    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b)));
-    h = s;
-  }
-  __device__ __forceinline__ void merge(const SplitSum &o) {
-    add(o.h);
-    l = __fadd_rn(l, o.l);
-  }
-  __device__ __forceinline__ double value() const {
-    return l == l ? (double)h + (double)l : (double)h;  // (an overflowed sum has no low part)
-  }
-};
+template <> struct SplitSum<float> : Sum3 {};
 template <> struct SplitSum<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
-  __device__ __forceinline__ void merge(const SplitSum &o) { s += o.s; }
+  __device__ __forceinline__ void add(const SplitSum &o) { s += o.s; }
+  __device__ __forceinline__ bool finite() const { return true; }  // (nothing to add again)
   __device__ __forceinline__ double value() const { return s; }
 };
 
 // out(i, j) = the summed tile element, zero outside p x p, both triangles of S and D.
 // A CTA of kRedLanes x kRedGroups threads: group g sums every kRedGroups-th split, the first
 // group adds the sums up.  One thread per element and all its splits was a serial chain of up to
-// 228 loads and two-sums: 24 us at 262144 x 128, now 13.
+// 228 loads and two-sums: 24 us at 262144 x 128, now 13.  An element whose sum leaves the FP32 range
+// is summed in FP64.
 template <typename P>
 __device__ __forceinline__ void reduce_tile(int prod, int ti, int tj, int slice, int slices,
                                             const P *part, long long stride, int nsplit, int p,
@@ -590,8 +579,12 @@ __device__ __forceinline__ void reduce_tile(int prod, int ti, int tj, int slice,
     __syncthreads();
     if (g == 0 && i < ld && j < ld) {
 #pragma unroll
-      for (int q = 0; q < kRedGroups - 1; ++q) s.merge(sh[q][lane]);
-      const double v = (i < p && j < p) ? s.value() : 0.0;
+      for (int q = 0; q < kRedGroups - 1; ++q) s.add(sh[q][lane]);
+      double v = (i < p && j < p) ? s.value() : 0.0;
+      if (!s.finite()) {
+        v = 0.0;
+        for (int sp = 0; sp < nsplit; ++sp) v += (double)part[e + sp * stride];
+      }
       out[(long long)i * ld + j] = v;
       if (prod != PROD_C && ti != tj) out[(long long)j * ld + i] = v;
     }
