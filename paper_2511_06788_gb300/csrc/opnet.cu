@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "opnet.h"
+#include "sums.cuh"
 
 namespace opevo {
 namespace {
@@ -424,33 +425,29 @@ __global__ void k_wgrad_copy(int N, int C, const float *__restrict__ X, float *_
 }
 
 // out[e] = sum_s part[s][e] (fixed order): blocks of 32 elements by 16 interleaved sums over the
-// splits, each an error-free pair of floats (two-sum, 48 bits; a warp's FP64 conversion and
-// addition take 64 clocks each), joined in FP64.  The 11 layers at 48^3: 467 us with one FP64 sum
-// an element, 293 us so (cold).
+// splits, each a triple of floats (sums.cuh; a warp's FP64 conversion and addition take 64 clocks
+// each), joined as they are; in FP64 where a sum leaves the FP32 range.  The 11 layers at 48^3:
+// 467 us with one FP64 sum an element, 293 us with pairs of floats joined in FP64 (cold); the loss and
+// gradient there 3.81 ms with the latter, 3.71 so.
 __global__ void __launch_bounds__(512) k_reduce_parts(const float *__restrict__ part, int splits,
                                                       long long count, float *__restrict__ out) {
-  __shared__ float2 red[16][33];
+  __shared__ Sum3 red[16][33];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   for (long long e0 = blockIdx.x * 32ll; e0 < count; e0 += gridDim.x * 32ll) {
     const long long e = e0 + x;
-    float h = 0.f, l = 0.f;
+    Sum3 t;
     if (e < count)
 #pragma unroll 8
-      for (int k = y; k < splits; k += 16) {
-        const float v = part[(long long)k * count + e];
-        const float s = __fadd_rn(h, v), b = __fsub_rn(s, h);
-        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b)));
-        h = s;
-      }
-    red[y][x] = make_float2(h, l);
+      for (int k = y; k < splits; k += 16) t.add(part[(long long)k * count + e]);
+    red[y][x] = t;
     __syncthreads();
     if (y == 0 && e < count) {
-      // (an overflowed sum has no low part)
-      double s = 0.0;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float2 v = red[j][x];
-        s += v.y == v.y ? (double)v.x + (double)v.y : (double)v.x;
+      for (int j = 1; j < 16; ++j) t.add(red[j][x]);
+      double s = t.value();
+      if (!t.finite()) {
+        s = 0.0;
+        for (int k = 0; k < splits; ++k) s += (double)part[(long long)k * count + e];
       }
       out[e] = (float)s;
     }
