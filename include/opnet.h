@@ -108,7 +108,9 @@ op_status opnet_set_conv(opnet *net, int kind);
  * the parameter layout above), bias [cout] or NULL, Z and A [N^3][cout] (either may be
  * NULL), all FP32 device arrays; taps 27 (3x3x3, zero padded) or 1; 1 <= cout <= 128,
  * cin <= 512, N <= 512; X 16-byte aligned.  `kind` as opnet_set_conv.  Allocates and
- * frees a small scratch and synchronises `stream` (cudaStream_t, may be NULL). */
+ * frees scratch (OPNET_CONV_BF16_TC: the weights and a copy of X in BF16, at most 8 GiB;
+ * the weights alone where the copy does not fit, same result) and synchronises `stream`
+ * (cudaStream_t, may be NULL). */
 op_status opnet_conv(int kind, const float *X, int N, int taps, int cin, int cout,
                      const float *W, const float *bias, float *Z, float *A, void *stream);
 
@@ -119,7 +121,7 @@ op_status opnet_conv(int kind, const float *X, int N, int taps, int cin, int cou
  * dZ [N^3][cout] (16-byte aligned), W [taps * cin][cout], dX [N^3][cin], FP32 device
  * arrays; taps 27 or 1; cin, cout <= 512, N <= 512.  OPNET_CONV_BF16_TC: on the tensor
  * cores (BF16 dZ and W, FP32 accumulation) when cin <= 128, else as OPNET_CONV_FP32 (FP32
- * CUDA cores).  Allocates and frees a small scratch and synchronises `stream`. */
+ * CUDA cores).  Allocates and frees scratch as opnet_conv and synchronises `stream`. */
 op_status opnet_conv_dgrad(int kind, const float *dZ, int N, int taps, int cin, int cout,
                            const float *W, float *dX, void *stream);
 

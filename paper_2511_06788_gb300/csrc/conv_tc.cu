@@ -25,7 +25,7 @@
 // The 11 layers at 48^3, widths 24, 48, 96, p = 64: 0.39 ms and 0.12 ms for the BF16 copies; one
 // CTA a tile and a box per tap 0.51 and 0.10, by k_conv_tc 1.37 ms.
 //
-// k_conv_tc (other layers).  K in slabs of 64; the 256 threads gather a slab of A from FP32 (27
+// k_conv_tc (other layers, and scratch without room for the copy).  K in slabs of 64; the 256 threads gather a slab of A from FP32 (27
 // taps, zero padding) and convert it, one thread issues the slab's MMAs; the gather of slab
 // s + 1 runs while the tensor core works on slab s.
 //
@@ -627,6 +627,7 @@ size_t weight_bytes(int taps, int cin, int cout) {
 
 }  // namespace
 
+size_t conv_tc_scratch_min(int taps, int cin, int cout) { return weight_bytes(taps, cin, cout); }
 size_t conv_tc_scratch_bytes(int N, int taps, int cin, int cout) {
   return weight_bytes(taps, cin, cout) +
          (size_t)copy_rows(N, taps, cin) * copy_len(N, taps, cin) * 2;
@@ -636,7 +637,7 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
                        const float *bias, float *Z, float *A, void *scratch, size_t scratch_bytes,
                        int *err, cudaStream_t st) {
   if (!X || !W || !scratch || !err || N < 1 || (taps != 1 && taps != 27) || cin < 1 ||
-      cout < 1 || cout > 128 || scratch_bytes < conv_tc_scratch_bytes(N, taps, cin, cout) ||
+      cout < 1 || cout > 128 || scratch_bytes < conv_tc_scratch_min(taps, cin, cout) ||
       ((uintptr_t)scratch & 15) != 0) {
     set_error("conv_bf16_tc: bad arguments (N=%d taps=%d cin=%d cout=%d)", N, taps, cin, cout);
     return OP_ERR_ARG;
@@ -647,8 +648,8 @@ op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const
   }
   const int K = taps * cin, coutp = (cout + 15) / 16 * 16, Kp = (K + kCK - 1) / kCK * kCK;
   const int clen = copy_len(N, taps, cin);
-  if (clen > 0 && (!Z || ((uintptr_t)Z & 15) == 0) &&
-      (!A || ((uintptr_t)A & 15) == 0)) {
+  if (clen > 0 && scratch_bytes >= conv_tc_scratch_bytes(N, taps, cin, cout) &&
+      (!Z || ((uintptr_t)Z & 15) == 0) && (!A || ((uintptr_t)A & 15) == 0)) {
     uint16_t *Wt = (uint16_t *)scratch;
     uint16_t *Xb = (uint16_t *)((char *)scratch + weight_bytes(taps, cin, cout));
     const int gcin = cin % 8 == 0 ? 0 : cin, pad = taps == 27 && !gcin ? 1 : 0;

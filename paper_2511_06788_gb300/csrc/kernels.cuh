@@ -179,9 +179,11 @@ op_status refine_residual(const Geom &g, const double *Vt, double sigma, const d
 // [N^3][cin] FP32, W [taps * cin][cout] FP32 (taps 27: the 3x3x3 cross-correlation, zero
 // padded; taps 1: pointwise), BF16 operands with FP32 accumulation; Z = conv + bias and
 // A = silu(Z) ([N^3][cout] FP32, either may be null).  cout <= 128.  scratch: device memory
-// of conv_tc_scratch_bytes (the BF16 weights, K-major, and a BF16 copy of X), 256-byte aligned;
-// *err is set when a bounded wait of the kernel gives up.
+// of conv_tc_scratch_bytes (the BF16 weights, K-major, and a BF16 copy of X), 256-byte aligned; with
+// less, down to conv_tc_scratch_min (the weights), the kernel that needs no copy runs (the same
+// bits).  *err is set when a bounded wait of the kernel gives up.
 size_t conv_tc_scratch_bytes(int N, int taps, int cin, int cout);
+size_t conv_tc_scratch_min(int taps, int cin, int cout);
 op_status conv_bf16_tc(const float *X, int N, int taps, int cin, int cout, const float *W,
                        const float *bias, float *Z, float *A, void *scratch, size_t scratch_bytes,
                        int *err, cudaStream_t st);

@@ -645,7 +645,8 @@ struct opnet {
   opnet_config cfg;
   int N, p, c0, c1, c2;
   int conv_kind;         // OPNET_CONV_*: the forward convolutions' arithmetic
-  void *conv_ws;         // BF16 weights of the tensor-core convolution (one layer at a time)
+  void *conv_ws;         // BF16 weights and input copy of the tensor-core convolution (one layer
+                         // at a time), or the weights alone where the copy does not fit
   size_t conv_ws_bytes;
   int *dev_err;          // set when a bounded wait of a tensor-core kernel gives up
   long long n0, n1, n2;  // points at the three levels
@@ -769,7 +770,8 @@ op_status forward(opnet *net, const double *V) {
 // (k_flip into Wf, taps * cin * cout floats of scratch).  OPNET_CONV_BF16_TC runs it on the
 // tensor cores when cin <= 128 (the kernel's output-channel limit; BF16 operands, FP32
 // accumulation), otherwise it runs on the FP32 CUDA cores.  tc_ws: scratch of
-// conv_tc_scratch_bytes(N, taps, cout, cin) bytes for the tensor-core form.
+// conv_tc_scratch_bytes(N, taps, cout, cin) bytes for the tensor-core form (or of
+// conv_tc_scratch_min; none for the other one).
 op_status conv_dgrad(int kind, const float *dZ, int N, int taps, int cin, int cout,
                      const float *W, float *Wf, float *dX, void *tc_ws, size_t tc_bytes, int *err,
                      cudaStream_t st) {
@@ -969,6 +971,19 @@ op_status read_loss(opnet *net, double *out) {
   return OP_OK;
 }
 
+// Device scratch of a single-layer call: `head` bytes, *conv bytes for the convolution and 256 for its
+// error word; without room for all of it *conv = least.
+op_status layer_scratch(void **ws, size_t head, size_t *conv, size_t least) {
+  cudaError_t e = cudaMalloc(ws, head + *conv + 256);
+  if (e == cudaErrorMemoryAllocation && least < *conv) {
+    (void)cudaGetLastError();
+    *conv = least;
+    e = cudaMalloc(ws, head + *conv + 256);
+  }
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e == cudaSuccess ? OP_OK : cuda_status(e, "scratch of a convolution");
+}
+
 bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 
 }  // namespace
@@ -1072,19 +1087,27 @@ op_status opnet_create(opnet **out, const opnet_config *cfg) {
     s = net_alloc(net, &net->gram_ws, net->gram_bytes);
   }
   if (s == OP_OK) {
-    // the tensor-core convolutions (the default): scratch for the widest layer's weights
+    // the tensor-core convolutions (the default): scratch for the largest layer
     net->conv_kind = OPNET_CONV_BF16_TC;
     net->conv_ws_bytes = 0;
+    size_t least = 0;
     for (int i = 0; i < kLayers; ++i) {
       const Layer &l = net->L[i];
       net->conv_ws_bytes =
           std::max(net->conv_ws_bytes, conv_tc_scratch_bytes(l.grid, l.taps, l.cin, l.cout));
+      least = std::max(least, conv_tc_scratch_min(l.taps, l.cin, l.cout));
       // the tensor-core data gradient: the same kernel with cin and cout exchanged
-      if (l.cin <= 128)
+      if (l.cin <= 128) {
         net->conv_ws_bytes =
             std::max(net->conv_ws_bytes, conv_tc_scratch_bytes(l.grid, l.taps, l.cout, l.cin));
+        least = std::max(least, conv_tc_scratch_min(l.taps, l.cout, l.cin));
+      }
     }
     s = net_alloc(net, &net->conv_ws, net->conv_ws_bytes);
+    if (s == OP_ERR_OOM) {
+      net->conv_ws_bytes = least;
+      s = net_alloc(net, &net->conv_ws, least);
+    }
   }
   if (s == OP_OK) {
     const cudaError_t e = cudaMemsetAsync(net->dev_err, 0, 4 * sizeof(int), net->st);
@@ -1202,9 +1225,9 @@ op_status opnet_conv(int kind, const float *X, int N, int taps, int cin, int cou
     OP_CUDA(cudaStreamSynchronize(st));
     return OP_OK;
   }
-  const size_t wb = conv_tc_scratch_bytes(N, taps, cin, cout);
+  size_t wb = conv_tc_scratch_bytes(N, taps, cin, cout);
   void *ws = nullptr;
-  OP_CUDA(cudaMalloc(&ws, wb + 256));
+  OP_TRY(layer_scratch(&ws, 0, &wb, conv_tc_scratch_min(taps, cin, cout)));
   int *err = (int *)((char *)ws + wb);
   auto ck = [](cudaError_t e, const char *what) {
     return e == cudaSuccess ? OP_OK : cuda_status(e, what);
@@ -1232,9 +1255,10 @@ op_status opnet_conv_dgrad(int kind, const float *dZ, int N, int taps, int cin, 
   }
   cudaStream_t st = (cudaStream_t)stream;
   const size_t wf = ((size_t)taps * cin * cout * sizeof(float) + 255) / 256 * 256;
-  const size_t wb = conv_tc_scratch_bytes(N, taps, cout, cin);
+  const bool tensor = kind == OPNET_CONV_BF16_TC && cin <= 128;  // (as conv_dgrad decides)
+  size_t wb = tensor ? conv_tc_scratch_bytes(N, taps, cout, cin) : 0;
   void *ws = nullptr;
-  OP_CUDA(cudaMalloc(&ws, wf + wb + 256));
+  OP_TRY(layer_scratch(&ws, wf, &wb, tensor ? conv_tc_scratch_min(taps, cout, cin) : 0));
   float *Wf = (float *)ws;
   void *tc = (char *)ws + wf;
   int *err = (int *)((char *)ws + wf + wb);
