@@ -45,7 +45,8 @@ constexpr int kBarrierPolls = 1 << 23;
 // ctl words (256 bytes): 2 iterations, 3 error, 32 the barrier's arrivals
 constexpr int kCtlBar = 32;
 
-// Grid-wide barrier: `target` is the number of arrivals that completes it.  False when the
+// Grid-wide barrier: `target` is the number of arrivals (mod 2^32: some 10^7 iterations of a full
+// grid) that completes it.  False when the
 // wait gave up (the error word is set and every CTA gives up in turn).
 __device__ __forceinline__ bool grid_barrier(int *ctl, unsigned target, int *ok_sh) {
   __syncthreads();
@@ -58,7 +59,7 @@ __device__ __forceinline__ bool grid_barrier(int *ctl, unsigned target, int *ok_
     for (;;) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-      if (v >= target) break;
+      if (count_reached(v, target)) break;
       if (--left == 0) {
         atomicExch(ctl + 3, 1);
         ok = 0;

@@ -138,6 +138,12 @@ struct NvtxRange {
   NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// Whether a 32-bit counter of arrivals has come to `target`; the counter may have wrapped since (it
+// is never 2^31 or more past or before a target that is waited for).
+__host__ __device__ inline bool count_reached(unsigned count, unsigned target) {
+  return (int)(count - target) >= 0;
+}
+
 inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 
 }  // namespace opevo
