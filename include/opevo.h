@@ -321,6 +321,14 @@ op_status op_restore(op_ctx *ctx, const void *buf, size_t len);
  * a second. */
 op_status op_selftest_bounded_waits(double *seconds, void *stream);
 
+/* Self-test of Step 1's kernels: op_cg_solve by a route that its rule takes for other
+ * sizes.  route 1: the general kernels (a launch per pass), whatever the block's size;
+ * 2: as where the device cannot hold the cooperative launch's CTAs together, so that the
+ * general kernels take over.  The other arguments as op_cg_solve's. */
+op_status op_selftest_cg(int route, const op_problem *pb, int ld, const void *V_t, double sigma,
+                         const void *U, void *W, double rtol, int max_iter, void *ws,
+                         size_t ws_bytes, int *iters, void *stream);
+
 /* Peak-rate microbenchmarks (the paper has no counterpart): the roofline denominators of
  * the units the kernels are bound by, measured by this library on the current device
  * without reading or changing any GPU setting.  OP_PEAK_FP64_FMA: FP64 FMA on the CUDA

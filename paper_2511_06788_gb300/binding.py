@@ -127,6 +127,7 @@ def lib():
         "op_ws_status": (i32, [vp, vp]),
         "op_get_U_device": (i32, [vp, vp, i32]),
         "op_selftest_bounded_waits": (i32, [P(f64), vp]),
+        "op_selftest_cg": (i32, [i32, P(OpProblem), i32, vp, f64, vp, vp, f64, i32, vp, sz, P(i32), vp]),
         "op_peak_rate": (i32, [i32, P(f64), vp]),
         "op_checkpoint_size": (sz, [vp]),
         "op_checkpoint": (i32, [vp, vp, sz]),
@@ -734,3 +735,19 @@ def selftest_bounded_waits(stream=None):
     secs = (C.c_double * 2)()
     check(lib().op_selftest_bounded_waits(secs, _stream_ptr(stream)))
     return secs[0], secs[1]
+
+
+def selftest_cg(route, shape, lo, hi, V_t, sigma, U, W, p, rtol, max_iter=5000, stream=None,
+                precond="none"):
+    """cg_solve by a given route (op_selftest_cg): 1 the general kernels, 2 as where the
+    cooperative launch is refused."""
+    import torch
+    ld = U.shape[1]
+    pb = make_problem(shape, lo, hi, p, prec=_prec_of(U), precond=precond)
+    nbytes = lib().op_cg_workspace(C.byref(pb), ld)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=U.device)
+    it = C.c_int()
+    check(lib().op_selftest_cg(int(route), C.byref(pb), ld, _tptr(V_t), float(sigma), _tptr(U),
+                               _tptr(W), float(rtol), int(max_iter), _tptr(ws), nbytes,
+                               C.byref(it), _stream_ptr(stream)))
+    return it.value

@@ -1147,9 +1147,9 @@ size_t op_cg_workspace(const op_problem *pb, int ld) {
   return cg_workspace_bytes(g.n, ld, elem) + 64;
 }
 
-op_status op_cg_solve(const op_problem *pb, int ld, const void *V_t, double sigma, const void *U,
-                      void *W, double rtol, int max_iter, void *ws, size_t ws_bytes, int *iters,
-                      void *stream) {
+static op_status cg_solve_by(int route, const op_problem *pb, int ld, const void *V_t, double sigma,
+                             const void *U, void *W, double rtol, int max_iter, void *ws,
+                             size_t ws_bytes, int *iters, void *stream) {
   Geom g;
   OP_TRY(make_geom(pb, &g));
   OP_TRY(check_blocks(pb->prec, pb->p, ld, U, W));
@@ -1166,6 +1166,7 @@ op_status op_cg_solve(const op_problem *pb, int ld, const void *V_t, double sigm
   CGWork w;
   cg_carve(ws, g.n, ld, elem, &w);
   w.jacobi = pb->cg_precond == OP_PRECOND_JACOBI;
+  w.route = route;
   int host_ctl[4] = {0, 0, 0, 0};
   w.host_ctl = host_ctl;
   cudaStream_t st = (cudaStream_t)stream;
@@ -1177,6 +1178,22 @@ op_status op_cg_solve(const op_problem *pb, int ld, const void *V_t, double sigm
     s = cg_solve<float>(g, (const float *)V_t, sigma, (const float *)U, (float *)W, pb->p, ld,
                         rtol, max_iter, w, iters, st);
   return s;
+}
+
+op_status op_cg_solve(const op_problem *pb, int ld, const void *V_t, double sigma, const void *U,
+                      void *W, double rtol, int max_iter, void *ws, size_t ws_bytes, int *iters,
+                      void *stream) {
+  return cg_solve_by(0, pb, ld, V_t, sigma, U, W, rtol, max_iter, ws, ws_bytes, iters, stream);
+}
+
+op_status op_selftest_cg(int route, const op_problem *pb, int ld, const void *V_t, double sigma,
+                         const void *U, void *W, double rtol, int max_iter, void *ws,
+                         size_t ws_bytes, int *iters, void *stream) {
+  if (route != 1 && route != 2) {
+    set_error("op_selftest_cg: route 1 or 2");
+    return OP_ERR_ARG;
+  }
+  return cg_solve_by(route, pb, ld, V_t, sigma, U, W, rtol, max_iter, ws, ws_bytes, iters, stream);
 }
 
 // Kernel-level scratch of op_gram / op_update starts with a 256-byte header whose first

@@ -657,7 +657,8 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
   }
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+  const cudaError_t e =
+      w.route == 2 ? cudaErrorCooperativeLaunchTooLarge : cudaLaunchKernelExC(&cfg, fn, args);
   prof_end(w.prof, st);
   // a process confined to a few SMs may not hold the CTAs together: the general path needs no such thing
   *ran = e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorInvalidClusterSize &&

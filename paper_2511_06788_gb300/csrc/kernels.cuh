@@ -134,6 +134,8 @@ struct CGWork {
   int max_blocks;
   int expect_iters = 0;  // iterations of the previous solve (first chunk length)
   bool jacobi = false;   // CG preconditioned with diag(H + sigma)
+  int route = 0;         // of cg_solve: 0 by its rule, 1 the general kernels, 2 as if the device
+                         // refused the cooperative launch (self-tests)
   Prof *prof = nullptr;  // optional timing
 };
 // bytes of the CTA-partials scratch used by the reductions of a row width ld
