@@ -288,7 +288,8 @@ op_status op_eigenvalues(op_ctx *ctx, double *lam, int kind);
 op_status op_get_stats(op_ctx *ctx, op_stats *st);
 
 /* Per-kernel timing with CUDA events recorded on the context's stream around each
- * launch group of a step (kinds: op_profile_name(0 .. op_profile_kinds()-1)).
+ * launch group of a step (kinds: op_profile_name(0 .. op_profile_kinds()-1); a Step 1 that
+ * runs as one launch is "cg_solve", else "cg_init", "cg_apply" and so on).
  * Enabling (or disabling) synchronises the stream and resets the totals. */
 op_status op_profile_enable(op_ctx *ctx, int enable);
 int op_profile_kinds(void);

@@ -639,7 +639,6 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
   while (lanes < 32 && 2 * lanes * ld <= kSumThreads<T>) lanes *= 2;
   const void *fn = w.jacobi ? coop_kernel<T, true>(lanes) : coop_kernel<T, false>(lanes);
   OP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoopSmem));
-  prof_begin(w.prof, PK_CG_APPLY, st);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(G);
   cfg.blockDim = dim3(kCoopThreads);
@@ -657,9 +656,9 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
   }
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  prof_begin(w.prof, PK_CG_SOLVE, st);
   const cudaError_t e =
       w.route == 2 ? cudaErrorCooperativeLaunchTooLarge : cudaLaunchKernelExC(&cfg, fn, args);
-  prof_end(w.prof, st);
   // a process confined to a few SMs may not hold the CTAs together: the general path needs no such thing
   *ran = e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorInvalidClusterSize &&
          e != cudaErrorLaunchOutOfResources;
@@ -668,6 +667,7 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
     return OP_OK;
   }
   OP_CUDA(e);
+  prof_end(w.prof, st);
   count_launch();
   OP_CUDA(cudaMemcpyAsync(w.host_ctl, w.ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
   OP_CUDA(cudaStreamSynchronize(st));

@@ -21,6 +21,7 @@ enum ProfKind {
   PK_ENERGY,
   PK_RESIDUAL,
   PK_REFINE,   // FP64 residual, scaling and correction of the mixed-precision Step 1
+  PK_CG_SOLVE, // a whole CG in one cooperative launch
   PK_COUNT
 };
 struct Prof {

@@ -1312,7 +1312,7 @@ op_status launch_b_energy(const BatchProb *B, const RowItem *items, int nitems, 
 const char *prof_name(int kind) {
   static const char *names[PK_COUNT] = {"cg_init", "cg_apply", "cg_axpy", "cg_dir",
                                         "cg_finalize", "gram", "core", "update", "energy",
-                                        "residual", "cg_refine"};
+                                        "residual", "cg_refine", "cg_solve"};
   return (kind >= 0 && kind < PK_COUNT) ? names[kind] : "";
 }
 

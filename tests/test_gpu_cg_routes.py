@@ -78,3 +78,13 @@ def test_large_blocks_meet_the_residual_test(prec, shape, p, precond):
     res = np.linalg.norm(Uh - A @ Wh, axis=0)
     assert np.all(res <= (rtol + 2 * (its + 1) * eps * kappa) * norm)
     assert np.all(Wh[:, p:] == 0)
+
+
+def test_a_cooperative_solve_is_a_group_of_its_own_in_the_profile():
+    P = syn.config_2d_laplace()
+    with pkg.Solver(P.shape, P.lo, P.hi, P.V, syn.gaussian_block(0, P.n, P.p), P.p, prec="fp32") as s:
+        s.profile(True)
+        s.step(3)
+        prof = s.profile_read()
+    assert prof["cg_solve"][1] == 3 and prof["cg_solve"][0] > 0.0
+    assert prof["cg_apply"][1] == 0 and prof["cg_axpy"][1] == 0
