@@ -585,15 +585,13 @@ template <typename T> int coop_ctas(long long n, int ld, int *rows) {
   return (int)((n + *rows - 1) / *rows);
 }
 
-template <typename T, bool JAC> const void *coop_kernel(int lanes) {
-  switch (lanes) {
-    case 1: return (const void *)k_cg_coop<T, JAC, 1>;
-    case 2: return (const void *)k_cg_coop<T, JAC, 2>;
-    case 4: return (const void *)k_cg_coop<T, JAC, 4>;
-    case 8: return (const void *)k_cg_coop<T, JAC, 8>;
-    case 16: return (const void *)k_cg_coop<T, JAC, 16>;
-    default: return (const void *)k_cg_coop<T, JAC, 32>;
-  }
+// Lanes a column: FP32 blocks have at most 256 columns for 512 threads, FP64 ones at least 8 for 128.
+template <typename T> constexpr int kMinLanes = sizeof(T) == 4 ? 2 : 1;
+template <typename T> constexpr int kMaxLanes = sizeof(T) == 4 ? 32 : 16;
+template <typename T, bool JAC, int L = kMinLanes<T>> const void *coop_kernel(int lanes) {
+  if constexpr (L < kMaxLanes<T>)
+    if (lanes > L) return coop_kernel<T, JAC, 2 * L>(lanes);
+  return (const void *)k_cg_coop<T, JAC, L>;
 }
 
 }  // namespace
@@ -635,8 +633,8 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
                       ((size_t)kCoopThreads * N * 3 + kCoopThreads / (ld / N) + 1) * sizeof(T);
   OP_CUDA(cudaMemsetAsync(w.ctl, 0, 256, st));
   void *args[] = {&a};
-  int lanes = 1;
-  while (lanes < 32 && 2 * lanes * ld <= kSumThreads<T>) lanes *= 2;
+  int lanes = kMinLanes<T>;
+  while (lanes < kMaxLanes<T> && 2 * lanes * ld <= kSumThreads<T>) lanes *= 2;
   const void *fn = w.jacobi ? coop_kernel<T, true>(lanes) : coop_kernel<T, false>(lanes);
   OP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoopSmem));
   cudaLaunchConfig_t cfg{};
