@@ -11,9 +11,10 @@
 // two barriers an iteration; FP64 stores Q and P and takes three (recomputing would cost six
 // more FP64 operations per element, and GB300 runs two a clock and SM).
 //
-// What is left of an iteration: tiny solves 5.4 us of shuffles, barriers and latency (32 x 32 x 8,
-// one cluster; 28 us by kernels), FP64 the FP64 pipe (199 x 199 x 16: 25 us, of which 11 for its
-// 10 operations an element; 55 us by kernels), FP32 the L2 latency of its stencil loads.
+// What is left of an iteration: tiny solves 5.0 us of shuffles, barriers and latency (32 x 32 x 8,
+// FP32, one cluster; 37 us by kernels), FP64 the FP64 pipe (199 x 199 x 16: 31 us with the Jacobi
+// preconditioner, of which 11 for its 10 operations an element; 58 us by kernels), FP32 the L2 latency
+// of its stencil loads (200 x 200 x 16 15 us, 39 by kernels).
 //
 // Every wait of the barrier is bounded; a CTA that gives up sets the error word and returns.
 #include <string.h>
@@ -31,11 +32,16 @@ namespace opevo {
 namespace {
 
 constexpr int kCoopThreads = 512;
-// Largest block of a cooperative solve.  FP32: the four blocks of an iteration have to stay in
-// the 126 MB L2, and on 3-D grids the TMA direction kernel takes over: 56^3 x 40 (28 MB) 1.80 ms
-// here and 2.90 ms by kernels, 56^3 x 64 (45 MB) 3.43 and 3.54, 64^3 x 84 (92 MB) 8.9 and 7.7.
-// FP64: bound by the FP64 pipe either way: 64^3 x 64 (134 MB, the largest tried) 32.9 and 38.1.
-template <typename T> constexpr long long kCoopBytes = (sizeof(T) == 4 ? 48ll : 140ll) << 20;
+// Largest block of a cooperative solve; microseconds an iteration here and by the general kernels
+// (Jacobi).  FP32: the four blocks of an iteration have to stay in the 126 MB L2, and on 3-D grids the
+// TMA direction kernel takes over: 48^3 x 80 (34 MB) 88 and 97, 36^3 x 200 (36 MB) 111 and 118,
+// 56^3 x 56 (38 MB) 97 and 94, 56^3 x 64 (43 MB) 112 and 100.  2-D grids: 700 x 700 x 24 (45 MB) 99 and
+// 114, and 127 against 141 at 61 MB, 208 against 196 at 92 MB, beyond the line.  FP64, bound by the FP64
+// pipe either way: 64^3 x 64 (128 MB) 568 and 645; the line is not a crossing (72^3 x 128, 365 MB: 1581
+// and 1721).
+template <typename T> constexpr long long coop_bytes(int dim) {
+  return (sizeof(T) == 8 ? 140ll : (dim == 3 ? 36ll : 48ll)) << 20;
+}
 // Dynamic shared memory a launch may ask for (the largest any size below takes is 140 KB).  The
 // limit belongs to the kernel on the device, so every call sets this one value: a limit of the
 // call's own size could be lowered by another thread's solve between setting it and the launch.
@@ -596,8 +602,8 @@ template <typename T, bool JAC, int L = kMinLanes<T>> const void *coop_kernel(in
 
 }  // namespace
 
-template <typename T> bool cg_coop_eligible(long long n, int ld) {
-  return ld / Pack<T>::N <= 64 && n * ld * (long long)sizeof(T) <= kCoopBytes<T>;
+template <typename T> bool cg_coop_eligible(const Geom &g, int ld) {
+  return ld / Pack<T>::N <= 64 && g.n * ld * (long long)sizeof(T) <= coop_bytes<T>(g.dim);
 }
 
 template <typename T>
@@ -680,7 +686,7 @@ op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, in
 }
 
 #define OPEVO_INST(T)                                                                          \
-  template bool cg_coop_eligible<T>(long long, int);                                           \
+  template bool cg_coop_eligible<T>(const Geom &, int);                                        \
   template op_status cg_coop<T>(const Geom &, const T *, double, const T *, T *, int, int,     \
                                 double, int, CGWork &, int *, bool *, cudaStream_t);
 OPEVO_INST(float)

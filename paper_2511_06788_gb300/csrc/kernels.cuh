@@ -151,7 +151,7 @@ op_status cg_solve(const Geom &g, const T *Vt, double sigma, const T *U, T *W, i
 // The same solve in one cooperative launch for blocks that stay in L2 (cg_coop.cu); cg_solve
 // takes it where cg_coop_eligible; *ran = false (and no work done) where the device cannot hold
 // its CTAs together.
-template <typename T> bool cg_coop_eligible(long long n, int ld);
+template <typename T> bool cg_coop_eligible(const Geom &g, int ld);
 template <typename T>
 op_status cg_coop(const Geom &g, const T *Vt, double sigma, const T *U, T *W, int p, int ld,
                   double rtol, int max_iter, CGWork &w, int *iters, bool *ran, cudaStream_t st);

@@ -696,7 +696,7 @@ void cg_carve(void *ws, long long n, int ld, int elem, CGWork *w) {
 template <typename T>
 op_status cg_solve(const Geom &g, const T *Vt, double sigma, const T *U, T *W, int p, int ld,
                    double rtol, int max_iter, CGWork &w, int *iters, cudaStream_t st) {
-  if (w.route != 1 && cg_coop_eligible<T>(g.n, ld)) {
+  if (w.route != 1 && cg_coop_eligible<T>(g, ld)) {
     bool ran = true;
     OP_TRY(cg_coop<T>(g, Vt, sigma, U, W, p, ld, rtol, max_iter, w, iters, &ran, st));
     if (ran) return OP_OK;
