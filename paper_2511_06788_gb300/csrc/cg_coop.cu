@@ -11,7 +11,7 @@
 // two barriers an iteration; FP64 stores Q and P and takes three (recomputing would cost six
 // more FP64 operations per element, and GB300 runs two a clock and SM).
 //
-// What is left of an iteration: tiny solves 5.0 us of shuffles, barriers and latency (32 x 32 x 8,
+// What is left of an iteration: tiny solves 4.9 us of shuffles, barriers and latency (32 x 32 x 8,
 // FP32, one cluster; 37 us by kernels), FP64 the FP64 pipe (199 x 199 x 16: 31 us with the Jacobi
 // preconditioner, of which 11 for its 10 operations an element; 58 us by kernels), FP32 the L2 latency
 // of its stencil loads (200 x 200 x 16 15 us, 39 by kernels).
@@ -592,8 +592,11 @@ template <typename T> int coop_ctas(long long n, int ld, int *rows) {
 }
 
 // Lanes a column: FP32 blocks have at most 256 columns for 512 threads, FP64 ones at least 8 for 128.
+// FP32 no more than 8: a level of the shuffle tree (three shuffles, three dependent two-sums) takes
+// as long as five terms summed in turn (20 steps of 32 x 32 x 8 in FP64: 24.0 ms by up
+// to 32 lanes, 23.7 by 16, 22.9 by 8, 23.3 by 4).
 template <typename T> constexpr int kMinLanes = sizeof(T) == 4 ? 2 : 1;
-template <typename T> constexpr int kMaxLanes = sizeof(T) == 4 ? 32 : 16;
+template <typename T> constexpr int kMaxLanes = sizeof(T) == 4 ? 8 : 16;
 template <typename T, bool JAC, int L = kMinLanes<T>> const void *coop_kernel(int lanes) {
   if constexpr (L < kMaxLanes<T>)
     if (lanes > L) return coop_kernel<T, JAC, 2 * L>(lanes);

@@ -81,8 +81,8 @@ __host__ __device__ __forceinline__ bool quotient(const Sum3 &a, const Sum3 &b, 
     *q = 0.f;
     return true;
   }
-  const float p = ah / bh;
-  *q = add_rn(p, add_rn(fmaf(-p, bh, ah), fmaf(-p, bl, al)) / bh);
+  const float rb = 1.f / bh, p = mul_rn(ah, rb);  // (p is within 2 ulp: its remainder has 25 bits)
+  *q = fmaf(add_rn(fmaf(-p, bh, ah), fmaf(-p, bl, al)), rb, p);
   return al == al && bl == bl && ah > 8.27e-25f && ah < 1.26e30f && bh > 8.27e-25f &&
          bh < 1.26e30f && p > 1e-30f && p < 1e30f;
 }

@@ -43,3 +43,33 @@ def test_columns_of_large_norm_are_solved(shape, p, precond):
     res = np.linalg.norm(U - A @ W, axis=0)
     tol = (rtol + 2 * (its + 1) * eps * kappa) * norm
     assert np.all(res <= tol), float((res[:p] / tol[:p]).max())
+
+
+@pytest.mark.parametrize("shape,p", [((16, 16), 8), ((128, 128), 8), ((31, 30, 29), 40)],
+                         ids=lambda v: str(v).replace(" ", ""))
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64], ids=["fp32", "fp64"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_a_non_finite_column_leaves_the_others_alone(shape, p, dtype, bad):
+    """Cooperative solve and general kernels: the other columns meet the residual test, and the solve
+    ends with them (a NaN column is inactive from the start, an infinite one has no finite target)."""
+    n = int(np.prod(shape))
+    rng = np.random.default_rng(n + 1)
+    half = 0.25 * max(shape)
+    lo, hi = (-half,) * len(shape), (half,) * len(shape)
+    np_t = np.float32 if dtype == torch.float32 else np.float64
+    V = (4.0 * rng.random(n)).astype(np_t)
+    U = rng.uniform(-1.0, 1.0, (n, p)).astype(np_t)
+    U[n // 3, 2] = bad
+    rtol, eps = (1e-4, 2.0**-23) if dtype == torch.float32 else (1e-10, 2.0**-52)
+    A = o.hamiltonian(shape, lo, hi, V.astype(np.float64)) + scipy.sparse.identity(n)
+    kappa = float(abs(A).sum(axis=1).max())
+    keep = np.arange(p) != 2
+    Vd, Ud = torch.from_numpy(V).cuda(), torch.from_numpy(U).cuda()
+    for route in (0, 1):
+        Wd = torch.zeros_like(Ud)
+        args = (shape, lo, hi, Vd, 1.0, Ud, Wd, p, rtol)
+        its = pkg.cg_solve(*args) if route == 0 else pkg.selftest_cg(route, *args)
+        assert 0 < its < 500
+        W, Uk = Wd.cpu().numpy().astype(np.float64)[:, keep], U.astype(np.float64)[:, keep]
+        res = np.linalg.norm(Uk - A @ W, axis=0)
+        assert np.all(res <= (rtol + 2 * (its + 1) * eps * kappa) * np.linalg.norm(Uk, axis=0)), route
