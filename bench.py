@@ -66,11 +66,11 @@ ALGO_BYTES = {
 # product and three scaled subtractions (10); p.q adds 2.  axpy: w += a p, z -= a q / d,
 # rk = d z and two sums (10); dir: p = z + b p (2); init: apply, u - Aw, / d, three sums (18).
 FP64_CG_FLOPS = {"cg_apply": 12, "cg_axpy": 10, "cg_dir": 2, "cg_init": 18, "energy": 14}
-# digit-product kernels: 28 BF16 MMAs per digit pair set, 2 flops per multiply-add
+# digit-product kernels: 28 (36) digit pairs per K step, 2 flops per multiply-add
 
 
 def digit_flops(group, n, ld):
-    """BF16 tensor flops one step's FP64 Gram (7 digits: 28 digit-pair MMAs per K step) /
+    """BF16 tensor flops one step's FP64 Gram (7 digits: 28 digit pairs per K step) /
     update (8 digits: 36) issues on the tensor cores."""
     if group == "gram":
         nc = 2 * ld
@@ -97,9 +97,9 @@ def fp64_rooflines(prof, n, p, ld, steps, ms, peaks, hbm, bf16_sust):
     """Rooflines of the FP64 mode's kernel groups over a timed region (`prof`: group ->
     (device ms, launch ranges); `ms`: the region's time), each against the unit that bounds
     it:
-    - gram / update: the digit-pair MMAs on the tensor cores (BF16 flops; with the digit
+    - gram / update: the digit products on the tensor cores (BF16 flops; with the digit
       split in the group's time) against the sustained cuBLAS BF16 rate, and against the
-      library's best N = 64 MMA rate;
+      library's best rate of MMAs of one digit pair (N = 64; the kernel merges up to four);
     - cg_*: with the mixed-precision Step 1 (a cg_refine group present) these are the FP32
       inner CG kernels, bound by HBM (FP32 bytes over ld columns); in plain FP64 CG the FP64
       kernels, bound by the FP64 ALU;
@@ -123,8 +123,8 @@ def fp64_rooflines(prof, n, p, ld, steps, ms, peaks, hbm, bf16_sust):
                                       "seconds-long loop)",
                           frac_of_n64_mma_peak=a / peaks["bf16_mma_n64_areuse"],
                           n64_peak_source="op_peak_rate(OP_PEAK_BF16_MMA_N64_AREUSE) in this "
-                                          "run: the kernel's MMA shape, 128 x 64 x 16, at its "
-                                          "best measured rate",
+                                          "run: one digit pair, 128 x 64 x 16, at its best "
+                                          "measured rate (the kernel merges up to four pairs)",
                           algo_flops_per_launch=fl)
         elif g == "cg_refine":
             # ranges per step: (residual, rhs, correction) per cycle and a closing residual

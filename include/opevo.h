@@ -59,7 +59,8 @@ typedef enum {
                             update by op_problem.fp64_gemm)                          */
   OP_FP32 = 1,           /* blocks, stencil and CG in FP32; Gram and update on the
                             tensor cores with a TF32 hi/lo split (FP32-class accuracy),
-                            Gram chunk sums in FP64; Step 2-3 core in FP64           */
+                            Gram chunk sums as precise as FP64; Step 2-3 core in
+                            FP64                                                     */
   OP_MIX_TF32 = 2,       /* as OP_FP32 but one TF32 MMA per product (operands rounded
                             to TF32, 10-bit mantissa); context-level API only        */
   OP_MIX_BF16X3 = 3,     /* as OP_FP32 but the Gram and update take BF16 operands split
@@ -341,11 +342,10 @@ typedef enum {
   OP_PEAK_FP64_FMA = 0,
   OP_PEAK_TF32_MMA = 1,
   OP_PEAK_BF16_MMA = 2,
-  OP_PEAK_BF16_MMA_N64 = 3,  /* BF16 at N = 64 (the FP64 digit products' MMA shape), a new
-                                A tile every MMA */
+  OP_PEAK_BF16_MMA_N64 = 3,  /* BF16 at N = 64 (one digit pair of the FP64 products, which
+                                take up to four in one MMA), a new A tile every MMA */
   OP_PEAK_BF16_MMA_N64_AREUSE = 4  /* the same, each A tile kept in the tensor core's
-                                      collector buffer over four MMAs with different B
-                                      (the digit products' issue pattern) */
+                                      collector buffer over four MMAs with different B */
 } op_peak_kind;
 op_status op_peak_rate(int kind, double *tflops, void *stream);
 
@@ -426,8 +426,8 @@ size_t op_cg_workspace(const op_problem *pb, int ld);
  * each ld x ld FP64 row-major on the device (entries with i or j >= p are zero).
  * Any of C, S, D may be NULL to skip it.  OP_FP64: FP64 FMA, chunk partials in FP64.
  * OP_FP32: tcgen05 tensor-core MMAs (TF32 inputs split hi + lo, four MMAs per
- * product, FP32 accumulation per chunk of grid points, chunk partials summed as error-free
- * pairs of floats).
+ * product, FP32 accumulation per chunk of grid points, chunk partials summed as triples of
+ * floats, in FP64 where a sum leaves the FP32 range).
  * OP_MIX_BF16X3: FP32 blocks, BF16 inputs split in three, six kind::f16 MMAs per product.
  * ws: device scratch of at least op_gram_workspace() bytes; its first int is set when a
  * bounded device wait gave up (check with op_ws_status). */

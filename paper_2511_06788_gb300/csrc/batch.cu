@@ -181,7 +181,7 @@ op_status build_lists(op_batch *b) {
     pb.core_X = M + m2;
     pb.core_B = M + 2 * m2;
     pb.core_R = M + 3 * m2;
-    pb.gram_part = (double *)c->gram_ws;
+    pb.gram_part = (float *)c->gram_ws;
     pb.err = c->dev_err;
     pb.dsc = c->dsc;
     pb.frozen = b->d_frozen + i;

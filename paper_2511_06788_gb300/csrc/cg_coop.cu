@@ -592,7 +592,7 @@ template <typename T> int coop_ctas(long long n, int ld, int *rows) {
 }
 
 // Lanes a column: FP32 blocks have at most 256 columns for 512 threads, FP64 ones at least 8 for 128.
-// FP32 no more than 8: a level of the shuffle tree (three shuffles, three dependent two-sums) takes
+// FP32 no more than 8: a level of the shuffle tree (three shuffles, two dependent two-sums) takes
 // as long as five terms summed in turn (20 steps of 32 x 32 x 8 in FP64: 24.0 ms by up
 // to 32 lanes, 23.7 by 16, 22.9 by 8, 23.3 by 4).
 template <typename T> constexpr int kMinLanes = sizeof(T) == 4 ? 2 : 1;

@@ -19,7 +19,7 @@
 // a systematic error of the orthogonality).  Each 32-point slab therefore starts a fresh
 // accumulator (four TMEM accumulators in turn), which is drained into FP32 registers
 // (round-to-nearest additions); a chunk's FP32 sums are its partial tile, and the partials are
-// added over the chunks in a fixed order as error-free pairs of floats.
+// added over the chunks in a fixed order as triples of floats (sums.cuh).
 //
 // Roles (k_gram_ws), meeting only at mbarriers: eight warps stage slabs into a ring of three,
 // one thread issues the MMAs (16 a slab, 74 clocks each: the bound), eight warps drain.  With
@@ -179,7 +179,7 @@ struct GramBatchSrc {
     int prod, ti, tj;
     decode_job(it.job, 7, (pb.ld + kTM - 1) / kTM, &prod, &ti, &tj);
     set_task(t, pb.g.n, pb.ld, pb.U[parity], pb.W, prod, ti, tj, it.r0, it.r1);
-    t->part = (float *)pb.gram_part + ((long long)it.split * pb.gram_jobs + it.job) * (kTM * kTM);
+    t->part = pb.gram_part + ((long long)it.split * pb.gram_jobs + it.job) * (kTM * kTM);
     t->sum = nullptr;
     t->err = pb.err;
     return true;
@@ -599,7 +599,7 @@ __global__ void k_b_gram_tc_reduce(const BatchProb *__restrict__ Bp) {
   int prod, ti, tj;
   decode_job(blockIdx.x, 7, (pb.ld + kTM - 1) / kTM, &prod, &ti, &tj);
   reduce_tile(prod, ti, tj, blockIdx.z, gridDim.z,
-              (const float *)pb.gram_part + (long long)blockIdx.x * (kTM * kTM),
+              pb.gram_part + (long long)blockIdx.x * (kTM * kTM),
               (long long)pb.gram_jobs * (kTM * kTM), pb.n_gram_splits, pb.p, pb.ld,
               prod == PROD_C ? pb.C : (prod == PROD_S ? pb.S : pb.D));
 }

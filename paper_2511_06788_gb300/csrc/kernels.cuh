@@ -65,7 +65,7 @@ struct BatchProb {
   float *KT_hi, *KT_lo;
   int *core_status;
   double *core_M, *core_X, *core_B, *core_R;  // ld x ld each
-  double *gram_part;       // Gram chunk partials [splits][jobs][128 x 128]
+  float *gram_part;        // Gram chunk partials [splits][jobs][128 x 128]
   int *err;
   double *dsc;             // scalars: 0..2 core stats, 4..5 energy
   int *frozen;             // non-zero: converged, every batched kernel skips it
@@ -129,8 +129,8 @@ struct CGWork {
   double *part;          // CTA partials [max_blocks][2][ld] + per-column sums [2][ld]
   double *state;         // [6][ld]: rr, target, alpha, beta, bnorm2, scratch
   int *active;           // [ld]
-  int *ctl;              // [4] device: active counts (two parities), iterations done,
-                         // error flag (a bounded wait of a TMA kernel gave up)
+  int *ctl;              // 256 bytes: [4] active counts (two parities), iterations done,
+                         // error flag (a bounded wait gave up); the cooperative solve's own
   int *host_ctl;         // >= 4 ints of host memory (pinned for the context)
   int max_blocks;
   int expect_iters = 0;  // iterations of the previous solve (first chunk length)

@@ -844,8 +844,8 @@ op_status back_layer(opnet *net, int i, const float *X, const float *dZ, float *
     while (w.ng > 1 && bytes(w.ng) > kWSmem) w.ng /= 3;
     const int threads = (per * w.ng + 31) / 32 * 32, gx = groups / w.ng * w.kblocks;
     // runs of at most 2048 points, more of them while CTAs are missing, down to 128 points (four
-    // stages; loss and gradient at 48^3: from 96 points 3.85 ms, 128 3.80, 64 3.84), and the
-    // partials fit
+    // stages; not a sharp line: loss and gradient at 48^3, the one shape measured, from 96 points
+    // 3.85 ms, 128 3.80, 64 3.84), and the partials fit
     const long long points = w.q1 - w.q0, cap = net->part_floats / ((K + 1) * (long long)l.cout);
     long long want = std::min<long long>((4LL * num_sms() + gx - 1) / gx, points / 128);
     want = std::max(std::min(want, cap), std::min((points + 2047) / 2048, cap));

@@ -4,7 +4,7 @@
 //                      thread, 2 flops each;
 //   OP_PEAK_TF32_MMA   tcgen05.mma kind::tf32, M = 128, N = 256, K = 8 per instruction;
 //   OP_PEAK_BF16_MMA   tcgen05.mma kind::f16 (BF16), M = 128, N = 256, K = 16;
-//   OP_PEAK_BF16_MMA_N64  the same at N = 64, the shape of the FP64 digit products, on
+//   OP_PEAK_BF16_MMA_N64  the same at N = 64, one digit pair of the FP64 products, on
 //                      eight accumulators in turn, every MMA with a new A tile: reading
 //                      A (128 x 16) from shared memory for each 128 x 64 x 16 product
 //                      holds N = 64 to about half the N = 256 rate;

@@ -10,7 +10,7 @@
 // Per-column dot products are accumulated per thread in the block type T and
 // combined across threads and CTAs in FP64 (per-element FP64 work would make
 // the FP32 kernels FP64-pipe bound on GB300).  Partial sums per CTA are
-// reduced by one warp per column in a fixed order (deterministic).
+// reduced four columns a block in a fixed order (deterministic).
 //
 // CG control lives on the device: the finalisers compute alpha, beta and the
 // number of still-active columns; every kernel of an iteration returns at once
