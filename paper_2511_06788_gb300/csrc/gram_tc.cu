@@ -26,6 +26,8 @@
 // every warp staging, waiting and draining in lockstep (one CTA per item) a slab took 3050
 // clocks, 1190 of them the MMAs.  262144 x 128, C, S and D: 216 us, 301 before (an MMA takes 111
 // clocks beside the staging: both load shared memory).
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.cuh"
 #include "sums.cuh"
@@ -553,14 +555,13 @@ template <> struct SplitSum<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
   __device__ __forceinline__ void add(const SplitSum &o) { s += o.s; }
-  __device__ __forceinline__ bool finite() const { return true; }  // (nothing to add again)
   __device__ __forceinline__ double value() const { return s; }
 };
 
 // out(i, j) = the summed tile element, zero outside p x p, both triangles of S and D.
 // A CTA of kRedLanes x kRedGroups threads: group g sums every kRedGroups-th split, the first
 // group adds the sums up.  One thread per element and all its splits was a serial chain of up to
-// 228 loads and two-sums: 24 us at 262144 x 128, now 13.  An element whose sum leaves the FP32 range
+// 228 loads and two-sums: 24 us at 262144 x 128, now 15 (13 with pairs of floats).  An element whose sum leaves the FP32 range
 // is summed in FP64.
 template <typename P>
 __device__ __forceinline__ void reduce_tile(int prod, int ti, int tj, int slice, int slices,
@@ -581,10 +582,8 @@ __device__ __forceinline__ void reduce_tile(int prod, int ti, int tj, int slice,
 #pragma unroll
       for (int q = 0; q < kRedGroups - 1; ++q) s.add(sh[q][lane]);
       double v = (i < p && j < p) ? s.value() : 0.0;
-      if (!s.finite()) {
-        v = 0.0;
-        for (int sp = 0; sp < nsplit; ++sp) v += (double)part[e + sp * stride];
-      }
+      if constexpr (std::is_same<P, float>::value)
+        if (!s.finite()) v = sum64(part + e, stride, nsplit);
       out[(long long)i * ld + j] = v;
       if (prod != PROD_C && ti != tj) out[(long long)j * ld + i] = v;
     }
@@ -593,7 +592,9 @@ __device__ __forceinline__ void reduce_tile(int prod, int ti, int tj, int slice,
 }
 
 // Batched reduce: grid (jobs, problems, element slices).
-__global__ void k_b_gram_tc_reduce(const BatchProb *__restrict__ Bp) {
+// (eight CTAs an SM: the sums are a chain of loads)
+__global__ void __launch_bounds__(kRedLanes * kRedGroups, 8)
+    k_b_gram_tc_reduce(const BatchProb *__restrict__ Bp) {
   const BatchProb &pb = Bp[blockIdx.y];
   if (*pb.frozen || (int)blockIdx.x >= pb.gram_jobs) return;
   int prod, ti, tj;
@@ -605,9 +606,9 @@ __global__ void k_b_gram_tc_reduce(const BatchProb *__restrict__ Bp) {
 }
 
 template <typename P>
-__global__ void k_gram_tc_reduce(int mask, int nt, int njobs, int nsplit,
-                                 const P *__restrict__ part, int p, int ld, double *C, double *S,
-                                 double *D) {
+__global__ void __launch_bounds__(kRedLanes * kRedGroups, 8)
+    k_gram_tc_reduce(int mask, int nt, int njobs, int nsplit, const P *__restrict__ part, int p,
+                     int ld, double *C, double *S, double *D) {
   int prod, ti, tj;
   decode_job(blockIdx.x, mask, nt, &prod, &ti, &tj);
   reduce_tile(prod, ti, tj, blockIdx.y, gridDim.y, part + (long long)blockIdx.x * (kTM * kTM),

@@ -427,8 +427,7 @@ __global__ void k_wgrad_copy(int N, int C, const float *__restrict__ X, float *_
 // out[e] = sum_s part[s][e] (fixed order): blocks of 32 elements by 16 interleaved sums over the
 // splits, each a triple of floats (sums.cuh; a warp's FP64 conversion and addition take 64 clocks
 // each), joined as they are; in FP64 where a sum leaves the FP32 range.  The 11 layers at 48^3:
-// 467 us with one FP64 sum an element, 293 us with pairs of floats joined in FP64 (cold); the loss and
-// gradient there 3.81 ms with the latter, 3.71 so.
+// 467 us with one FP64 sum an element, 293 us with pairs of floats joined in FP64, 206 us so (cold).
 __global__ void __launch_bounds__(512) k_reduce_parts(const float *__restrict__ part, int splits,
                                                       long long count, float *__restrict__ out) {
   __shared__ Sum3 red[16][33];
@@ -444,11 +443,7 @@ __global__ void __launch_bounds__(512) k_reduce_parts(const float *__restrict__ 
     if (y == 0 && e < count) {
 #pragma unroll
       for (int j = 1; j < 16; ++j) t.add(red[j][x]);
-      double s = t.value();
-      if (!t.finite()) {
-        s = 0.0;
-        for (int k = 0; k < splits; ++k) s += (double)part[(long long)k * count + e];
-      }
+      const double s = t.finite() ? t.value() : sum64(part + e, count, splits);
       out[e] = (float)s;
     }
     __syncthreads();

@@ -68,6 +68,17 @@ struct Sum3 {
   }
 };
 
+#ifdef __CUDACC__
+// The sum of n terms, `stride` apart, in FP64: where a triple is not finite.  A call: inlined into a
+// reduction its registers halved the warps in flight (the Gram's reduce 12.6 -> 22 us).
+__device__ __noinline__ static double sum64(const float *x, long long stride, int n) {
+  double s = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) s += (double)x[i * stride];
+  return s;
+}
+#endif
+
 // q = a / b in FP32 (0 where b <= 0): the quotient of the leading parts corrected by its remainder,
 // exact to about 2^-46 before the last rounding.  False, with no q, where a sum is not finite or
 // a, b (2^-80 .. 2^100) or the quotient are so small or large that the remainder could leave the
